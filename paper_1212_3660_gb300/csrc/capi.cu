@@ -376,9 +376,9 @@ struct Solve {
   int32_t *cyc, *sst, *mj, *sched, *rep_cyc, *rep_mj, *singular, *flags, *counter, *bcount;
   // multigrid, cycle precision
   std::vector<void*> f, z, z2, invd;
-  void* cinv;      // coarse inverse in cycle precision
+  void* cinv;      // coarse inverses in cycle precision, transposed
   z64* cwork;      // dense coarse matrices
-  z64* cinv64;
+  z64* cwork2;     // the inversion's second buffer
   // CSR operators: BiCGSTAB cycle work vectors (cycle precision), scalars, Jacobi diagonals
   int inner_steps = 8;
   double relax = 0.0;  // relaxed inner tolerance constant (0: fixed eps)
@@ -652,6 +652,11 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     tb += cv * nc * nc;
     tf += 8.0 * nc * nc;
     PROF(FKS_K_CLUSTER, lc, ns * tb, ns * tf, launch_cluster_vcycle<VT>(CP, csmem, S.st, S.nslot, s));
+  } else if (lt == nl - 1 && Ls[lt].n > COARSE_ALONE) {
+    // the coarsest level alone: its dense product over the chip
+    const double nc = (double)Ls[lt].n;
+    PROF(FKS_K_COARSE, lt, ns * (cv * nc * nc + 2 * cv * nc), ns * 8.0 * nc * nc,
+         launch_coarse_solve<VT>((const cx<VT>*)S.cinv, (int)Ls[lt].n, S.st, F(lt), Zl(lt), Ls[lt].n, S.nslot, s));
   } else {
     // levels lt .. coarsest in one block per slot
     TailParams<VT> P{};
@@ -1135,12 +1140,7 @@ static void setup_levels(Solve& S) {
   CK(cudaMemsetAsync(S.counter, 0, sizeof(int), S.s));
   CK(cudaMemsetAsync(S.bcount, 0, sizeof(int) * S.nslot, S.s));
   S.lane->prof.all_launches += 3;
-  launch_coarse_inverse(C, S.taus, S.n_tau, S.cwork, S.cinv64, S.singular, S.s, bf);
-  if constexpr (sizeof(VT) == 8) {
-    CK(cudaMemcpyAsync(S.cinv, S.cinv64, sizeof(z64) * S.n_tau * nc * nc, cudaMemcpyDeviceToDevice, S.s));
-  } else {
-    PROF(-1, -1, 0, 0, launch_to_prec<VT>(S.cinv64, (cx<VT>*)S.cinv, (int64_t)S.n_tau * nc * nc, S.s));
-  }
+  launch_coarse_inverse<VT>(C, S.taus, S.n_tau, S.cwork, S.cwork2, (cx<VT>*)S.cinv, S.singular, S.s, bf);
   ClusterParams<VT> CP{};
   const int lc = cluster_level<VT>(S.op, &CP);
   if (lc >= 0) {
@@ -1190,7 +1190,7 @@ static void carve(Solve& S, Arena& A, bool x_internal) {
     }
     S.bsc = A.take<BcgScal>(ns);
     S.bpart = A.take<double>((size_t)ns * csr_blocks(n) * 3);
-    S.cwork = S.cinv64 = nullptr;
+    S.cwork = S.cwork2 = nullptr;
     S.cinv = nullptr;
   } else {
     S.f.assign(Ls.size(), nullptr);
@@ -1211,7 +1211,7 @@ static void carve(Solve& S, Arena& A, bool x_internal) {
                                                 : nullptr;
     int64_t nc = Ls.back().n;
     S.cwork = A.take<z64>((size_t)S.n_tau * nc * nc);
-    S.cinv64 = A.take<z64>((size_t)S.n_tau * nc * nc);
+    S.cwork2 = A.take<z64>((size_t)S.n_tau * nc * nc);
     S.cinv = A.take<cx<VT>>((size_t)S.n_tau * nc * nc);
   }
   S.singular = A.take<int32_t>(1);

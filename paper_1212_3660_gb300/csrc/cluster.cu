@@ -247,8 +247,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
         const cx<T>* AI = (const cx<T>*)(csm + P.ainv);
         for (int rr = tid; rr < P.nc; rr += nt) {
           cx<T> acc = mk(T(0), T(0));
-          const cx<T>* row = AI + (int64_t)rr * P.nc;
-          for (int l = 0; l < P.nc; ++l) acc = acc + row[l] * FC[l];
+          for (int l = 0; l < P.nc; ++l) acc = acc + AI[l * P.nc + rr] * FC[l];
           ZC[rr] = acc;
         }
       }

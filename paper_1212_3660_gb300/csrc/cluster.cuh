@@ -49,7 +49,7 @@ struct ClusterParams {
 template <typename T>
 bool cluster_layout(const std::vector<LevelHost>& Ls, int l0, ClusterParams<T>* P, size_t* smem_bytes);
 // The per-tau coefficient regions of every CTA (levels of P, the coarsest
-// inverse Ainv [n_tau][nc][nc]); blob holds n_tau * CL_SIZE * P.region bytes.
+// inverse Ainv [n_tau][nc][nc], transposed); blob holds n_tau * CL_SIZE * P.region bytes.
 template <typename T>
 void launch_cluster_blob(const std::vector<LevelHost>& Ls, int l0, const ClusterParams<T>& P, const cx<T>* const* invd,
                          const cx<T>* Ainv, int ntau, unsigned char* blob, cudaStream_t s);

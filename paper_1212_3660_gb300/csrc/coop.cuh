@@ -16,7 +16,7 @@ struct CoopParams {
   cx<T>* f[MAX_LEVELS];             // right-hand sides, slot stride n
   cx<T>* z[MAX_LEVELS];             // iterates, slot stride n
   int rx[MAX_LEVELS], ry[MAX_LEVELS], rz[MAX_LEVELS];
-  const cx<T>* Ainv;                // [n_tau][nc][nc] coarsest inverses
+  const cx<T>* Ainv;                // [n_tau][nc][nc] coarsest inverses, transposed
   int nc;
   uint32_t mask;
   const z64* taus;

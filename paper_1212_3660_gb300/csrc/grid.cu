@@ -174,28 +174,30 @@ __global__ void k_invd(LevelView<double, C> L, const z64* __restrict__ taus, int
   }
 }
 
-// Dense coarsest-level matrix K + tau M (row-major, n x n) for every tau.
+// Dense coarsest-level matrix K + tau M (row-major, n x n, zeroed before) for
+// every tau: the nonzero entries of row c. col0 (optional, [n_tau][n]) receives
+// the first column, contiguous.
 template <typename C>
-__global__ void k_coarse_dense(LevelView<double, C> L, const z64* __restrict__ taus, int ntau, z64* __restrict__ A) {
+__global__ void k_coarse_dense(LevelView<double, C> L, const z64* __restrict__ taus, z64* __restrict__ A,
+                               z64* __restrict__ col0) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int q = blockIdx.y;
   if (c >= L.n) return;
   Cell p = cell_of(c, L.nx, L.ny);
   Faces<double> f = faces_at(L, p);
   double d = fsum(f), m = ldc<double>(L.mm, c);
   int64_t n = L.n, sxy = (int64_t)L.nx * L.ny;
-  for (int q = 0; q < ntau; ++q) {
-    z64* row = A + (int64_t)q * n * n + c * n;
-    for (int64_t l = 0; l < n; ++l) row[l] = mk(0.0, 0.0);
-    row[c] = mk(d + taus[q].re * m, taus[q].im * m);
-    if (p.i > 0) row[c - 1] = mk(-f.xl, 0.0);
-    if (p.i < L.nx - 1) row[c + 1] = mk(-f.xh, 0.0);
-    if (p.j > 0) row[c - L.nx] = mk(-f.yl, 0.0);
-    if (p.j < L.ny - 1) row[c + L.nx] = mk(-f.yh, 0.0);
-    if (L.nz > 1) {
-      if (p.k > 0) row[c - sxy] = mk(-f.zl, 0.0);
-      if (p.k < L.nz - 1) row[c + sxy] = mk(-f.zh, 0.0);
-    }
+  z64* row = A + (int64_t)q * n * n + c * n;
+  row[c] = mk(d + taus[q].re * m, taus[q].im * m);
+  if (p.i > 0) row[c - 1] = mk(-f.xl, 0.0);
+  if (p.i < L.nx - 1) row[c + 1] = mk(-f.xh, 0.0);
+  if (p.j > 0) row[c - L.nx] = mk(-f.yl, 0.0);
+  if (p.j < L.ny - 1) row[c + L.nx] = mk(-f.yh, 0.0);
+  if (L.nz > 1) {
+    if (p.k > 0) row[c - sxy] = mk(-f.zl, 0.0);
+    if (p.k < L.nz - 1) row[c + sxy] = mk(-f.zh, 0.0);
   }
+  if (col0) col0[(int64_t)q * n + c] = row[0];
 }
 
 // --------------------------------------------------------------------- apply
@@ -696,8 +698,8 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail_vcycle(TailParams<T> P
     const cx<T>* Ainv = P.Ainv + (int64_t)tau * P.nc * P.nc;
     for (int r = tid; r < P.nc; r += nt) {
       cx<T> acc = mk(T(0), T(0));
-      const cx<T>* row = Ainv + (int64_t)r * P.nc;
-      for (int l = 0; l < P.nc; ++l) acc = acc + row[l] * F[l];
+#pragma unroll 8
+      for (int l = 0; l < P.nc; ++l) acc = acc + Ainv[l * P.nc + r] * F[l];
       Z[r] = acc;
     }
     __syncthreads();
@@ -891,8 +893,8 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
     const cx<T>* Ainv = (const cx<T>*)(t2_smem + P.ainv_off);
     for (int r = tid; r < P.nc; r += nt) {
       cx<T> acc = mk(T(0), T(0));
-      const cx<T>* row = Ainv + r * P.nc;
-      for (int l = 0; l < P.nc; ++l) acc = acc + row[l] * F[l];
+#pragma unroll 4
+      for (int l = 0; l < P.nc; ++l) acc = acc + Ainv[l * P.nc + r] * F[l];
       Z[r] = acc;
     }
     __syncthreads();
@@ -947,100 +949,229 @@ bool tail2d_ok(const std::vector<LevelHost>& Ls, int lt) {
 }
 
 // --------------------------------------------------------------------- coarsest
-// Gauss-Jordan inversion with partial pivoting of one n x n complex matrix per
-// block (blockIdx.x = tau index), in place on A (row-major) with the inverse
-// written to Ainv. n <= MAX_COARSE.
-__global__ void k_gauss_jordan(z64* A, z64* Ainv, int n, int* singular) {
-  z64* a = A + (int64_t)blockIdx.x * n * n;
-  z64* inv = Ainv + (int64_t)blockIdx.x * n * n;
-  __shared__ int piv;
-  __shared__ double best[1024];
-  __shared__ int besti[1024];
-  for (int64_t t = threadIdx.x; t < (int64_t)n * n; t += blockDim.x)
-    inv[t] = (t / n == t % n) ? mk(1.0, 0.0) : mk(0.0, 0.0);
-  __syncthreads();
-  for (int col = 0; col < n; ++col) {
-    double bv = -1.0;
-    int bi = col;
-    for (int r = col + threadIdx.x; r < n; r += blockDim.x) {
-      double v = abs2(a[(int64_t)r * n + col]);
-      if (v > bv) { bv = v; bi = r; }
-    }
-    best[threadIdx.x] = bv;
-    besti[threadIdx.x] = bi;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-      if (threadIdx.x < s) {
-        double o = best[threadIdx.x + s];
-        int oi = besti[threadIdx.x + s];
-        if (o > best[threadIdx.x] || (o == best[threadIdx.x] && oi < besti[threadIdx.x])) {
-          best[threadIdx.x] = o;
-          besti[threadIdx.x] = oi;
-        }
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      piv = besti[0];
-      if (!(best[0] > 0.0)) *singular = 1;
-    }
-    __syncthreads();
-    int pr = piv;
-    if (pr != col) {
-      for (int l = threadIdx.x; l < n; l += blockDim.x) {
-        z64 t1 = a[(int64_t)pr * n + l];
-        a[(int64_t)pr * n + l] = a[(int64_t)col * n + l];
-        a[(int64_t)col * n + l] = t1;
-        z64 t2 = inv[(int64_t)pr * n + l];
-        inv[(int64_t)pr * n + l] = inv[(int64_t)col * n + l];
-        inv[(int64_t)col * n + l] = t2;
-      }
-    }
-    __syncthreads();
-    z64 d = a[(int64_t)col * n + col];
-    double den = abs2(d);
-    z64 rd = den > 0.0 ? mk(d.re / den, -d.im / den) : mk(0.0, 0.0);
-    __syncthreads();
-    for (int l = threadIdx.x; l < n; l += blockDim.x) {
-      a[(int64_t)col * n + l] = rd * a[(int64_t)col * n + l];
-      inv[(int64_t)col * n + l] = rd * inv[(int64_t)col * n + l];
-    }
-    __syncthreads();
-    for (int64_t t = threadIdx.x; t < (int64_t)n * n; t += blockDim.x) {
-      int r = (int)(t / n), l = (int)(t % n);
-      if (r == col) continue;
-      z64 fct = a[(int64_t)r * n + col];
-      if (l != col) {
-        a[t] = a[t] - fct * a[(int64_t)col * n + l];
-      }
-      inv[t] = inv[t] - fct * inv[(int64_t)col * n + l];
-    }
-    __syncthreads();
-    for (int r = threadIdx.x; r < n; r += blockDim.x)
-      if (r != col) a[(int64_t)r * n + col] = mk(0.0, 0.0);
-    __syncthreads();
+// Gauss-Jordan inversion with partial pivoting of the n x n complex matrices
+// K + tau M of the coarsest level (n <= MAX_COARSE), in place: the columns
+// already eliminated hold the columns of the inverse that have left the
+// identity. With d the pivot, column `col` of the step:
+//   pivot row:   p_l = (1/d) a_l,  p_col = 1/d
+//   other rows:  a_l - f p_l with f the row's entry in column col; -f p_col there
+// The inverse's column of position c is that of the row that was swapped into c.
+__device__ __forceinline__ z64 gj_recip(z64 d) {
+  const double den = abs2(d);
+  return den > 0.0 ? mk(d.re / den, -d.im / den) : mk(0.0, 0.0);
+}
+
+// larger |v|^2 wins, the smaller row on a tie
+__device__ __forceinline__ void gj_better(double ov, int oi, double* v, int* i) {
+  if (ov > *v || (ov == *v && oi < *i)) {
+    *v = ov;
+    *i = oi;
   }
 }
 
-template <typename T>
-__global__ void k_to_prec(const z64* __restrict__ a, cx<T>* __restrict__ b, int64_t n) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < n) b[t] = cvt<T>(a[t]);
+// One elimination step over the whole chip. One block per tau, as this was
+// before, is bound by one SM's FP64 rate (2 fused multiply-adds a clock) and
+// by its reads of the matrix: 265 ms for four 625 x 625 matrices. Here a block
+// updates a 32 x 32 tile, read from S and written to D (the two buffers
+// alternate, so a step needs no barrier inside the grid). Every block finds
+// the pivot itself from the step's column, which the step before left
+// contiguous in `cin`. The matrix is banded (5 or 7 diagonals): rows whose
+// entry in the column is zero and tiles whose pivot row is zero are copied.
+constexpr int GJ_T = 32;
+__global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64* __restrict__ D,
+                                                 const z64* __restrict__ cin, z64* __restrict__ cout,
+                                                 int32_t* __restrict__ piv, int n, int col, int* singular) {
+  pdl_enter();
+  const int q = blockIdx.z, lane = threadIdx.x, w = threadIdx.y, t = w * 32 + lane;
+  const z64* a = S + (int64_t)q * n * n;
+  z64* o = D + (int64_t)q * n * n;
+  const z64* cc = cin + (int64_t)q * n;
+  __shared__ double sv[8];
+  __shared__ int si[8];
+  const int l = blockIdx.x * GJ_T + lane, r0 = blockIdx.y * GJ_T;
+  // the tile's rows, before the swap (their latency overlaps the search)
+  z64 v[GJ_T / 8], f[GJ_T / 8];
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int r = r0 + w + 8 * h;
+    v[h] = l < n && r < n ? a[(int64_t)r * n + l] : mk(0.0, 0.0);
+    f[h] = r < n ? cc[r] : mk(0.0, 0.0);
+  }
+  double bv = -1.0;
+  int bi = col;
+  for (int r = col + t; r < n; r += 256) gj_better(abs2(cc[r]), r, &bv, &bi);
+  for (int d = 16; d > 0; d >>= 1) {
+    const double ov = __shfl_xor_sync(0xffffffffu, bv, d);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, d);
+    gj_better(ov, oi, &bv, &bi);
+  }
+  if (lane == 0) {
+    sv[w] = bv;
+    si[w] = bi;
+  }
+  __syncthreads();
+  bv = sv[0];
+  bi = si[0];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) gj_better(sv[k], si[k], &bv, &bi);
+  const int pr = bi;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) {
+    piv[(int64_t)q * n + col] = pr;
+    if (!(bv > 0.0)) *singular = 1;
+  }
+  const z64 rd = gj_recip(cc[pr]);
+  z64 p = mk(0.0, 0.0);
+  if (l < n) p = l == col ? rd : rd * a[(int64_t)pr * n + l];
+  const bool any = __any_sync(0xffffffffu, p.re != 0.0 || p.im != 0.0);
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int r = r0 + w + 8 * h;
+    if (l >= n || r >= n) continue;
+    z64 x = v[h], fr = f[h];
+    if (r == pr && pr != col) {
+      x = a[(int64_t)col * n + l];
+      fr = cc[col];
+    }
+    if (l == col) x = mk(0.0, 0.0);
+    if (r == col) x = p;
+    else if (any && (fr.re != 0.0 || fr.im != 0.0)) x = x - fr * p;
+    o[(int64_t)r * n + l] = x;
+    if (l == col + 1) cout[(int64_t)q * n + r] = x;
+  }
 }
 
-// z = Ainv[tau] f on the coarsest level, one row per thread.
+// The inverse in the cycle precision, transposed (Ainv[l][r], so that the
+// threads that own the rows of a product read consecutive values) and with its
+// columns put back in the order of the rows before pivoting.
 template <typename T>
-__global__ void k_coarse_solve(const cx<T>* __restrict__ Ainv, int n, const SlotState* st,
-                               const cx<T>* __restrict__ f, cx<T>* __restrict__ z, int64_t vs) {
-  int slot = blockIdx.y;
+__global__ void __launch_bounds__(256) k_gj_finish(const z64* __restrict__ S, const int32_t* __restrict__ piv,
+                                                   cx<T>* __restrict__ out, int n) {
+  __shared__ int org[MAX_COARSE];
+  __shared__ cx<T> tile[GJ_T][GJ_T + 1];
+  const int q = blockIdx.z, lane = threadIdx.x, w = threadIdx.y, t = w * 32 + lane;
+  const int32_t* pv = piv + (int64_t)q * n;
+  int moved = 0;
+  for (int c = t; c < n; c += 256) {
+    org[c] = c;
+    moved |= pv[c] != c;
+  }
+  if (__syncthreads_or(moved)) {
+    if (t == 0)
+      for (int c = 0; c < n; ++c) {
+        const int pr = pv[c], k = org[c];
+        org[c] = org[pr];
+        org[pr] = k;
+      }
+    __syncthreads();
+  }
+  const int l0 = blockIdx.x * GJ_T, r0 = blockIdx.y * GJ_T;
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int r = r0 + w + 8 * h;
+    if (r < n && l0 + lane < n) tile[w + 8 * h][lane] = cvt<T>(S[((int64_t)q * n + r) * n + l0 + lane]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int l = l0 + w + 8 * h;
+    if (l < n && r0 + lane < n) out[((int64_t)q * n + org[l]) * n + r0 + lane] = tile[lane][w + 8 * h];
+  }
+}
+
+// Up to GJ_SMALL unknowns: the whole inversion in one block per tau, the
+// matrix in shared memory, one warp searching the pivot. A step costs three
+// block barriers (about 0.5 us) against the 2.5 us of a launch; from about 40
+// unknowns on, the FP64 rate of one SM costs more than the launches.
+constexpr int GJ_SMALL = 40;
+template <typename T>
+__global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<T>* __restrict__ out, int n,
+                                                  int* singular) {
+  __shared__ z64 m[GJ_SMALL * GJ_SMALL];
+  __shared__ int org[GJ_SMALL];
+  __shared__ int spr;
+  const int t = threadIdx.x, q = blockIdx.x, nn = n * n;
+  constexpr int PER = (GJ_SMALL * GJ_SMALL + 511) / 512;
+  for (int e = t; e < nn; e += 512) m[e] = A[(int64_t)q * nn + e];
+  if (t < n) org[t] = t;
+  __syncthreads();
+  for (int col = 0; col < n; ++col) {
+    if (t < 32) {
+      double bv = -1.0;
+      int bi = col;
+      for (int r = col + t; r < n; r += 32) gj_better(abs2(m[r * n + col]), r, &bv, &bi);
+      for (int d = 16; d > 0; d >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, d);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, d);
+        gj_better(ov, oi, &bv, &bi);
+      }
+      if (t == 0) {
+        spr = bi;
+        if (!(bv > 0.0)) *singular = 1;
+        const int k = org[col];
+        org[col] = org[bi];
+        org[bi] = k;
+      }
+    }
+    __syncthreads();
+    const int pr = spr;
+    const z64 rd = gj_recip(m[pr * n + col]);
+    z64 x[PER];
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      const int e = t + 512 * h;
+      if (e >= nn) break;
+      const int r = e / n, l = e - r * n;
+      const int sr = r == col ? pr : (r == pr ? col : r);
+      const z64 p = l == col ? rd : rd * m[pr * n + l];
+      const z64 f = m[sr * n + col];
+      x[h] = l == col ? mk(0.0, 0.0) : m[sr * n + l];
+      if (r == col) x[h] = p;
+      else if (f.re != 0.0 || f.im != 0.0) x[h] = x[h] - f * p;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      const int e = t + 512 * h;
+      if (e < nn) m[e] = x[h];
+    }
+    __syncthreads();
+  }
+  for (int e = t; e < nn; e += 512) {
+    const int l = e / n, r = e - l * n;
+    out[((int64_t)q * n + org[l]) * n + r] = cvt<T>(m[r * n + l]);
+  }
+}
+
+// z = Ainv[tau] f on the coarsest level when it is a level of its own (Ainv
+// transposed): a block owns CS_BYTES / sizeof rows. All of its threads form the
+// products of those rows, from coalesced reads; then one thread per row adds
+// its products in the order of the tail kernels' loop, so the bits are theirs.
+// The single-block tail reads the n x n inverse through one SM.
+template <typename T>
+__global__ void __launch_bounds__(256) k_coarse_solve(const cx<T>* __restrict__ Ainv, int n, const SlotState* st,
+                                                      const cx<T>* __restrict__ f, cx<T>* __restrict__ z,
+                                                      int64_t vs) {
+  pdl_enter();
+  constexpr int RB = coarse_rows<T>();
+  extern __shared__ __align__(16) unsigned char cs_smem[];
+  cx<T>* pr = (cx<T>*)cs_smem;
+  const int slot = blockIdx.y;
   if (!slot_running(st, slot)) return;
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  const cx<T>* a = Ainv + ((int64_t)st[slot].tau * n + r) * n;
+  const int r0 = blockIdx.x * RB;
+  const cx<T>* a = Ainv + (int64_t)st[slot].tau * n * n;
   const cx<T>* fs = f + slot * vs;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < n * RB; e += 256) {
+    const int l = e / RB, r = r0 + (e - l * RB);
+    pr[e] = r < n ? a[(int64_t)l * n + r] * fs[l] : mk(T(0), T(0));
+  }
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t >= RB || r0 + t >= n) return;
   cx<T> acc = mk(T(0), T(0));
-  for (int l = 0; l < n; ++l) acc = acc + a[l] * fs[l];
-  z[slot * vs + r] = acc;
+#pragma unroll 16
+  for (int l = 0; l < n; ++l) acc = acc + pr[l * RB + t];
+  z[slot * vs + r0 + t] = acc;
 }
 
 // --------------------------------------------------------------------- defect correction
@@ -1295,20 +1426,39 @@ void launch_invd(const LevelHost& L, const z64* taus, int ntau, cx<T>* out, cuda
   else k_invd<T, double><<<nb(L.n, 256), 256, 0, s>>>(view<double>(L), taus, ntau, out);
 }
 
-void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* inv, int* singular,
-                           cudaStream_t s, int from_f32) {
-  if (from_f32) k_coarse_dense<float><<<nb(L.n, 128), 128, 0, s>>>(view_as<double, float>(L), taus, ntau, work);
-  else k_coarse_dense<double><<<nb(L.n, 128), 128, 0, s>>>(view<double>(L), taus, ntau, work);
-  k_gauss_jordan<<<ntau, 1024, 0, s>>>(work, inv, (int)L.n, singular);
+template <typename T>
+void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
+                           int* singular, cudaStream_t s, int from_f32) {
+  const int n = (int)L.n;
+  const int64_t nn = (int64_t)n * n;
+  const bool small = n <= GJ_SMALL;
+  // the steps' column buffers and pivots live in inv's memory until the finish
+  // overwrites it (48 n bytes or fewer of its n^2 sizeof(cx<T>) per tau); the
+  // pivots move to the dead matrix buffer first
+  z64* cb[2] = {(z64*)inv, (z64*)inv + (int64_t)ntau * n};
+  int32_t* piv = (int32_t*)(cb[1] + (int64_t)ntau * n);
+  cudaMemsetAsync(work, 0, sizeof(z64) * nn * ntau, s);
+  z64* c0 = small ? nullptr : cb[0];
+  const dim3 gd(nb(n, 128), ntau);
+  if (from_f32) k_coarse_dense<float><<<gd, 128, 0, s>>>(view_as<double, float>(L), taus, work, c0);
+  else k_coarse_dense<double><<<gd, 128, 0, s>>>(view<double>(L), taus, work, c0);
+  if (small) {
+    k_gj_small<T><<<ntau, 512, 0, s>>>(work, inv, n, singular);
+    return;
+  }
+  z64 *src = work, *dst = work2;
+  const unsigned nt = nb(n, GJ_T);
+  for (int col = 0; col < n; ++col) {
+    launch_pdl(k_gj_step, dim3(nt, nt, ntau), dim3(32, 8), 0, s, src, dst, cb[col & 1], cb[(col + 1) & 1], piv, n, col,
+               singular);
+    std::swap(src, dst);
+  }
+  cudaMemcpyAsync(dst, piv, sizeof(int32_t) * n * ntau, cudaMemcpyDeviceToDevice, s);
+  k_gj_finish<T><<<dim3(nt, nt, ntau), dim3(32, 8), 0, s>>>(src, (const int32_t*)dst, inv, n);
 }
 
 void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, cudaStream_t s) {
   k_round_bf16<<<nb(n, 256), 256, 0, s>>>(a, b, r, n);
-}
-
-template <typename T>
-void launch_to_prec(const z64* a, cx<T>* b, int64_t n, cudaStream_t s) {
-  k_to_prec<T><<<nb(n, 256), 256, 0, s>>>(a, b, n);
 }
 
 template <typename T>
@@ -1449,6 +1599,8 @@ template <typename T>
 void tail_prepare(size_t smem_bytes) {
   cudaFuncSetAttribute(k_tail_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_tail2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(MAX_COARSE * coarse_rows<T>() * sizeof(cx<T>)));
 }
 
 template <typename T>
@@ -1462,8 +1614,8 @@ void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st,
 template <typename T>
 void launch_coarse_solve(const cx<T>* Ainv, int n, const SlotState* st, const cx<T>* f, cx<T>* z, int64_t vs,
                          int nslot, cudaStream_t s) {
-  dim3 g(nb(n, 128), nslot);
-  k_coarse_solve<T><<<g, 128, 0, s>>>(Ainv, n, st, f, z, vs);
+  dim3 g(nb(n, coarse_rows<T>()), nslot);
+  launch_pdl(k_coarse_solve<T>, g, 256, (size_t)n * coarse_rows<T>() * sizeof(cx<T>), s, Ainv, n, st, f, z, vs);
 }
 
 template <typename T>
@@ -1528,7 +1680,8 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
   template void tail_prepare<T>(size_t);                                                                          \
   template void launch_tail<T>(const TailParams<T>&, size_t, const SlotState*, int, cudaStream_t);                \
   template void launch_invd<T>(const LevelHost&, const z64*, int, cx<T>*, cudaStream_t, int);                     \
-  template void launch_to_prec<T>(const z64*, cx<T>*, int64_t, cudaStream_t);                                     \
+  template void launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \
+                                         int);                                                                    \
   template void launch_apply<T>(const LevelHost&, z64, const SlotState*, const z64*, const cx<T>*, cx<T>*, int64_t, \
                                 int, cudaStream_t);                                                               \
   template void launch_gs<T>(const LevelHost&, const SlotState*, const cx<T>*, const cx<T>*, cx<T>*, int64_t, int,  \

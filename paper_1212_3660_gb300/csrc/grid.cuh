@@ -23,7 +23,7 @@ template <typename T>
 struct TailParams {
   int nlev;                // levels lt .. coarsest
   TailLevel<T> lev[MAX_LEVELS];
-  const cx<T>* Ainv;       // [n_tau][nc][nc]
+  const cx<T>* Ainv;       // [n_tau][nc][nc], each inverse transposed
   int nc;
   uint32_t mask;
   const cx<T>* f_in;       // level-lt right-hand side (global), slot stride vs
@@ -88,12 +88,13 @@ void launch_to_f32(const double* a, float* b, int64_t n, cudaStream_t s);
 // rounded values) instead of its fp64 ones
 template <typename T>
 void launch_invd(const LevelHost& L, const z64* taus, int ntau, cx<T>* out, cudaStream_t s, int from_f32 = 0);
-void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* inv, int* singular,
-                           cudaStream_t s, int from_f32 = 0);
+// inv[q] = (K + tau_q M)^{-1} of the coarsest level in the cycle precision,
+// transposed; work, work2: n_tau n^2 values each.
+template <typename T>
+void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
+                           int* singular, cudaStream_t s, int from_f32 = 0);
 // b = a rounded to bf16, r = the same value as fp32
 void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, cudaStream_t s);
-template <typename T>
-void launch_to_prec(const z64* a, cx<T>* b, int64_t n, cudaStream_t s);
 template <typename T>
 void launch_apply(const LevelHost& L, z64 sfix, const SlotState* st, const z64* taus, const cx<T>* x, cx<T>* y,
                   int64_t vs, int nslot, cudaStream_t s);
@@ -111,6 +112,11 @@ void launch_residual_restrict(const LevelHost& F, const LevelHost& C, const Slot
 template <typename T>
 void launch_prolong_add(const LevelHost& F, const LevelHost& C, uint32_t mask, const SlotState* st, const cx<T>* zc,
                         int64_t vsc, cx<T>* z, int64_t vs, int nslot, cudaStream_t s);
+// rows per block of the coarsest product on its own: 64 KB of products at 1024 unknowns
+template <typename T>
+constexpr int coarse_rows() { return sizeof(T) == 8 ? 4 : 8; }
+// coarsest levels above this run in launch_coarse_solve when no other level is in the tail
+constexpr int COARSE_ALONE = 64;
 template <typename T>
 void launch_coarse_solve(const cx<T>* Ainv, int n, const SlotState* st, const cx<T>* f, cx<T>* z, int64_t vs,
                          int nslot, cudaStream_t s);
