@@ -129,16 +129,19 @@ __global__ void k_mass(const SlotState* st, const double* __restrict__ mm, const
 }
 
 // Partial h_i = sum_rows conj(V_i[row]) w[row] for columns i < k, over a
-// block of MD_THREADS * MD_ROWS rows and a chunk of MD_COLS columns.
+// block of MD_THREADS * MD_ROWS rows and a chunk of COLS columns (mdot_cols;
+// the sums do not depend on it).
+template <int COLS>
 __global__ void __launch_bounds__(MD_THREADS) k_mdot(const SlotState* st, const z64* __restrict__ V, int64_t vsV,
-                                                     const z64* __restrict__ w, int64_t n, z64* __restrict__ partial) {
+                                                     const z64* __restrict__ w, int64_t n,
+                                                     z64* __restrict__ partial) {
   int slot = blockIdx.y;
   if (!st[slot].active) return;
   int k = st[slot].k;
-  int c0 = blockIdx.z * MD_COLS;
+  int c0 = blockIdx.z * COLS;
   if (c0 >= k) return;
-  int c1 = min(k, c0 + MD_COLS);
-  __shared__ z64 red[MD_THREADS / 32][MD_COLS];
+  int c1 = min(k, c0 + COLS);
+  __shared__ z64 red[MD_THREADS / 32][COLS];
   int64_t row0 = (int64_t)blockIdx.x * MD_THREADS * MD_ROWS + threadIdx.x;
   z64 wr[MD_ROWS];
 #pragma unroll
@@ -180,16 +183,17 @@ __global__ void __launch_bounds__(MD_THREADS) k_mdot(const SlotState* st, const 
 // summed by k_hreduce). Its error (about 1e-7 ||w||) is removed by the second,
 // complex128 projection; both updates w -= V h stay complex128, so the Arnoldi
 // relation M z_k = V_{k+1} h holds to complex128 rounding with h = h1 + h2.
+template <int COLS>
 __global__ void __launch_bounds__(MD_THREADS) k_mdot32(const SlotState* st, const z32* __restrict__ V, int64_t vsV,
                                                        const z64* __restrict__ w, int64_t n,
                                                        z64* __restrict__ partial) {
   int slot = blockIdx.y;
   if (!st[slot].active) return;
   int k = st[slot].k;
-  int c0 = blockIdx.z * MD_COLS;
+  int c0 = blockIdx.z * COLS;
   if (c0 >= k) return;
-  int c1 = min(k, c0 + MD_COLS);
-  __shared__ z32 red[MD_THREADS / 32][MD_COLS];
+  int c1 = min(k, c0 + COLS);
+  __shared__ z32 red[MD_THREADS / 32][COLS];
   int64_t row0 = (int64_t)blockIdx.x * MD_THREADS * MD_ROWS + threadIdx.x;
   z32 wr[MD_ROWS];
 #pragma unroll
@@ -627,15 +631,40 @@ void launch_mass(const SlotState* st, const double* mm, const z64* Z, int64_t vs
   k_mass<<<g, 256, 0, s>>>(st, mm, Z, vsZ, w, n, partial);
 }
 int mdot_blocks(int64_t n) { return (int)nbk(n, MD_THREADS * MD_ROWS); }
+// Columns per block of the projections. A block's 4096 rows of one column keep
+// one SM's FP64 pipe busy for 4.6 us, so with 16 columns each the few row
+// blocks of a small problem left most SMs idle (65 us per projection from 4096
+// rows up to 512^2). Fewer columns per block until 24 of them (a usual step)
+// give two blocks per SM; w is then read again per chunk, from L2.
+static int mdot_cols(int64_t n, int nslot) {
+  const int64_t rb = (int64_t)mdot_blocks(n) * nslot;
+  int c = MD_COLS;
+  while (c > 1 && rb * 24 < (int64_t)c * 304) c /= 2;
+  return c;
+}
 void launch_mdot(const SlotState* st, const z64* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
                  int nslot, cudaStream_t s) {
-  dim3 g(mdot_blocks(n), nslot, nbk(kmax, MD_COLS));
-  k_mdot<<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial);
+  const int cols = mdot_cols(n, nslot);
+  const dim3 g(mdot_blocks(n), nslot, nbk(kmax, cols));
+  switch (cols) {
+    case 1: k_mdot<1><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 2: k_mdot<2><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 4: k_mdot<4><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 8: k_mdot<8><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    default: k_mdot<MD_COLS><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial);
+  }
 }
 void launch_mdot32(const SlotState* st, const z32* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
                    int nslot, cudaStream_t s) {
-  dim3 g(mdot_blocks(n), nslot, nbk(kmax, MD_COLS));
-  k_mdot32<<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial);
+  const int cols = mdot_cols(n, nslot);
+  const dim3 g(mdot_blocks(n), nslot, nbk(kmax, cols));
+  switch (cols) {
+    case 1: k_mdot32<1><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 2: k_mdot32<2><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 4: k_mdot32<4><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    case 8: k_mdot32<8><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
+    default: k_mdot32<MD_COLS><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial);
+  }
 }
 void launch_hreduce(const SlotState* st, const z64* partial, int64_t n, z64* h, int64_t hstride, int nslot,
                     cudaStream_t s) {
