@@ -414,7 +414,8 @@ __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, i
 }
 
 // --------------------------------------------------------------------- fused 2D level kernels
-// One level of the V-cycle on a 2D grid coarsened in both axes, in two
+// One level of the V-cycle on a 2D grid coarsened in both axes (odd sides
+// included: their last coarse cell has one child), in two
 // kernels over TX x TY tiles with a halo of H = 4 cells held in shared memory.
 // Red-black half sweeps only read the other colour, so every half sweep is
 // recomputed on a region that shrinks by one cell per sweep; the tile interior
@@ -489,7 +490,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (TX == 32 ? 6 : 8) : 4) 
     if (gx < L.nx && gy < L.ny) zs[gy * L.nx + gx] = sZ[(yy + FH) * RX + xx + FH];
   }
   // residual + restriction to the (TX/2) x (TY/2) coarse cells of the tile
-  const int cnx = L.nx >> 1, cny = L.ny >> 1;
+  const int cnx = (L.nx + 1) >> 1, cny = (L.ny + 1) >> 1;
   cx<T>* fcs = fc + slot * vsc;
   for (int q = tid; q < (TX / 2) * (TY / 2); q += nt) {
     int Yl = q / (TX / 2), Xl = q - Yl * (TX / 2);
@@ -500,6 +501,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (TX == 32 ? 6 : 8) : 4) 
     for (int b = 0; b < 2; ++b)
       for (int a = 0; a < 2; ++a) {
         int gx = 2 * X + a, gy = 2 * Y + b;
+        if (gx >= L.nx || gy >= L.ny) continue;
         int r = (gy - y0) * RX + (gx - x0);
         int c = gy * L.nx + gx;
         Faces<T> fa = faces_at(L, Cell{gx, gy, 0});
@@ -534,7 +536,7 @@ __global__ void __launch_bounds__(256) k_post2d(LevelView<T> L, uint32_t mask, c
   const cx<T>* zs = z + slot * vs;
   cx<T>* zo = zout + slot * vs;
   const cx<T>* zcs = zc + slot * vsc;
-  const int cnx = L.nx >> 1, cny = L.ny >> 1;
+  const int cnx = (L.nx + 1) >> 1, cny = (L.ny + 1) >> 1;
   const int x0 = blockIdx.x * TX - FH, y0 = blockIdx.y * TY - FH;
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int q = tid; q < RX * RY; q += nt) {
@@ -1549,7 +1551,7 @@ static size_t fused_smem() {
 }
 
 bool fused_level_ok(const LevelHost& L) {
-  return L.nz == 1 && L.rx == 2 && L.ry == 2 && L.rz == 1 && L.nx % 2 == 0 && L.ny % 2 == 0;
+  return L.nz == 1 && L.rx == 2 && L.ry == 2 && L.rz == 1;
 }
 
 template <typename T>
