@@ -6,6 +6,7 @@
 // Every vector kernel takes a batch of sources ("slots") on gridDim.y; vector
 // arguments point at slot 0 and consecutive slots are `vs` elements apart.
 #include <algorithm>
+#include <climits>
 
 #include "grid.cuh"
 #include "stencil.cuh"
@@ -958,16 +959,31 @@ bool tail2d_ok(const std::vector<LevelHost>& Ls, int lt) {
 //   pivot row:   p_l = (1/d) a_l,  p_col = 1/d
 //   other rows:  a_l - f p_l with f the row's entry in column col; -f p_col there
 // The inverse's column of position c is that of the row that was swapped into c.
-__device__ __forceinline__ z64 gj_recip(z64 d) {
+// 1/d, its two parts divided by two lanes of a warp (an FP64 division is a
+// sequence of dependent instructions that costs a whole warp its issue slots)
+__device__ __forceinline__ void gj_recip(z64 d, int lane, z64* out) {
   const double den = abs2(d);
-  return den > 0.0 ? mk(d.re / den, -d.im / den) : mk(0.0, 0.0);
+  if (lane < 2) ((double*)out)[lane] = den > 0.0 ? (lane ? -d.im : d.re) / den : 0.0;
 }
 
-// larger |v|^2 wins, the smaller row on a tie
-__device__ __forceinline__ void gj_better(double ov, int oi, double* v, int* i) {
+// Pivot candidates are compared as integers (the order of non-negative
+// doubles; NaN as 0), which leaves the FP64 pipe to the updates: the larger
+// |v|^2 wins, the smaller row on a tie.
+__device__ __forceinline__ unsigned long long gj_key(z64 v) {
+  const unsigned long long k = (unsigned long long)__double_as_longlong(abs2(v));
+  return k > 0x7ff0000000000000ull ? 0ull : k;
+}
+__device__ __forceinline__ void gj_better(unsigned long long ov, int oi, unsigned long long* v, int* i) {
   if (ov > *v || (ov == *v && oi < *i)) {
     *v = ov;
     *i = oi;
+  }
+}
+__device__ __forceinline__ void gj_warp_best(unsigned long long* v, int* i) {
+  for (int d = 16; d > 0; d >>= 1) {
+    const unsigned long long ov = __shfl_xor_sync(0xffffffffu, *v, d);
+    const int oi = __shfl_xor_sync(0xffffffffu, *i, d);
+    gj_better(ov, oi, v, i);
   }
 }
 
@@ -979,7 +995,9 @@ __device__ __forceinline__ void gj_better(double ov, int oi, double* v, int* i) 
 // the pivot itself from the step's column, which the step before left
 // contiguous in `cin`. The matrix is banded (5 or 7 diagonals): rows whose
 // entry in the column is zero and tiles whose pivot row is zero are copied.
+// GJ_R rows per warp: one while that still fits the chip a few times over.
 constexpr int GJ_T = 32;
+template <int GJ_R>
 __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64* __restrict__ D,
                                                  const z64* __restrict__ cin, z64* __restrict__ cout,
                                                  int32_t* __restrict__ piv, int n, int col, int* singular) {
@@ -988,25 +1006,22 @@ __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64*
   const z64* a = S + (int64_t)q * n * n;
   z64* o = D + (int64_t)q * n * n;
   const z64* cc = cin + (int64_t)q * n;
-  __shared__ double sv[8];
+  __shared__ unsigned long long sv[8];
   __shared__ int si[8];
-  const int l = blockIdx.x * GJ_T + lane, r0 = blockIdx.y * GJ_T;
+  __shared__ z64 srd;
+  const int l = blockIdx.x * GJ_T + lane, r0 = blockIdx.y * 8 * GJ_R;
   // the tile's rows, before the swap (their latency overlaps the search)
-  z64 v[GJ_T / 8], f[GJ_T / 8];
+  z64 v[GJ_R], f[GJ_R];
 #pragma unroll
-  for (int h = 0; h < GJ_T / 8; ++h) {
+  for (int h = 0; h < GJ_R; ++h) {
     const int r = r0 + w + 8 * h;
     v[h] = l < n && r < n ? a[(int64_t)r * n + l] : mk(0.0, 0.0);
     f[h] = r < n ? cc[r] : mk(0.0, 0.0);
   }
-  double bv = -1.0;
-  int bi = col;
-  for (int r = col + t; r < n; r += 256) gj_better(abs2(cc[r]), r, &bv, &bi);
-  for (int d = 16; d > 0; d >>= 1) {
-    const double ov = __shfl_xor_sync(0xffffffffu, bv, d);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, d);
-    gj_better(ov, oi, &bv, &bi);
-  }
+  unsigned long long bv = 0ull;
+  int bi = INT_MAX;
+  for (int r = col + t; r < n; r += 256) gj_better(gj_key(cc[r]), r, &bv, &bi);
+  gj_warp_best(&bv, &bi);
   if (lane == 0) {
     sv[w] = bv;
     si[w] = bi;
@@ -1019,14 +1034,16 @@ __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64*
   const int pr = bi;
   if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) {
     piv[(int64_t)q * n + col] = pr;
-    if (!(bv > 0.0)) *singular = 1;
+    if (bv == 0ull) *singular = 1;
   }
-  const z64 rd = gj_recip(cc[pr]);
-  z64 p = mk(0.0, 0.0);
-  if (l < n) p = l == col ? rd : rd * a[(int64_t)pr * n + l];
-  const bool any = __any_sync(0xffffffffu, p.re != 0.0 || p.im != 0.0);
+  z64 p = l < n ? a[(int64_t)pr * n + l] : mk(0.0, 0.0);
+  if (w == 0) gj_recip(cc[pr], lane, &srd);
+  __syncthreads();
+  const z64 rd = srd;
+  const bool any = __any_sync(0xffffffffu, l == col || p.re != 0.0 || p.im != 0.0);
+  if (any && l < n) p = l == col ? rd : rd * p;
 #pragma unroll
-  for (int h = 0; h < GJ_T / 8; ++h) {
+  for (int h = 0; h < GJ_R; ++h) {
     const int r = r0 + w + 8 * h;
     if (l >= n || r >= n) continue;
     z64 x = v[h], fr = f[h];
@@ -1091,6 +1108,7 @@ __global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<
   __shared__ z64 m[GJ_SMALL * GJ_SMALL];
   __shared__ int org[GJ_SMALL];
   __shared__ int spr;
+  __shared__ z64 srd;
   const int t = threadIdx.x, q = blockIdx.x, nn = n * n;
   constexpr int PER = (GJ_SMALL * GJ_SMALL + 511) / 512;
   for (int e = t; e < nn; e += 512) m[e] = A[(int64_t)q * nn + e];
@@ -1098,17 +1116,14 @@ __global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<
   __syncthreads();
   for (int col = 0; col < n; ++col) {
     if (t < 32) {
-      double bv = -1.0;
-      int bi = col;
-      for (int r = col + t; r < n; r += 32) gj_better(abs2(m[r * n + col]), r, &bv, &bi);
-      for (int d = 16; d > 0; d >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, d);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, d);
-        gj_better(ov, oi, &bv, &bi);
-      }
+      unsigned long long bv = 0ull;
+      int bi = INT_MAX;
+      for (int r = col + t; r < n; r += 32) gj_better(gj_key(m[r * n + col]), r, &bv, &bi);
+      gj_warp_best(&bv, &bi);
+      gj_recip(m[bi * n + col], t, &srd);
       if (t == 0) {
         spr = bi;
-        if (!(bv > 0.0)) *singular = 1;
+        if (bv == 0ull) *singular = 1;
         const int k = org[col];
         org[col] = org[bi];
         org[bi] = k;
@@ -1116,7 +1131,7 @@ __global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<
     }
     __syncthreads();
     const int pr = spr;
-    const z64 rd = gj_recip(m[pr * n + col]);
+    const z64 rd = srd;
     z64 x[PER];
 #pragma unroll
     for (int h = 0; h < PER; ++h) {
@@ -1450,9 +1465,12 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
   }
   z64 *src = work, *dst = work2;
   const unsigned nt = nb(n, GJ_T);
+  // one row per warp up to about eight blocks per SM (312 unknowns at four taus)
+  const bool one = (int64_t)nt * nb(n, 8) * ntau <= 8 * 152 + 400;
   for (int col = 0; col < n; ++col) {
-    launch_pdl(k_gj_step, dim3(nt, nt, ntau), dim3(32, 8), 0, s, src, dst, cb[col & 1], cb[(col + 1) & 1], piv, n, col,
-               singular);
+    z64 *ci = cb[col & 1], *co = cb[(col + 1) & 1];
+    if (one) launch_pdl(k_gj_step<1>, dim3(nt, nb(n, 8), ntau), dim3(32, 8), 0, s, src, dst, ci, co, piv, n, col, singular);
+    else launch_pdl(k_gj_step<4>, dim3(nt, nt, ntau), dim3(32, 8), 0, s, src, dst, ci, co, piv, n, col, singular);
     std::swap(src, dst);
   }
   cudaMemcpyAsync(dst, piv, sizeof(int32_t) * n * ntau, cudaMemcpyDeviceToDevice, s);
