@@ -424,8 +424,6 @@ __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, i
 //   pre : z = four half sweeps from z = 0 (red, black, red, black); write z;
 //         coarse f = sum over children of (f - A z)
 //   post: z += P z_coarse; four half sweeps (black, red, black, red); write z
-constexpr int DEFECT_ROWS = 2;  // rows of cells per thread in the defect kernel
-
 // sum over existing neighbours of t_face * z_nb for a 2D cell held at r in a
 // shared tile of row length RX (same order as nb_sum)
 template <typename T>
@@ -1266,11 +1264,16 @@ struct DecideArgs {
 // partial sums of |r|^2 (and |v|^2 when `with_v`). With D.on the last block of
 // each slot sums the partials in a fixed order and takes the inner-solve
 // decision (the work of k_inner_decide, without a launch of its own).
-template <typename T>
-__global__ void k_defect(LevelView<double> L, SlotState* st, const z64* taus, const z64* __restrict__ diag64,
-                         const z64* __restrict__ v, int64_t vsv, const z64* __restrict__ z, int64_t vsz, int64_t col,
-                         int zero_z, cx<T>* __restrict__ f0, int64_t vsf, double* __restrict__ partial, int with_v,
-                         DecideArgs D) {
+// Bound by the FP64 pipe: 12 fused multiply-adds for the neighbours, 4 for the
+// diagonal, 2 for the norm per cell of a 3D grid. A thread therefore marches
+// over R cells along z (3D) or y (2D), so that the block's reduction (5 warp
+// additions and the block's own) is paid once per R cells, and the neighbours
+// below and above stay in registers.
+template <typename T, bool D3>
+__global__ void __launch_bounds__(GX * GY)
+    k_defect(LevelView<double> L, SlotState* st, const z64* taus, const z64* __restrict__ diag64,
+             const z64* __restrict__ v, int64_t vsv, const z64* __restrict__ z, int64_t vsz, int64_t col, int zero_z,
+             cx<T>* __restrict__ f0, int64_t vsf, double* __restrict__ partial, int with_v, int R, DecideArgs D) {
   pdl_enter();
   int slot = blockIdx.z;
   __shared__ double red[2][GX * GY / 32];
@@ -1283,45 +1286,88 @@ __global__ void k_defect(LevelView<double> L, SlotState* st, const z64* taus, co
     return;
   }
   double r2 = 0.0, v2 = 0.0;
+  const int nx = L.nx, ny = L.ny, sxy = nx * ny;
   const int i = blockIdx.x * GX + threadIdx.x;
-  const int rows = L.ny * L.nz;
   const int64_t off = (int64_t)(st[slot].k - 1) * col;
   const int tau = st[slot].tau;
-  const z64* dg = diag64 ? diag64 + (int64_t)tau * L.n : nullptr;
+  // the column of cells: (i, j, m0 .. m1) in 3D, (i, m0 .. m1) in 2D
+  const int nby = (ny + GY - 1) / GY;
+  const int bz = D3 ? blockIdx.y / nby : 0;
+  const int j = D3 ? (int)(blockIdx.y - bz * nby) * GY + (int)threadIdx.y : 0;
+  const int nm = D3 ? L.nz : ny, step = D3 ? sxy : nx;
+  const int m0 = (D3 ? bz : (int)(blockIdx.y * GY + threadIdx.y)) * R;
+  const int m1 = (i < nx && j < ny) ? min(m0 + R, nm) : m0;
+  const z64* vv = v + slot * vsv + off;
   const z64* zz = z + slot * vsz + off;
-#pragma unroll
-  for (int q = 0; q < DEFECT_ROWS; ++q) {
-    const int row = (blockIdx.y * DEFECT_ROWS + q) * GY + threadIdx.y;
-    if (i >= L.nx || row >= rows) continue;
-    const int k = row / L.ny;
-    const Cell p{i, row - k * L.ny, k};
-    const int c = row * L.nx + i;
-    const z64 vv = v[slot * vsv + off + c];
-    z64 r = vv;
-    if (!zero_z) r = dg ? defect_at(L, p, c, dg[c], vv, zz) : vv - apply_at(L, p, c, taus[tau], zz);
-    f0[slot * vsf + c] = cvt<T>(r);
-    r2 = fmaT(r.re, r.re, r2);
-    r2 = fmaT(r.im, r.im, r2);
-    if (with_v) {
-      v2 = fmaT(vv.re, vv.re, v2);
-      v2 = fmaT(vv.im, vv.im, v2);
+  cx<T>* fo = f0 + slot * vsf;
+  if (m0 < m1 && zero_z) {
+    int c = m0 * step + j * nx + i;
+    for (int m = m0; m < m1; ++m, c += step) {
+      const z64 r = vv[c];
+      fo[c] = cvt<T>(r);
+      r2 = fmaT(r.re, r.re, r2);
+      r2 = fmaT(r.im, r.im, r2);
+      if (with_v) {
+        v2 = fmaT(r.re, r.re, v2);
+        v2 = fmaT(r.im, r.im, v2);
+      }
+    }
+  } else if (m0 < m1) {
+    const z64* dg = diag64 + (int64_t)tau * L.n;
+    int c = m0 * step + j * nx + i;
+    z64 below = m0 > 0 ? zz[c - step] : mk(0.0, 0.0), here = zz[c];
+    // the faces below and above along the march: one load per cell
+    int fm = c;  // face below cell c: fz[c] in 3D, fy[c] in 2D
+    const double* fl = D3 ? L.fz : L.fy;
+    double lo = fl[fm];
+    for (int m = m0; m < m1; ++m, c += step, fm += step) {
+      const bool top = m + 1 < nm;
+      const double hi = fl[fm + step];
+      const z64 above = top ? zz[c + step] : mk(0.0, 0.0);
+      const int row = D3 ? m * ny + j : m;
+      const double xl = L.fx[c + row], xh = L.fx[c + row + 1];
+      z64 a = vv[c];
+      const z64 d = dg[c];
+      // the neighbours in nb_sum's order, then the diagonal as in defect_at
+      if (i > 0) a = axpy(xl, zz[c - 1], a);
+      if (i < nx - 1) a = axpy(xh, zz[c + 1], a);
+      if constexpr (D3) {
+        const int fy = c + m * nx;
+        if (j > 0) a = axpy(L.fy[fy], zz[c - nx], a);
+        if (j < ny - 1) a = axpy(L.fy[fy + nx], zz[c + nx], a);
+      }
+      if (m > 0) a = axpy(lo, below, a);
+      if (top) a = axpy(hi, above, a);
+      a.re = fmaT(-d.re, here.re, fmaT(d.im, here.im, a.re));
+      a.im = fmaT(-d.re, here.im, fmaT(-d.im, here.re, a.im));
+      fo[c] = cvt<T>(a);
+      r2 = fmaT(a.re, a.re, r2);
+      r2 = fmaT(a.im, a.im, r2);
+      below = here;
+      here = above;
+      lo = hi;
     }
   }
   for (int o = 16; o > 0; o >>= 1) r2 += __shfl_down_sync(0xffffffffu, r2, o);
   if (with_v)
     for (int o = 16; o > 0; o >>= 1) v2 += __shfl_down_sync(0xffffffffu, v2, o);
+  constexpr int NW = GX * GY / 32;
   int w = tl >> 5, lane = tl & 31;
   if (lane == 0) { red[0][w] = r2; red[1][w] = v2; }
   __syncthreads();
   const int nblk = gridDim.x * gridDim.y;
-  if (tl == 0) {
-    double a = 0.0, b = 0.0;
-    for (int q = 0; q < GX * GY / 32; ++q) { a += red[0][q]; b += red[1][q]; }
-    partial[((int64_t)slot * nblk + block_linear()) * 2 + 0] = a;
-    partial[((int64_t)slot * nblk + block_linear()) * 2 + 1] = b;
-    if (D.on) {
-      __threadfence();
-      last_blk = atomicAdd(&D.bcount[slot], 1) == nblk - 1;
+  if (w == 0) {
+    double a = lane < NW ? red[0][lane] : 0.0, b = lane < NW ? red[1][lane] : 0.0;
+    for (int o = NW / 2; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (with_v)
+      for (int o = NW / 2; o > 0; o >>= 1) b += __shfl_down_sync(0xffffffffu, b, o);
+    if (lane == 0) {
+      partial[((int64_t)slot * nblk + block_linear()) * 2 + 0] = a;
+      partial[((int64_t)slot * nblk + block_linear()) * 2 + 1] = b;
+      if (D.on) {
+        __threadfence();
+        last_blk = atomicAdd(&D.bcount[slot], 1) == nblk - 1;
+      }
     }
   }
   if (!D.on) return;
@@ -1332,11 +1378,11 @@ __global__ void k_defect(LevelView<double> L, SlotState* st, const z64* taus, co
   double a = 0.0, b = 0.0;
   for (int q = tl; q < nblk; q += GX * GY) {
     a += __ldcg(ps + 2 * q);
-    b += __ldcg(ps + 2 * q + 1);
+    if (with_v) b += __ldcg(ps + 2 * q + 1);
   }
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
+    if (with_v) b += __shfl_down_sync(0xffffffffu, b, o);
   }
   __syncthreads();
   if (lane == 0) { red[0][w] = a; red[1][w] = b; }
@@ -1344,7 +1390,7 @@ __global__ void k_defect(LevelView<double> L, SlotState* st, const z64* taus, co
   if (tl == 0) {
     a = 0.0;
     b = 0.0;
-    for (int q = 0; q < GX * GY / 32; ++q) { a += red[0][q]; b += red[1][q]; }
+    for (int q = 0; q < NW; ++q) { a += red[0][q]; b += red[1][q]; }
     D.bcount[slot] = 0;
     int running = decide_slot(st[slot], slot, a, b, zero_z, D.eps, D.max_cycles, D.replay_cycles, D.m_max, D.relax,
                               D.tol);
@@ -1645,22 +1691,24 @@ void launch_correct(const SlotState* st, z64* z, int64_t zs, int64_t zcol, const
   k_correct<T><<<g, 256, 0, s>>>(st, z, zs, zcol, e, es, n);
 }
 
-static dim3 defect_grid(const LevelHost& L, int nslot) {
-  return dim3(nb(L.nx, GX), nb((int64_t)L.ny * L.nz, GY * DEFECT_ROWS), nslot);
+// Cells per thread of the defect march: 4 while that leaves 5 blocks per SM
+// (then the last wave is a few percent), halved on smaller grids. A function of
+// the grid alone, so that a source's norms do not depend on its batch.
+static int defect_march(const LevelHost& L) {
+  const int64_t cols = L.nz > 1 ? (int64_t)nb(L.nx, GX) * nb(L.ny, GY) : nb(L.nx, GX);
+  int R = 4;
+  while (R > 1 && cols * (L.nz > 1 ? nb(L.nz, R) : nb(L.ny, GY * R)) < 5 * 152) R /= 2;
+  while (L.nz > 1 && (int64_t)nb(L.ny, GY) * nb(L.nz, R) > 65535) R *= 2;  // gridDim.y
+  return R;
+}
+static dim3 defect_grid(const LevelHost& L, int R, int nslot) {
+  return L.nz > 1 ? dim3(nb(L.nx, GX), nb(L.ny, GY) * nb(L.nz, R), nslot)
+                  : dim3(nb(L.nx, GX), nb(L.ny, GY * R), nslot);
 }
 
 int defect_blocks(const LevelHost& L) {
-  dim3 g = defect_grid(L, 1);
+  dim3 g = defect_grid(L, defect_march(L), 1);
   return (int)(g.x * g.y);
-}
-
-template <typename T>
-void launch_defect(const LevelHost& L, const SlotState* st, const z64* taus, const z64* v, int64_t vsv, const z64* z,
-                   int64_t vsz, int64_t col, int zero_z, cx<T>* f0, int64_t vsf, double* partial, int with_v,
-                   int nslot, cudaStream_t s) {
-  DecideArgs D{};
-  launch_pdl(k_defect<T>, defect_grid(L, nslot), B2, 0, s, view<double>(L), const_cast<SlotState*>(st), taus, nullptr, v, vsv,
-                                                   z, vsz, col, zero_z, f0, vsf, partial, with_v, D);
 }
 
 template <typename T>
@@ -1670,8 +1718,14 @@ void launch_defect_decide(const LevelHost& L, SlotState* st, const z64* taus, co
                           int use_cond, cudaGraphConditionalHandle cond, int* flags, int* counter, int* bcount,
                           int nslot, double relax, double tol, cudaStream_t s) {
   DecideArgs D{1, eps, max_cycles, replay_cycles, m_max, use_cond, cond, flags, counter, bcount, nslot, relax, tol};
-  launch_pdl(k_defect<T>, defect_grid(L, nslot), B2, 0, s, view<double>(L), st, taus, diag64, v, vsv, z, vsz, col, zero_z,
-                                                   f0, vsf, partial, zero_z, D);
+  const int R = defect_march(L);
+  const dim3 g = defect_grid(L, R, nslot);
+  if (L.nz > 1)
+    launch_pdl(k_defect<T, true>, g, B2, 0, s, view<double>(L), st, taus, diag64, v, vsv, z, vsz, col, zero_z, f0, vsf,
+               partial, zero_z, R, D);
+  else
+    launch_pdl(k_defect<T, false>, g, B2, 0, s, view<double>(L), st, taus, diag64, v, vsv, z, vsz, col, zero_z, f0,
+               vsf, partial, zero_z, R, D);
 }
 
 void launch_diag64(const LevelHost& L, const z64* taus, int ntau, z64* out, cudaStream_t s) {
@@ -1715,8 +1769,6 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
                                        cudaStream_t);                                                             \
   template void launch_correct<T>(const SlotState*, z64*, int64_t, int64_t, const cx<T>*, int64_t, int64_t, int,  \
                                   cudaStream_t);                                                                  \
-  template void launch_defect<T>(const LevelHost&, const SlotState*, const z64*, const z64*, int64_t, const z64*,  \
-                                 int64_t, int64_t, int, cx<T>*, int64_t, double*, int, int, cudaStream_t);       \
   template void launch_defect_decide<T>(const LevelHost&, SlotState*, const z64*, const z64*, const z64*, int64_t, \
                                         const z64*, int64_t, int64_t, int, cx<T>*, int64_t, double*, double, int, \
                                         const int32_t*, int, int, cudaGraphConditionalHandle, int*, int*, int*, int, \

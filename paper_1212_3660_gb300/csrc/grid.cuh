@@ -124,14 +124,10 @@ template <typename T>
 void launch_correct(const SlotState* st, z64* z, int64_t zs, int64_t zcol, const cx<T>* e, int64_t es, int64_t n,
                     int nslot, cudaStream_t s);
 int defect_blocks(const LevelHost& L);
-template <typename T>
-void launch_defect(const LevelHost& L, const SlotState* st, const z64* taus, const z64* v, int64_t vsv, const z64* z,
-                   int64_t vsz, int64_t col, int zero_z, cx<T>* f0, int64_t vsf, double* partial, int with_v,
-                   int nslot, cudaStream_t s);
-// The defect of launch_defect with the inner-solve decision of
+// r = v - (K + tau M) z into f0 with the inner-solve decision of
 // launch_inner_decide taken by the last block of each slot (one launch);
 // bcount: nslot zero ints, left zero.
-// diag64: [n_tau][n] K_cc + tau M_cc of this level (launch_diag64), or null.
+// diag64: [n_tau][n] K_cc + tau M_cc of this level (launch_diag64).
 template <typename T>
 void launch_defect_decide(const LevelHost& L, SlotState* st, const z64* taus, const z64* diag64, const z64* v,
                           int64_t vsv, const z64* z, int64_t vsz, int64_t col, int zero_z, cx<T>* f0, int64_t vsf,
