@@ -1924,8 +1924,11 @@ fks_status fks_op_grid(fks_ctx* ctx, int dim, const int64_t ncell[3], const doub
         CK(cudaFree(fac_d));
       }
     }
-    CK(cudaMalloc(&op->levels[0].kd64, sizeof(double) * n));
-    launch_kdiag(op->levels[0], op->levels[0].kd64, s);
+    // K's diagonal per level: the complex128 residuals read it instead of summing the faces
+    for (auto& L : op->levels) {
+      CK(cudaMalloc(&L.kd64, sizeof(double) * L.n));
+      launch_kdiag(L, L.kd64, s);
+    }
     for (auto& L : op->levels)
       for (int a = 0; a < 4; ++a) {
         int64_t cnt = a < 3 ? (a == 2 && L.nz == 1 ? 1 : face_count(L, a)) : L.n;

@@ -263,15 +263,17 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
       const ClLevel B = P.lev[li + 1];
       cx<T>* ZB = (cx<T>*)(csm + B.z);
       auto get = [&](int X, int Y, int) -> cx<T> { return zrow(B, ZB, Y - b * B.R, X); };
-      for (int t = tid; t < A.R * A.nx; t += nt) {
-        const int lj = t / A.nx, i = t - lj * A.nx;
+      for (int h = tid; h < A.R * (A.nx / 2); h += nt) {
+        // red cells only (nx is even)
+        const int lj = h / (A.nx / 2), i = 2 * (h - lj * (A.nx / 2)) + ((b * A.R + lj) & 1), t = lj * A.nx + i;
         Z[t] = Z[t] + prolong_value_at<T>(Cell{i, b * A.R + lj, 0}, 2, 2, 1, B.nx, B.ny, 1, P.mask, get);
       }
     } else {
       const cx<T>* ZC = cl.map_shared_rank((cx<T>*)(csm + P.zC), 0);
       auto get = [&](int X, int Y, int) -> cx<T> { return ZC[Y * P.ncx + X]; };
-      for (int t = tid; t < A.R * A.nx; t += nt) {
-        const int lj = t / A.nx, i = t - lj * A.nx;
+      for (int h = tid; h < A.R * (A.nx / 2); h += nt) {
+        // red cells only (nx is even)
+        const int lj = h / (A.nx / 2), i = 2 * (h - lj * (A.nx / 2)) + ((b * A.R + lj) & 1), t = lj * A.nx + i;
         Z[t] = Z[t] + prolong_value_at<T>(Cell{i, b * A.R + lj, 0}, 2, 2, 1, P.ncx, P.ncy, 1, P.mask, get);
       }
     }

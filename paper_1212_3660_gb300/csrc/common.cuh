@@ -139,7 +139,7 @@ struct LevelHost {
   double h[3];
   double* d64[4];     // fx, fy, fz, mm (device)
   float* d32[4];      // fp32 copies (device)
-  double* kd64;       // diagonal of K in fp64 (finest level only; else null)
+  double* kd64;       // diagonal of K in fp64
   // the bf16-smoother option: the coefficients rounded to bf16 (d16), and the
   // same rounded values as fp32 (d32b) for the kernels that read fp32
   __nv_bfloat16* d16[4];

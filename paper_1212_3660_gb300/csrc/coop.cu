@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(COOP_THREADS) k_coop_vcycle(CoopParams<T> P, c
       if (!coop_running(st, slot)) continue;
       const int c = (int)(w - (slot - s0) * A.n);
       const Cell p = cell_of(c, A.nx, A.ny);
+      if ((p.i + p.j + p.k) & 1) continue;  // black cells are overwritten unread
       cx<T>* Z = P.z[l] + (int64_t)slot * A.n;
       Z[c] = Z[c] + prolong_value(p, P.rx[l], P.ry[l], P.rz[l], B.nx, B.ny, B.nz, P.mask,
                                   P.z[l + 1] + (int64_t)slot * B.n);

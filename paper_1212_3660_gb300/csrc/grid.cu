@@ -349,7 +349,8 @@ __global__ void __launch_bounds__(256) k_residual_restrict3(LevelView<T, C> F, i
   fc[slot * vsc + ((int64_t)K * cny + J) * cnx + I] = acc;
 }
 
-// z_fine += P z_coarse
+// z_fine += P z_coarse on the red cells (the black ones are overwritten by the
+// next half sweep before anything reads them)
 template <typename T>
 __global__ void k_prolong_add(LevelView<T> F, int rx, int ry, int rz, int cnx, int cny, int cnz, uint32_t mask,
                               const SlotState* st, const cx<T>* __restrict__ zc, int64_t vsc,
@@ -359,7 +360,7 @@ __global__ void k_prolong_add(LevelView<T> F, int rx, int ry, int rz, int cnx, i
   if (!slot_running(st, slot)) return;
   Cell p;
   int c;
-  if (!grid_cell(F.nx, F.ny, F.nz, &p, &c)) return;
+  if (!grid_color_cell(F.nx, F.ny, F.nz, 0, &p, &c)) return;
   cx<T>* zs = z + slot * vs;
   zs[c] = zs[c] + prolong_value(p, rx, ry, rz, cnx, cny, cnz, mask, zc + slot * vsc);
 }
@@ -369,7 +370,8 @@ __global__ void k_prolong_add(LevelView<T> F, int rx, int ry, int rz, int cnx, i
 // first stages the 18 x 6 x 3 coarse values they interpolate from (planes K -
 // 1, K and K + 1) in shared memory, so each coarse value is read once per
 // block instead of once per fine cell; the interpolation itself is
-// prolong_value_at's, on those values.
+// prolong_value_at's, on those values. Only red cells are updated: one of the
+// two planes' cells of each column.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, int cny, int cnz, uint32_t mask,
                                                       const SlotState* st, const cx<T>* __restrict__ zc,
@@ -384,20 +386,14 @@ __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, i
   const int x0 = blockIdx.x * GX, y0 = by * GY;
   const int X0 = x0 / 2 - 1, Y0 = y0 / 2 - 1;
   const cx<T>* zcs = zc + slot * vsc;
-  // the cells' own values are loaded before the staging barrier, so their
-  // latency overlaps that of the coarse values
+  // the cell's own value is loaded before the staging barrier, so its latency
+  // overlaps that of the coarse values
   const int i = x0 + threadIdx.x, j = y0 + threadIdx.y;
   cx<T>* zs = z + slot * vs;
-  bool own[2];
-  int64_t c[2];
-  cx<T> z0[2];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int k = 2 * K + q;
-    own[q] = i < F.nx && j < F.ny && k < F.nz;
-    c[q] = ((int64_t)k * F.ny + j) * F.nx + i;
-    z0[q] = own[q] ? zs[c[q]] : mk(T(0), T(0));
-  }
+  const int k = 2 * K + ((i + j) & 1);
+  const bool own = i < F.nx && j < F.ny && k < F.nz;
+  const int64_t c = ((int64_t)k * F.ny + j) * F.nx + i;
+  const cx<T> z0 = own ? zs[c] : mk(T(0), T(0));
   for (int t = threadIdx.y * GX + threadIdx.x; t < 3 * SY * SX; t += GX * GY) {
     const int q = t / (SY * SX), rem = t - q * (SY * SX);
     const int yy = rem / SX, xx = rem - yy * SX;
@@ -406,12 +402,9 @@ __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, i
     sc[q][yy][xx] = in ? zcs[((int64_t)Z * cny + Y) * cnx + X] : mk(T(0), T(0));
   }
   __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    if (!own[q]) continue;
-    zs[c[q]] = z0[q] + prolong_value_at<T>(Cell{i, j, 2 * K + q}, 2, 2, 2, cnx, cny, cnz, mask,
-                                            [&](int X, int Y, int Z) { return sc[Z - K + 1][Y - Y0][X - X0]; });
-  }
+  if (!own) return;
+  zs[c] = z0 + prolong_value_at<T>(Cell{i, j, k}, 2, 2, 2, cnx, cny, cnz, mask,
+                                   [&](int X, int Y, int Z) { return sc[Z - K + 1][Y - Y0][X - X0]; });
 }
 
 // --------------------------------------------------------------------- fused 2D level kernels
@@ -504,7 +497,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (TX == 32 ? 6 : 8) : 4) 
         int r = (gy - y0) * RX + (gx - x0);
         int c = gy * L.nx + gx;
         Faces<T> fa = faces_at(L, Cell{gx, gy, 0});
-        T d = fsum(fa), m = L.mm[c];
+        T d = sizeof(T) == 8 && L.kd ? L.kd[c] : fsum(fa), m = L.mm[c];
         cx<T> Az = mk(fmaT(sft.re, m, d), mulT(sft.im, m)) * sZ[r] - nb_sum_tile(L, Cell{gx, gy, 0}, r, RX, sZ);
         acc = acc + (sF[r] - Az);
       }
@@ -542,14 +535,18 @@ __global__ void __launch_bounds__(256) k_post2d(LevelView<T> L, uint32_t mask, c
     int ry = q / RX, rx = q - ry * RX;
     int gx = x0 + rx, gy = y0 + ry;
     bool in = gx >= 0 && gx < L.nx && gy >= 0 && gy < L.ny;
-    if (in) {
-      int c = gy * L.nx + gx;
-      sF[q] = fs[c];
-      sZ[q] = zs[c] + prolong_value(Cell{gx, gy, 0}, 2, 2, 1, cnx, cny, 1, mask, zcs);
-    } else {
-      sF[q] = mk(T(0), T(0));
-      sZ[q] = mk(T(0), T(0));
-    }
+    sF[q] = in ? fs[gy * L.nx + gx] : mk(T(0), T(0));
+  }
+  // z + P zc on the red cells of the region: the first half sweep overwrites the
+  // black ones unread
+  for (int q = tid; q < (RX / 2) * RY; q += nt) {
+    const int ry = q / (RX / 2);
+    const int gy = y0 + ry;
+    int rx = 2 * (q - ry * (RX / 2));
+    if ((x0 + rx + gy) & 1) ++rx;
+    const int gx = x0 + rx;
+    if (gx < 0 || gx >= L.nx || gy < 0 || gy >= L.ny) continue;
+    sZ[ry * RX + rx] = zs[gy * L.nx + gx] + prolong_value(Cell{gx, gy, 0}, 2, 2, 1, cnx, cny, 1, mask, zcs);
   }
   __syncthreads();
   for (int hs = 0; hs < 4; ++hs) {
@@ -710,9 +707,11 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail_vcycle(TailParams<T> P
     const TailLevel<T>& B = P.lev[l + 1];
     cx<T>* Z = sh + A.off + A.L.n;
     const cx<T>* ZC = sh + B.off + B.L.n;
-    for (int c = tid; c < A.L.n; c += nt) {
-      Cell p = cell_of(c, A.L.nx, A.L.ny);
-      Z[c] = Z[c] + prolong_value(p, A.rx, A.ry, A.rz, B.L.nx, B.L.ny, B.L.nz, P.mask, ZC);
+    for (int t = tid; t < ((A.L.nx + 1) >> 1) * A.L.ny * A.L.nz; t += nt) {
+      Cell p;
+      int c;
+      if (color_cell(A.L.nx, A.L.ny, A.L.nz, 0, t, &p, &c))
+        Z[c] = Z[c] + prolong_value(p, A.rx, A.ry, A.rz, B.L.nx, B.L.ny, B.L.nz, P.mask, ZC);
     }
     __syncthreads();
     for (int r = 0; r < 2; ++r) {
@@ -919,10 +918,11 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
     tail2d_load(A, t2_smem, F, tid, tau, q);
     if (q.own) {
       auto get = [&](int X, int Y, int) { return ZC[Y * cnx + X]; };
-      q.z0 = Z[q.c0] + prolong_value_at<T>(Cell{q.i0, q.j, 0}, 2, 2, 1, cnx, cny, 1, P.mask, get);
-      q.z1 = Z[q.c0 + 1] + prolong_value_at<T>(Cell{q.i0 + 1, q.j, 0}, 2, 2, 1, cnx, cny, 1, P.mask, get);
-      Z[q.c0] = q.z0;
-      Z[q.c0 + 1] = q.z1;
+      // the red cell of the pair
+      const int h = q.j & 1;
+      const cx<T> v = Z[q.c0 + h] + prolong_value_at<T>(Cell{q.i0 + h, q.j, 0}, 2, 2, 1, cnx, cny, 1, P.mask, get);
+      (h ? q.z1 : q.z0) = v;
+      Z[q.c0 + h] = v;
     }
     __syncthreads();
     for (int r = 0; r < 2; ++r) {
@@ -1603,7 +1603,7 @@ void launch_prolong_add(const LevelHost& F, const LevelHost& C, uint32_t mask, c
     launch_pdl(k_prolong_add3<T>, g, B2, 0, s, view<T>(F), C.nx, C.ny, C.nz, mask, st, zc, vsc, z, vs);
     return;
   }
-  launch_pdl(k_prolong_add<T>, grid2(F.nx, (int64_t)F.ny * F.nz, nslot), B2, 0, s, view<T>(F), F.rx, F.ry, F.rz, C.nx, C.ny,
+  launch_pdl(k_prolong_add<T>, grid2((F.nx + 1) / 2, (int64_t)F.ny * F.nz, nslot), B2, 0, s, view<T>(F), F.rx, F.ry, F.rz, C.nx, C.ny,
                                                                             C.nz, mask, st, zc, vsc, z, vs);
 }
 

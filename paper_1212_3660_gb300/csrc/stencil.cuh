@@ -168,54 +168,70 @@ __device__ __forceinline__ cx<T> restrict_value(const LevelView<T, C>& F, int rx
   return acc;
 }
 
+// a positive normal float as T (exact), without the FP64 pipe
+template <typename T>
+__device__ __forceinline__ T widen(float w) {
+  if constexpr (sizeof(T) == 4) {
+    return w;
+  } else {
+    const unsigned u = __float_as_uint(w);
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+  }
+}
+
 // (P zc)_c: cell-centred (bi/tri)linear interpolation from the coarser level.
 // Per coarsened axis: 3/4 on the parent, 1/4 on the coarse neighbour on the
 // child's side; past a zero-head face the ghost is -parent (weight 1/2 on the
 // parent), past a no-flow face +parent (weight 1).
 // get(X, Y, Z) returns the coarse value at coarse cell (X, Y, Z).
+// Post-smoothing starts with the black cells and does not read their old
+// values, so only the red ones (i + j + k even) are interpolated.
 template <typename T, typename Get>
 __device__ __forceinline__ cx<T> prolong_value_at(Cell p, int rx, int ry, int rz, int cnx, int cny, int cnz,
                                                   uint32_t mask, Get get) {
-  int par[3] = {p.i / rx, p.j / ry, p.k / rz};
   int idx[3] = {p.i, p.j, p.k};
   int rr[3] = {rx, ry, rz};
   int nn[3] = {cnx, cny, cnz};
   int ti[3][2];
-  T tw[3][2];
+  // the weights are products of 1, 3/4, 1/2 and 1/4, exact in float: they are
+  // formed there, and widened with integer instructions (in complex128 their
+  // multiplications and zero tests were 20 of the 38 FP64 instructions per cell)
+  float tw[3][2];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    ti[a][0] = par[a];
-    ti[a][1] = par[a];
+    const int par = rr[a] == 2 ? idx[a] >> 1 : idx[a];
+    ti[a][0] = par;
+    ti[a][1] = par;
     if (rr[a] == 1) {
-      tw[a][0] = T(1);
-      tw[a][1] = T(0);
+      tw[a][0] = 1.f;
+      tw[a][1] = 0.f;
       continue;
     }
-    int nb = (idx[a] & 1) ? par[a] + 1 : par[a] - 1;
+    int nb = (idx[a] & 1) ? par + 1 : par - 1;
     if (nb >= 0 && nb < nn[a]) {
-      tw[a][0] = T(0.75);
+      tw[a][0] = 0.75f;
       ti[a][1] = nb;
-      tw[a][1] = T(0.25);
+      tw[a][1] = 0.25f;
     } else {
       bool dir = nb < 0 ? ((mask >> (2 * a)) & 1u) : ((mask >> (2 * a + 1)) & 1u);
-      tw[a][0] = dir ? T(0.5) : T(1);
-      tw[a][1] = T(0);
+      tw[a][0] = dir ? 0.5f : 1.f;
+      tw[a][1] = 0.f;
     }
   }
   cx<T> acc = mk(T(0), T(0));
 #pragma unroll
   for (int c2 = 0; c2 < 2; ++c2) {
-    T wz = tw[2][c2];
-    if (wz == T(0)) continue;
+    const float wz = tw[2][c2];
+    if (wz == 0.f) continue;
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
-      T wy = tw[1][b];
-      if (wy == T(0)) continue;
+      const float wy = tw[1][b];
+      if (wy == 0.f) continue;
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        T wx = tw[0][a];
-        if (wx == T(0)) continue;
-        acc = axpy(mulT(mulT(wx, wy), wz), get(ti[0][a], ti[1][b], ti[2][c2]), acc);
+        const float wx = tw[0][a];
+        if (wx == 0.f) continue;
+        acc = axpy(widen<T>(wx * wy * wz), get(ti[0][a], ti[1][b], ti[2][c2]), acc);
       }
     }
   }
