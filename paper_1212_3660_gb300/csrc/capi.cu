@@ -505,23 +505,44 @@ static size_t tail_smem(const std::vector<LevelHost>& Ls, int lt) {
   return tail_layout<VT>(Ls, lt, tail_staged<VT>(Ls, lt), nullptr);
 }
 
-// Shared memory of the tail launch from level lt; *pairs = 1 when it is the
-// register-resident 2D kernel (coefficients staged, the levels qualify and the
-// coarsest inverse, staged at *ainv_off, fits as well).
+// Which kernel runs the tail from level lt, and its shared memory: the 2D pair
+// kernel (coefficients staged, the levels qualify and the coarsest inverse,
+// staged at ainv_off, fits as well), else the general pair kernel (up to 1024
+// pairs per level in complex64, 512 in complex128: no coefficients, but a
+// scratch of rlen values at element roff), else k_tail_vcycle.
+struct TailPlan {
+  size_t smem = 0;
+  int pairs = 0, ainv_off = 0;
+  int roff = 0, rlen = 0, threads = 0;
+};
 template <typename VT>
-static size_t tail_launch_smem(const std::vector<LevelHost>& Ls, int lt, int* pairs = nullptr,
-                               int* ainv_off = nullptr) {
-  const size_t b = tail_smem<VT>(Ls, lt);
-  if (pairs) *pairs = 0;
-  if (ainv_off) *ainv_off = 0;
-  if (!tail_staged<VT>(Ls, lt) || !tail2d_ok(Ls, lt)) return b;
+static TailPlan tail_plan(const std::vector<LevelHost>& Ls, int lt) {
+  TailPlan t;
+  t.smem = tail_smem<VT>(Ls, lt);
   const size_t nc = (size_t)Ls.back().n;
-  const size_t a = (b + 15) & ~(size_t)15;
-  const size_t b2 = a + nc * nc * sizeof(cx<VT>);
-  if (b2 > TAIL_SMEM_LIMIT) return b;
-  if (pairs) *pairs = 1;
-  if (ainv_off) *ainv_off = (int)a;
-  return b2;
+  if (tail_staged<VT>(Ls, lt) && tail2d_ok(Ls, lt)) {
+    const size_t a = (t.smem + 15) & ~(size_t)15;
+    const size_t b2 = a + nc * nc * sizeof(cx<VT>);
+    if (b2 <= TAIL_SMEM_LIMIT) {
+      t.smem = b2;
+      t.pairs = 1;
+      t.ainv_off = (int)a;
+      return t;
+    }
+  }
+  const int nt = tail_pairs_threads(Ls, lt, sizeof(VT) == 8);
+  if (nt) {
+    const size_t e = tail_layout<VT>(Ls, lt, false, nullptr) / sizeof(cx<VT>);
+    // the scratch: a level's residuals, or 8 terms of the coarsest product per thread
+    const size_t len = std::max<size_t>(std::max<size_t>((size_t)Ls[lt].n, nc), std::min<size_t>(nc * nc, 8 * (size_t)nt));
+    if ((e + len) * sizeof(cx<VT>) <= TAIL_SMEM_LIMIT) {
+      t.smem = (e + len) * sizeof(cx<VT>);
+      t.roff = (int)e;
+      t.rlen = (int)len;
+      t.threads = nt;
+    }
+  }
+  return t;
 }
 
 // Bytes per tau of the tail's staged coefficients and their shared-memory
@@ -530,7 +551,7 @@ template <typename VT>
 static size_t tail_blob_bytes(const std::vector<LevelHost>& Ls, int64_t tmax, int* coef0) {
   const int lt = tail_level<VT>(Ls, tmax);
   std::vector<int> cb;
-  if (!tail_staged<VT>(Ls, lt)) {
+  if (!tail_staged<VT>(Ls, lt) || tail_plan<VT>(Ls, lt).roff) {
     *coef0 = 0;
     return 0;
   }
@@ -661,6 +682,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     // levels lt .. coarsest in one block per slot
     TailParams<VT> P{};
     P.nlev = nl - lt;
+    const TailPlan tp = tail_plan<VT>(Ls, lt);
     P.staged = tail_staged<VT>(Ls, lt) ? 1 : 0;
     std::vector<int> cbyte;
     tail_layout<VT>(Ls, lt, P.staged != 0, &cbyte);
@@ -690,9 +712,12 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     P.coef0 = S.tcoef0;
     tb += cv * C.n * C.n;
     tf += 8.0 * C.n * C.n;
-    const size_t tsm = tail_launch_smem<VT>(Ls, lt, &P.pairs, &P.ainv_off);
-    if (!P.blob) P.pairs = 0;
-    PROF(FKS_K_TAIL, lt, ns * tb, ns * tf, launch_tail<VT>(P, tsm, S.st, S.nslot, s));
+    P.pairs = P.blob ? tp.pairs : 0;
+    P.ainv_off = tp.ainv_off;
+    P.roff = tp.roff;
+    P.rlen = tp.rlen;
+    P.threads = tp.threads;
+    PROF(FKS_K_TAIL, lt, ns * tb, ns * tf, launch_tail<VT>(P, tp.smem, S.st, S.nslot, s));
   }
   cx<VT>* zfin = Zl(lp);  // final correction of the level below
   for (int l = lp - 1; l >= 0; --l) {
@@ -1103,7 +1128,7 @@ static void setup_levels(Solve& S) {
   const int bf = bf16_of(S) ? 1 : 0;
   {
     std::lock_guard<std::mutex> build_lock(g_build_mu);
-    tail_prepare<VT>(tail_launch_smem<VT>(Ls, tail_level<VT>(Ls, tail_max_of<VT>(S.op))));
+    tail_prepare<VT>(tail_plan<VT>(Ls, tail_level<VT>(Ls, tail_max_of<VT>(S.op))).smem);
     fused_prepare<VT>();
     fused3d_prepare<VT>();
     size_t csm = 0;
@@ -2394,7 +2419,7 @@ fks_status fks_op_autotune(fks_op* op, int precision, fks_c128 tau, void* stream
         {
           // the tail's shared memory and coefficient blob follow the threshold
           std::lock_guard<std::mutex> build_lock(g_build_mu);
-          tail_prepare<VT>(tail_launch_smem<VT>(op->levels, tail_level<VT>(op->levels, ch.tail)));
+          tail_prepare<VT>(tail_plan<VT>(op->levels, tail_level<VT>(op->levels, ch.tail)).smem);
         }
         Arena probe2;
         carve<VT>(S, probe2, false);

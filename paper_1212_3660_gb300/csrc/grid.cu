@@ -939,6 +939,220 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
   }
 }
 
+// --------------------------------------------------------------------- tail by pairs
+// The tail V-cycle for any levels (2D or 3D, odd sides, any coarsening) of at
+// most TAILP_THREADS pairs of cells each: thread t owns the pair (2 p, 2 p + 1)
+// of one row and keeps its coefficients, right-hand side and iterate in
+// registers for the whole visit of the level, so a half sweep is a handful of
+// shared-memory reads and 16 multiply-adds per thread. k_tail_vcycle, which
+// finds its cells again in every half sweep, sums eight residuals per coarse
+// cell one after another and reads the coarsest inverse row by row, was bound
+// by those chains: 16 us for 8^3 and 4^3 cells in complex64.
+// The residuals go through shared memory and are added per coarse cell in
+// restrict_value's order; the coarsest product's terms are formed by all
+// threads (from coalesced reads, the inverse being transposed) and added per
+// row in order: the bits are k_tail_vcycle's.
+template <typename T>
+struct PairCell {  // the pair's coefficients: x faces left, inside, right; y and z faces below and above each cell
+  T x[3], yl[2], yh[2], zl[2], zh[2], m[2];
+  cx<T> id[2], f[2], z[2];
+  int c0, i0, j, k;
+  bool own, right;
+};
+
+template <typename T>
+__device__ __forceinline__ void pair_load(const TailLevel<T>& A, int tau, const cx<T>* F, int t, PairCell<T>& q) {
+  const LevelView<T>& L = A.L;
+  const int npx = (L.nx + 1) >> 1;
+  const int row = t / npx;
+  q.own = row < L.ny * L.nz;
+  if (!q.own) return;
+  q.i0 = 2 * (t - row * npx);
+  q.k = row / L.ny;
+  q.j = row - q.k * L.ny;
+  q.c0 = row * L.nx + q.i0;
+  q.right = q.i0 + 1 < L.nx;
+  const cx<T>* id = A.invd + (int64_t)tau * L.n + q.c0;
+  const T* fx = L.fx + q.c0 + row;
+  const T* fy = L.fy + q.c0 + q.k * L.nx;
+  const T* fz = L.fz + q.c0;
+  const int sxy = L.nx * L.ny;
+  q.x[0] = fx[0];
+  q.x[1] = fx[1];
+  q.x[2] = q.right ? fx[2] : T(0);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const bool on = h == 0 || q.right;
+    q.id[h] = on ? id[h] : mk(T(0), T(0));
+    q.f[h] = on ? F[q.c0 + h] : mk(T(0), T(0));
+    q.yl[h] = on ? fy[h] : T(0);
+    q.yh[h] = on ? fy[L.nx + h] : T(0);
+    q.zl[h] = on && L.nz > 1 ? fz[h] : T(0);
+    q.zh[h] = on && L.nz > 1 ? fz[sxy + h] : T(0);
+    q.m[h] = on ? L.mm[q.c0 + h] : T(0);
+  }
+}
+
+// s + sum t z_nb of cell h of the pair, in nb_sum's order; a neighbour outside
+// the grid adds t * 0
+template <typename T>
+__device__ __forceinline__ cx<T> pair_nb(const PairCell<T>& q, const LevelView<T>& L, const cx<T>* Z, int h, cx<T> s) {
+  const int c = q.c0 + h, sxy = L.nx * L.ny;
+  const cx<T> none = mk(T(0), T(0));
+  const cx<T> far = h ? (q.i0 + 2 < L.nx ? Z[c + 1] : none) : (q.i0 > 0 ? Z[c - 1] : none);
+  const cx<T> own = h ? q.z[0] : q.z[1];
+  s = axpy(h ? q.x[1] : q.x[0], h ? own : far, s);
+  s = axpy(h ? q.x[2] : q.x[1], h ? far : own, s);
+  s = axpy(h ? q.yl[1] : q.yl[0], q.j > 0 ? Z[c - L.nx] : none, s);
+  s = axpy(h ? q.yh[1] : q.yh[0], q.j < L.ny - 1 ? Z[c + L.nx] : none, s);
+  if (L.nz > 1) {
+    s = axpy(h ? q.zl[1] : q.zl[0], q.k > 0 ? Z[c - sxy] : none, s);
+    s = axpy(h ? q.zh[1] : q.zh[0], q.k < L.nz - 1 ? Z[c + sxy] : none, s);
+  }
+  return s;
+}
+
+template <typename T>
+__device__ __forceinline__ void pair_gs(PairCell<T>& q, const LevelView<T>& L, cx<T>* Z, int color, bool zero) {
+  const int h = (q.j + q.k + color) & 1;
+  if (!q.own || (h && !q.right)) return;
+  cx<T> rhs = h ? q.f[1] : q.f[0];
+  if (!zero) rhs = pair_nb(q, L, Z, h, rhs);
+  const cx<T> v = (h ? q.id[1] : q.id[0]) * rhs;
+  if (h) q.z[1] = v;
+  else q.z[0] = v;
+  Z[q.c0 + h] = v;
+}
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const SlotState* st) {
+  pdl_enter();
+  const int slot = blockIdx.x;
+  if (!slot_running(st, slot)) return;
+  extern __shared__ __align__(16) unsigned char tp_smem[];
+  cx<T>* sh = (cx<T>*)tp_smem;
+  cx<T>* R = sh + P.roff;  // residuals of a level, or terms of the coarsest product
+  const int tau = st[slot].tau, t = threadIdx.x;
+  const cx<T> sft = cvt<T>(P.taus[tau]);
+  const cx<T> none = mk(T(0), T(0));
+  PairCell<T> q;
+  {
+    const TailLevel<T>& A = P.lev[0];
+    const cx<T>* fin = P.f_in + slot * P.vs;
+    if (P.nlev > 1) {
+      pair_load(A, tau, fin, t, q);
+      if (q.own) {
+        sh[A.off + q.c0] = q.f[0];
+        if (q.right) sh[A.off + q.c0 + 1] = q.f[1];
+      }
+    } else {
+      for (int c = t; c < A.L.n; c += NT) sh[A.off + c] = fin[c];
+    }
+  }
+  for (int l = 0; l + 1 < P.nlev; ++l) {
+    const TailLevel<T>& A = P.lev[l];
+    const TailLevel<T>& B = P.lev[l + 1];
+    const LevelView<T>& L = A.L;
+    cx<T>* F = sh + A.off;
+    cx<T>* Z = F + L.n;
+    if (l > 0) pair_load(A, tau, F, t, q);
+    q.z[0] = q.z[1] = none;
+    pair_gs(q, L, Z, 0, true);
+    __syncthreads();
+    pair_gs(q, L, Z, 1, false);
+    __syncthreads();
+    pair_gs(q, L, Z, 0, false);
+    __syncthreads();
+    pair_gs(q, L, Z, 1, false);
+    __syncthreads();
+    if (q.own) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (h && !q.right) break;
+        const T d = ((q.x[h] + q.x[h + 1]) + (q.yl[h] + q.yh[h])) + (q.zl[h] + q.zh[h]);
+        const cx<T> Az = mk(fmaT(sft.re, q.m[h], d), mulT(sft.im, q.m[h])) * q.z[h] - pair_nb(q, L, Z, h, none);
+        R[q.c0 + h] = q.f[h] - Az;
+      }
+    }
+    __syncthreads();
+    cx<T>* FC = sh + B.off;
+    for (int C = t; C < B.L.n; C += NT) {
+      const Cell p = cell_of(C, B.L.nx, B.L.ny);
+      cx<T> acc = none;
+      for (int c = 0; c < A.rz; ++c)
+        for (int b = 0; b < A.ry; ++b)
+          for (int a = 0; a < A.rx; ++a) {
+            const int i = A.rx * p.i + a, j = A.ry * p.j + b, k = A.rz * p.k + c;
+            if (i < L.nx && j < L.ny && k < L.nz) acc = acc + R[(k * L.ny + j) * L.nx + i];
+          }
+      FC[C] = acc;
+    }
+    __syncthreads();
+  }
+  {
+    const TailLevel<T>& Cl = P.lev[P.nlev - 1];
+    const cx<T>* F = sh + Cl.off;
+    cx<T>* Z = sh + Cl.off + Cl.L.n;
+    const cx<T>* Ainv = P.Ainv + (int64_t)tau * P.nc * P.nc;
+    const int nc = P.nc, cols = min(nc, P.rlen / nc);
+    if (P.nlev == 1) __syncthreads();
+    cx<T> acc = none;  // nc <= NT
+    for (int l0 = 0; l0 < nc; l0 += cols) {
+      const int lc = min(cols, nc - l0);
+#pragma unroll 4
+      for (int e = t; e < lc * nc; e += NT) R[e] = Ainv[l0 * nc + e] * F[l0 + e / nc];
+      __syncthreads();
+      if (t < nc) {
+#pragma unroll 8
+        for (int l = 0; l < lc; ++l) acc = acc + R[l * nc + t];
+      }
+      __syncthreads();
+    }
+    if (t < nc) {
+      Z[t] = acc;
+      if (P.nlev == 1) P.z_out[slot * P.vs + t] = acc;
+    }
+    __syncthreads();
+  }
+  for (int l = P.nlev - 2; l >= 0; --l) {
+    const TailLevel<T>& A = P.lev[l];
+    const TailLevel<T>& B = P.lev[l + 1];
+    const LevelView<T>& L = A.L;
+    cx<T>* F = sh + A.off;
+    cx<T>* Z = F + L.n;
+    const cx<T>* ZC = sh + B.off + B.L.n;
+    pair_load(A, tau, F, t, q);
+    q.z[0] = q.z[1] = none;
+    const int h = (q.j + q.k) & 1;  // the red cell: the black one is overwritten unread
+    if (q.own && (h == 0 || q.right)) {
+      const cx<T> v = Z[q.c0 + h] +
+                      prolong_value(Cell{q.i0 + h, q.j, q.k}, A.rx, A.ry, A.rz, B.L.nx, B.L.ny, B.L.nz, P.mask, ZC);
+      if (h) q.z[1] = v;
+      else q.z[0] = v;
+      Z[q.c0 + h] = v;
+    }
+    __syncthreads();
+    for (int r = 0; r < 2; ++r) {
+      pair_gs(q, L, Z, 1, false);
+      __syncthreads();
+      pair_gs(q, L, Z, 0, false);
+      __syncthreads();
+    }
+  }
+  if (P.nlev > 1 && q.own) {
+    cx<T>* zout = P.z_out + slot * P.vs;
+    zout[q.c0] = q.z[0];
+    if (q.right) zout[q.c0 + 1] = q.z[1];
+  }
+}
+
+int tail_pairs_threads(const std::vector<LevelHost>& Ls, int lt, bool fp64) {
+  int64_t most = Ls.back().n;  // the coarsest product: a thread per row
+  for (size_t l = lt; l + 1 < Ls.size(); ++l)
+    most = std::max<int64_t>(most, (int64_t)((Ls[l].nx + 1) / 2) * Ls[l].ny * Ls[l].nz);
+  return most <= 512 ? 512 : (most <= 1024 && !fp64 ? 1024 : 0);
+}
+
 bool tail2d_ok(const std::vector<LevelHost>& Ls, int lt) {
   const int nl = (int)Ls.size();
   if (Ls[nl - 1].nz != 1) return false;
@@ -1665,6 +1879,9 @@ template <typename T>
 void tail_prepare(size_t smem_bytes) {
   cudaFuncSetAttribute(k_tail_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_tail2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  cudaFuncSetAttribute(k_tail_pairs<T, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  if constexpr (sizeof(T) == 4)
+    cudaFuncSetAttribute(k_tail_pairs<T, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)(MAX_COARSE * coarse_rows<T>() * sizeof(cx<T>)));
 }
@@ -1673,7 +1890,11 @@ template <typename T>
 void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s) {
   if (P.pairs)
     launch_pdl(k_tail2d<T>, nslot, TAIL_THREADS, smem_bytes, s, P, st);
-  else
+  else if (P.roff && P.threads == 512)
+    launch_pdl(k_tail_pairs<T, 512>, nslot, 512, smem_bytes, s, P, st);
+  else if (P.roff) {
+    if constexpr (sizeof(T) == 4) launch_pdl(k_tail_pairs<T, 1024>, nslot, 1024, smem_bytes, s, P, st);
+  } else
     launch_pdl(k_tail_vcycle<T>, nslot, TAIL_THREADS, smem_bytes, s, P, st);
 }
 

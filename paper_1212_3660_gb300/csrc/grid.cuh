@@ -39,6 +39,9 @@ struct TailParams {
   // inverse of the current tau is staged at shared byte offset ainv_off
   int pairs;
   int ainv_off;
+  // general pair-per-thread variant (tail_pairs_threads): offset and length in
+  // complex elements of its scratch in shared memory (0: not used), block size
+  int roff, rlen, threads;
 };
 
 template <typename T>
@@ -71,6 +74,8 @@ void launch_post3d(const LevelHost& F, uint32_t mask, const SlotState* st, const
 // P.pairs selects the register-resident 2D kernel (same results)
 template <typename T>
 void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s);
+// block size of the pair-per-thread tail of levels lt .. coarsest (0: too large for it)
+int tail_pairs_threads(const std::vector<LevelHost>& Ls, int lt, bool fp64);
 // whether levels lt .. coarsest qualify for the register-resident 2D tail
 bool tail2d_ok(const std::vector<LevelHost>& Ls, int lt);
 
