@@ -2579,7 +2579,7 @@ fks_status fks_op_apply(fks_op* op, fks_c128 sh, const fks_c128* x, fks_c128* y,
     if (op->csr)
       launch_csr_apply<double>(op->cd.view<double>(n), mk(sh.re, sh.im), nullptr, nullptr, xs, ys, n, n_vec, s);
     else
-      launch_apply<double>(op->levels[0], mk(sh.re, sh.im), nullptr, nullptr, xs, ys, n, n_vec, s);
+      launch_apply(op->levels[0], mk(sh.re, sh.im), xs, ys, n, n_vec, s);
     CK(cudaGetLastError());
     if (!yd) CK(cudaMemcpyAsync(y, ys, bytes, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

@@ -202,16 +202,48 @@ __global__ void k_coarse_dense(LevelView<double, C> L, const z64* __restrict__ t
 }
 
 // --------------------------------------------------------------------- apply
-// y = (K + s M) x; the shift is `s` or, with `st`, taus[st[slot].tau].
-template <typename T>
-__global__ void k_apply(LevelView<T> L, z64 s_fixed, const SlotState* st, const z64* taus,
-                        const cx<T>* __restrict__ x, cx<T>* __restrict__ y, int64_t vs) {
-  int slot = blockIdx.z;
-  Cell p;
-  int c;
-  if (!grid_cell(L.nx, L.ny, L.nz, &p, &c)) return;
-  z64 s = st ? taus[st[slot].tau] : s_fixed;
-  y[slot * vs + c] = apply_at(L, p, c, cvt<T>(s), x + slot * vs);
+// y = (K + s M) x, one vector per gridDim.z. Bound by the FP64 pipe, as the
+// defect: 12 fused multiply-adds for a 3D cell's neighbours, 4 for its
+// diagonal, 2 to form it. A thread marches over R cells along z (3D) or y (2D)
+// with the neighbours below and above in registers.
+template <bool D3>
+__global__ void __launch_bounds__(GX * GY) k_apply(LevelView<double> L, z64 s, const z64* __restrict__ x,
+                                                   z64* __restrict__ y, int64_t vs, int R) {
+  const int nx = L.nx, ny = L.ny, sxy = nx * ny;
+  const int i = blockIdx.x * GX + threadIdx.x;
+  const int nby = (ny + GY - 1) / GY;
+  const int bz = D3 ? blockIdx.y / nby : 0;
+  const int j = D3 ? (int)(blockIdx.y - bz * nby) * GY + (int)threadIdx.y : 0;
+  const int nm = D3 ? L.nz : ny, step = D3 ? sxy : nx;
+  const int m0 = (D3 ? bz : (int)(blockIdx.y * GY + threadIdx.y)) * R, m1 = min(m0 + R, nm);
+  if (i >= nx || j >= ny || m0 >= m1) return;
+  const z64* v = x + blockIdx.z * vs;
+  z64* o = y + blockIdx.z * vs;
+  const double* fl = D3 ? L.fz : L.fy;  // the face below cell c along the march
+  int c = m0 * step + j * nx + i;
+  z64 below = m0 > 0 ? v[c - step] : mk(0.0, 0.0), here = v[c];
+  double lo = fl[c];
+  for (int m = m0; m < m1; ++m, c += step) {
+    const bool top = m + 1 < nm;
+    const double hi = fl[c + step];
+    const z64 above = top ? v[c + step] : mk(0.0, 0.0);
+    const int row = D3 ? m * ny + j : m;
+    const double mm = L.mm[c], d = fmaT(s.re, mm, L.kd[c]), e = mulT(s.im, mm);
+    z64 a = mk(0.0, 0.0);
+    if (i > 0) a = axpy(L.fx[c + row], v[c - 1], a);
+    if (i < nx - 1) a = axpy(L.fx[c + row + 1], v[c + 1], a);
+    if constexpr (D3) {
+      const int fy = c + m * nx;
+      if (j > 0) a = axpy(L.fy[fy], v[c - nx], a);
+      if (j < ny - 1) a = axpy(L.fy[fy + nx], v[c + nx], a);
+    }
+    if (m > 0) a = axpy(lo, below, a);
+    if (top) a = axpy(hi, above, a);
+    o[c] = mk(fmaT(d, here.re, fmaT(-e, here.im, -a.re)), fmaT(d, here.im, fmaT(e, here.re, -a.im)));
+    below = here;
+    here = above;
+    lo = hi;
+  }
 }
 
 // --------------------------------------------------------------------- smoother
@@ -1741,12 +1773,6 @@ void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, c
   k_round_bf16<<<nb(n, 256), 256, 0, s>>>(a, b, r, n);
 }
 
-template <typename T>
-void launch_apply(const LevelHost& L, z64 sfix, const SlotState* st, const z64* taus, const cx<T>* x, cx<T>* y,
-                  int64_t vs, int nslot, cudaStream_t s) {
-  k_apply<T><<<grid2(L.nx, (int64_t)L.ny * L.nz, nslot), B2, 0, s>>>(view<T>(L), sfix, st, taus, x, y, vs);
-}
-
 // Sources per block of the multi-source smoother and restriction: a power of
 // two up to 8 (blockDim = (32, 8 / G, G)).
 static int spmm_group(int nslot) {
@@ -1912,23 +1938,30 @@ void launch_correct(const SlotState* st, z64* z, int64_t zs, int64_t zcol, const
   k_correct<T><<<g, 256, 0, s>>>(st, z, zs, zcol, e, es, n);
 }
 
-// Cells per thread of the defect march: 4 while that leaves 5 blocks per SM
+// Cells per thread of the complex128 stencil marches: 4 while that leaves 5 blocks per SM
 // (then the last wave is a few percent), halved on smaller grids. A function of
 // the grid alone, so that a source's norms do not depend on its batch.
-static int defect_march(const LevelHost& L) {
+int march_len(const LevelHost& L) {
   const int64_t cols = L.nz > 1 ? (int64_t)nb(L.nx, GX) * nb(L.ny, GY) : nb(L.nx, GX);
   int R = 4;
   while (R > 1 && cols * (L.nz > 1 ? nb(L.nz, R) : nb(L.ny, GY * R)) < 5 * 152) R /= 2;
   while (L.nz > 1 && (int64_t)nb(L.ny, GY) * nb(L.nz, R) > 65535) R *= 2;  // gridDim.y
   return R;
 }
-static dim3 defect_grid(const LevelHost& L, int R, int nslot) {
+dim3 march_grid(const LevelHost& L, int R, int nslot) {
   return L.nz > 1 ? dim3(nb(L.nx, GX), nb(L.ny, GY) * nb(L.nz, R), nslot)
                   : dim3(nb(L.nx, GX), nb(L.ny, GY * R), nslot);
 }
 
+void launch_apply(const LevelHost& L, z64 sh, const z64* x, z64* y, int64_t vs, int nvec, cudaStream_t s) {
+  const int R = march_len(L);
+  const dim3 g = march_grid(L, R, nvec);
+  if (L.nz > 1) k_apply<true><<<g, B2, 0, s>>>(view<double>(L), sh, x, y, vs, R);
+  else k_apply<false><<<g, B2, 0, s>>>(view<double>(L), sh, x, y, vs, R);
+}
+
 int defect_blocks(const LevelHost& L) {
-  dim3 g = defect_grid(L, defect_march(L), 1);
+  dim3 g = march_grid(L, march_len(L), 1);
   return (int)(g.x * g.y);
 }
 
@@ -1939,8 +1972,8 @@ void launch_defect_decide(const LevelHost& L, SlotState* st, const z64* taus, co
                           int use_cond, cudaGraphConditionalHandle cond, int* flags, int* counter, int* bcount,
                           int nslot, double relax, double tol, cudaStream_t s) {
   DecideArgs D{1, eps, max_cycles, replay_cycles, m_max, use_cond, cond, flags, counter, bcount, nslot, relax, tol};
-  const int R = defect_march(L);
-  const dim3 g = defect_grid(L, R, nslot);
+  const int R = march_len(L);
+  const dim3 g = march_grid(L, R, nslot);
   if (L.nz > 1)
     launch_pdl(k_defect<T, true>, g, B2, 0, s, view<double>(L), st, taus, diag64, v, vsv, z, vsz, col, zero_z, f0, vsf,
                partial, zero_z, R, D);
@@ -1977,8 +2010,6 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
   template void launch_invd<T>(const LevelHost&, const z64*, int, cx<T>*, cudaStream_t, int);                     \
   template void launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \
                                          int);                                                                    \
-  template void launch_apply<T>(const LevelHost&, z64, const SlotState*, const z64*, const cx<T>*, cx<T>*, int64_t, \
-                                int, cudaStream_t);                                                               \
   template void launch_gs<T>(const LevelHost&, const SlotState*, const cx<T>*, const cx<T>*, cx<T>*, int64_t, int,  \
                              int, int, cudaStream_t, z64*, int64_t, int64_t, int);                                \
   template void launch_residual_restrict<T>(const LevelHost&, const LevelHost&, const SlotState*, const z64*,      \

@@ -100,9 +100,8 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
                            int* singular, cudaStream_t s, int from_f32 = 0);
 // b = a rounded to bf16, r = the same value as fp32
 void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, cudaStream_t s);
-template <typename T>
-void launch_apply(const LevelHost& L, z64 sfix, const SlotState* st, const z64* taus, const cx<T>* x, cx<T>* y,
-                  int64_t vs, int nslot, cudaStream_t s);
+// y = (K + sh M) x for nvec vectors of the finest level, vs elements apart
+void launch_apply(const LevelHost& L, z64 sh, const z64* x, z64* y, int64_t vs, int nvec, cudaStream_t s);
 // Zk (optional): the finest level's last half sweep, fused with the defect
 // correction (both cells of each pair are added to column k - 1 of Zk, as
 // launch_correct does; z is not written)
@@ -129,6 +128,10 @@ template <typename T>
 void launch_correct(const SlotState* st, z64* z, int64_t zs, int64_t zcol, const cx<T>* e, int64_t es, int64_t n,
                     int nslot, cudaStream_t s);
 int defect_blocks(const LevelHost& L);
+// cells per thread and grid of the kernels that march along z (3D) or y (2D)
+// with blocks of (GX, GY) threads (nz of the grid: nslot)
+int march_len(const LevelHost& L);
+dim3 march_grid(const LevelHost& L, int R, int nslot);
 // r = v - (K + tau M) z into f0 with the inner-solve decision of
 // launch_inner_decide taken by the last block of each slot (one launch);
 // bcount: nslot zero ints, left zero.

@@ -8,6 +8,7 @@
 //    |g_{k+1}| and the inexact-solve bound of Eq. trueresidual; FFOM solves the
 //    square system (Algorithm 4)
 //  - assembly x_j = Z_{m_j} y_j and the true residual ||b - (K + sigma_j M) x_j||.
+#include "grid.cuh"
 #include "krylov.cuh"
 #include "stencil.cuh"
 
@@ -548,40 +549,69 @@ __global__ void k_assemble(const z64* __restrict__ Z, int64_t vsZ, const z64* __
     if (j0 + jj < nf) X[((int64_t)slot * nf + j0 + jj) * n + row] = acc[jj];
 }
 
-// Partial sums of |b - (K + sigma_j M) x_j|^2, grid (i blocks, row blocks, n_f * slots).
-__global__ void k_tres_partial(LevelView<double> L, const z64* __restrict__ sigma, int nf, const z64* __restrict__ b,
-                               const z64* __restrict__ X, double* __restrict__ partial) {
-  int slot = blockIdx.z / nf, j = blockIdx.z - slot * nf;
+// Partial sums of |b - (K + sigma_j M) x_j|^2, one (source, shift) per
+// gridDim.z. Bound by the FP64 pipe (a 3D cell takes 12 fused multiply-adds for
+// its neighbours, 4 + 2 for the diagonal, 2 for the norm; the arithmetic and
+// its order are defect_at's): as in the defect kernel a thread marches over R
+// cells along z (3D) or y (2D), which leaves the block's reduction a small
+// share.
+template <bool D3>
+__global__ void __launch_bounds__(GX * GY) k_tres_partial(LevelView<double> L, const z64* __restrict__ sigma, int nf,
+                                                          const z64* __restrict__ b, const z64* __restrict__ X,
+                                                          double* __restrict__ partial, int R) {
+  const int slot = blockIdx.z / nf, sh = blockIdx.z - slot * nf;
   __shared__ double red[GX * GY / 32];
-  double a = 0.0;
-  const z64 sg = sigma[j];
-  const z64* x = X + ((int64_t)slot * nf + j) * L.n;
+  const z64 sg = sigma[sh];
+  const z64* x = X + ((int64_t)slot * nf + sh) * L.n;
+  const z64* bs = b + slot * L.n;
+  const int nx = L.nx, ny = L.ny, sxy = nx * ny;
   const int i = blockIdx.x * GX + threadIdx.x;
-  const int rows = L.ny * L.nz;
-#pragma unroll
-  for (int q = 0; q < TRES_ROWS; ++q) {
-    const int row = (blockIdx.y * TRES_ROWS + q) * GY + threadIdx.y;
-    if (i >= L.nx || row >= rows) continue;
-    const int k = row / L.ny;
-    const Cell p{i, row - k * L.ny, k};
-    const int c = row * L.nx + i;
-    // b - (K + sigma M) x with the neighbour terms accumulated onto b
-    const double d = L.kd ? L.kd[c] : fsum(faces_at(L, p));
-    const double mc = L.mm[c];
-    const z64 r = defect_at(L, p, c, mk(fmaT(sg.re, mc, d), mulT(sg.im, mc)), b[slot * L.n + c], x);
-    a = fmaT(r.re, r.re, a);
-    a = fmaT(r.im, r.im, a);
+  const int nby = (ny + GY - 1) / GY;
+  const int bz = D3 ? blockIdx.y / nby : 0;
+  const int j = D3 ? (int)(blockIdx.y - bz * nby) * GY + (int)threadIdx.y : 0;
+  const int nm = D3 ? L.nz : ny, step = D3 ? sxy : nx;
+  const int m0 = (D3 ? bz : (int)(blockIdx.y * GY + threadIdx.y)) * R;
+  const int m1 = (i < nx && j < ny) ? min(m0 + R, nm) : m0;
+  double s = 0.0;
+  if (m0 < m1) {
+    const double* fl = D3 ? L.fz : L.fy;  // the face below cell c along the march
+    int c = m0 * step + j * nx + i;
+    z64 below = m0 > 0 ? x[c - step] : mk(0.0, 0.0), here = x[c];
+    double lo = fl[c];
+    for (int m = m0; m < m1; ++m, c += step) {
+      const bool top = m + 1 < nm;
+      const double hi = fl[c + step];
+      const z64 above = top ? x[c + step] : mk(0.0, 0.0);
+      const int row = D3 ? m * ny + j : m;
+      const double mc = L.mm[c], d = fmaT(sg.re, mc, L.kd[c]), e = mulT(sg.im, mc);
+      z64 a = bs[c];
+      if (i > 0) a = axpy(L.fx[c + row], x[c - 1], a);
+      if (i < nx - 1) a = axpy(L.fx[c + row + 1], x[c + 1], a);
+      if constexpr (D3) {
+        const int fy = c + m * nx;
+        if (j > 0) a = axpy(L.fy[fy], x[c - nx], a);
+        if (j < ny - 1) a = axpy(L.fy[fy + nx], x[c + nx], a);
+      }
+      if (m > 0) a = axpy(lo, below, a);
+      if (top) a = axpy(hi, above, a);
+      a.re = fmaT(-d, here.re, fmaT(e, here.im, a.re));
+      a.im = fmaT(-d, here.im, fmaT(-e, here.re, a.im));
+      s = fmaT(a.re, a.re, s);
+      s = fmaT(a.im, a.im, s);
+      below = here;
+      here = above;
+      lo = hi;
+    }
   }
-  a = warp_sum(a);
-  int tl = thread_linear();
-  if ((tl & 31) == 0) red[tl >> 5] = a;
+  s = warp_sum(s);
+  const int tl = thread_linear();
+  constexpr int NW = GX * GY / 32;
+  if ((tl & 31) == 0) red[tl >> 5] = s;
   __syncthreads();
-  if (tl == 0) {
-    double s = 0.0;
-    for (int q = 0; q < GX * GY / 32; ++q) s += red[q];
-    int nblk = gridDim.x * gridDim.y;
-    partial[((int64_t)slot * nf + j) * nblk + block_linear()] = s;
-  }
+  if (tl >= 32) return;
+  s = tl < NW ? red[tl] : 0.0;
+  for (int o = NW / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (tl == 0) partial[((int64_t)slot * nf + sh) * (gridDim.x * gridDim.y) + block_linear()] = s;
 }
 
 __global__ void k_tres_finish(const SlotState* st, const double* __restrict__ partial, int nblocks, int nf, int nslot,
@@ -704,11 +734,18 @@ void launch_assemble(const z64* Z, int64_t vsZ, const z64* Y, const int32_t* mj,
   dim3 g(nbk(n, 256), nslot, nbk(nf, AS_J));
   k_assemble<<<g, 256, 0, s>>>(Z, vsZ, Y, mj, nf, m, X, n, st, skip_k_le);
 }
-int tres_blocks(const LevelHost& L) { return (int)(nbk(L.nx, GX) * nbk((int64_t)L.ny * L.nz, GY * TRES_ROWS)); }
+// twice the defect's march: the shifts multiply the blocks
+static int tres_march(const LevelHost& L) { return 2 * march_len(L); }
+int tres_blocks(const LevelHost& L) {
+  const dim3 g = march_grid(L, tres_march(L), 1);
+  return (int)(g.x * g.y);
+}
 void launch_true_residual(const LevelHost& L, const z64* sigma, int nf, const z64* b, const z64* X, double* partial,
                           const SlotState* st, double* out, int nslot, cudaStream_t s) {
-  dim3 g(nbk(L.nx, GX), nbk((int64_t)L.ny * L.nz, GY * TRES_ROWS), nf * nslot);
-  k_tres_partial<<<g, dim3(GX, GY), 0, s>>>(view<double>(L), sigma, nf, b, X, partial);
+  const int R = tres_march(L);
+  const dim3 g = march_grid(L, R, nf * nslot);
+  if (L.nz > 1) k_tres_partial<true><<<g, dim3(GX, GY), 0, s>>>(view<double>(L), sigma, nf, b, X, partial, R);
+  else k_tres_partial<false><<<g, dim3(GX, GY), 0, s>>>(view<double>(L), sigma, nf, b, X, partial, R);
   launch_tres_finish(st, partial, tres_blocks(L), nf, nslot, out, s);
 }
 // X[idx[i]] += a[i] Xh[idx[i]] for the columns of a restart cycle (x_j += C_j d_j)
