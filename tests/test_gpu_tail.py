@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("precision", [fks.FKS_PREC_FP64, fks.FKS_PREC_MIXED])
 @pytest.mark.parametrize("shape,mask", [((12, 10, 14), 63), ((14, 12, 13), 21), ((8, 16, 16), 63), ((6, 8, 20), 42),
-                                        ((36, 37), 15), ((3, 90), 15), ((40, 26), 5), ((9, 12, 20), 63)])
+                                        ((36, 37), 15), ((6, 90), 15), ((40, 26), 5), ((9, 12, 20), 63)])
 def test_tail_thresholds_bitwise(shape, mask, precision):
     pr = synth.make_problem(shape, n_f=4, periods=(5.0, 3600.0), n_p=2, seed=37, dirichlet_mask=mask, n_src=2)
     s = Solver(pr)
