@@ -622,6 +622,196 @@ __global__ void __launch_bounds__(256) k_post2d(LevelView<T> L, uint32_t mask, c
   }
 }
 
+// --------------------------------------------------------------------- small tiles by pairs
+// The same two kernels for 8 x 8 tiles, and in complex64 16 x 16 ones, with a
+// pair of cells (2 p, 2 p + 1) of the tile's region per thread: the pair's
+// coefficients, right-hand side and iterate are loaded once, together, into
+// registers. On the small levels these tiles are for, k_pre2d's time is
+// latency: every half sweep waits for its faces and inverse diagonals after
+// its barrier (4.4 us a launch in complex64, 7.6 us in complex128). In
+// complex128 a 16 x 16 tile stays with k_pre2d, whose half sweeps pack the
+// shrinking region's cells into fewer FP64 instructions.
+// Cells outside the grid hold zero, which adds t * 0 for a missing neighbour;
+// cells whose neighbours the region does not hold get values nothing reads
+// (the region shrinks by one cell per half sweep).
+template <typename T, int TX>
+struct TilePair {
+  static constexpr int RX = TX + 2 * FH, PX = RX / 2, NT = PX * RX;
+  static constexpr int GUARD = RX + 2;               // cells read around the region
+  static constexpr int ZN = RX * RX + 2 * GUARD;
+  T x[3], yl[2], yh[2];
+  cx<T> id[2], f[2], z[2];
+  int ry, r, gx, gy, c;      // region row, region index, left cell and its flat index
+  bool in[2];
+  __device__ __forceinline__ void load(const LevelView<T>& L, const cx<T>* ID, const cx<T>* fs) {
+    const int t = threadIdx.x;
+    ry = t / PX;
+    const int rx = 2 * (t - ry * PX);
+    r = ry * RX + rx;
+    gx = (int)blockIdx.x * TX - FH + rx;
+    gy = (int)blockIdx.y * TX - FH + ry;
+    c = gy * L.nx + gx;
+    const bool row = gy >= 0 && gy < L.ny;
+    const T* fx = L.fx + c + gy;
+    const T* fy = L.fy + c;
+    x[0] = x[1] = x[2] = T(0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      in[h] = row && gx + h >= 0 && gx + h < L.nx;
+      id[h] = in[h] ? ID[c + h] : mk(T(0), T(0));
+      f[h] = in[h] ? fs[c + h] : mk(T(0), T(0));
+      z[h] = mk(T(0), T(0));
+      yl[h] = in[h] ? fy[h] : T(0);
+      yh[h] = in[h] ? fy[L.nx + h] : T(0);
+      if (in[h]) {
+        x[h] = fx[h];
+        x[h + 1] = fx[h + 1];
+      }
+    }
+  }
+  // s + sum t z_nb of cell h, in nb_sum's order; Z points at the region's cell 0
+  __device__ __forceinline__ cx<T> nb(const cx<T>* Z, int h, cx<T> s) const {
+    const cx<T> far = h ? Z[r + 2] : Z[r - 1];
+    const cx<T> own = h ? z[0] : z[1];
+    s = axpy(h ? x[1] : x[0], h ? own : far, s);
+    s = axpy(h ? x[2] : x[1], h ? far : own, s);
+    s = axpy(h ? yl[1] : yl[0], Z[r + h - RX], s);
+    s = axpy(h ? yh[1] : yh[0], Z[r + h + RX], s);
+    return s;
+  }
+  // half sweep of `color` on the rows sh .. RX - sh - 1 of the region
+  __device__ __forceinline__ void gs(cx<T>* Z, int color, int sh, bool zero) {
+    const int h = (gy + color) & 1;  // gx is even
+    if (ry < sh || ry >= RX - sh || !(h ? in[1] : in[0])) return;
+    cx<T> rhs = h ? f[1] : f[0];
+    if (!zero) rhs = nb(Z, h, rhs);
+    const cx<T> v = (h ? id[1] : id[0]) * rhs;
+    if (h) z[1] = v;
+    else z[0] = v;
+    Z[r + h] = v;
+  }
+  __device__ __forceinline__ bool interior() const {
+    const int rx = r - ry * RX;
+    return ry >= FH && ry < FH + TX && rx >= FH && rx < FH + TX;
+  }
+};
+
+template <typename T, int TX>
+__global__ void __launch_bounds__(TilePair<T, TX>::NT) k_pre2d_pairs(LevelView<T> L, const SlotState* st,
+                                                                    const cx<T>* __restrict__ invd, const z64* taus,
+                                                                    const cx<T>* __restrict__ f, cx<T>* __restrict__ z,
+                                                                    int64_t vs, cx<T>* __restrict__ fc, int64_t vsc) {
+  using Tile = TilePair<T, TX>;
+  pdl_enter();
+  __shared__ cx<T> zmem[Tile::ZN];
+  __shared__ cx<T> res[TX][TX];
+  const int slot = blockIdx.z;
+  if (!slot_running(st, slot)) return;
+  const int tau = st[slot].tau;
+  const cx<T> sft = cvt<T>(taus[tau]);
+  cx<T>* Z = zmem + Tile::GUARD;
+  Tile q;
+  q.load(L, invd + (int64_t)tau * L.n, f + slot * vs);
+  const bool mine = q.interior();
+  T d[2] = {T(0), T(0)}, m[2] = {T(0), T(0)};
+  if (mine) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (q.in[h]) {
+        m[h] = L.mm[q.c + h];
+        if (sizeof(T) == 8 && L.kd) d[h] = L.kd[q.c + h];
+      }
+  }
+  for (int e = threadIdx.x; e < Tile::ZN; e += Tile::NT) zmem[e] = mk(T(0), T(0));
+  __syncthreads();
+  q.gs(Z, 0, 0, true);
+  __syncthreads();
+  q.gs(Z, 1, 1, false);
+  __syncthreads();
+  q.gs(Z, 0, 2, false);
+  __syncthreads();
+  q.gs(Z, 1, 3, false);
+  __syncthreads();
+  if (mine) {
+    cx<T>* zs = z + slot * vs;
+    const int yy = q.ry - FH, xx = q.r - q.ry * Tile::RX - FH;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!q.in[h]) continue;
+      zs[q.c + h] = q.z[h];
+      if (!(sizeof(T) == 8 && L.kd)) d[h] = ((q.x[h] + q.x[h + 1]) + (q.yl[h] + q.yh[h])) + T(0);
+      const cx<T> Az = mk(fmaT(sft.re, m[h], d[h]), mulT(sft.im, m[h])) * q.z[h] - q.nb(Z, h, mk(T(0), T(0)));
+      res[yy][xx + h] = q.f[h] - Az;
+    }
+  }
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t >= (TX / 2) * (TX / 2)) return;
+  const int Yl = t / (TX / 2), Xl = t - Yl * (TX / 2);
+  const int X = blockIdx.x * (TX / 2) + Xl, Y = blockIdx.y * (TX / 2) + Yl;
+  const int cnx = (L.nx + 1) >> 1, cny = (L.ny + 1) >> 1;
+  if (X >= cnx || Y >= cny) return;
+  cx<T> acc = mk(T(0), T(0));
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+      if (2 * X + a < L.nx && 2 * Y + b < L.ny) acc = acc + res[2 * Yl + b][2 * Xl + a];
+  fc[slot * vsc + (int64_t)Y * cnx + X] = acc;
+}
+
+template <typename T, int TX>
+__global__ void __launch_bounds__(TilePair<T, TX>::NT)
+    k_post2d_pairs(LevelView<T> L, uint32_t mask, const SlotState* st, const cx<T>* __restrict__ invd,
+                   const cx<T>* __restrict__ f, const cx<T>* __restrict__ z, cx<T>* __restrict__ zout, int64_t vs,
+                   const cx<T>* __restrict__ zc, int64_t vsc, z64* __restrict__ Zk, int64_t vsZk, int64_t zcol) {
+  using Tile = TilePair<T, TX>;
+  pdl_enter();
+  __shared__ cx<T> zmem[Tile::ZN];
+  const int slot = blockIdx.z;
+  if (!slot_running(st, slot)) return;
+  const int tau = st[slot].tau;
+  cx<T>* Z = zmem + Tile::GUARD;
+  Tile q;
+  q.load(L, invd + (int64_t)tau * L.n, f + slot * vs);
+  const int cnx = (L.nx + 1) >> 1, cny = (L.ny + 1) >> 1;
+  for (int e = threadIdx.x; e < Tile::ZN; e += Tile::NT) zmem[e] = mk(T(0), T(0));
+  // the red cell of the pair (the black one is overwritten unread)
+  const int h = q.gy & 1;
+  cx<T> v = mk(T(0), T(0));
+  if (h ? q.in[1] : q.in[0])
+    v = z[slot * vs + q.c + h] +
+        prolong_value(Cell{q.gx + h, q.gy, 0}, 2, 2, 1, cnx, cny, 1, mask, zc + slot * vsc);
+  __syncthreads();
+  if (h) q.z[1] = v;
+  else q.z[0] = v;
+  Z[q.r + h] = v;
+  __syncthreads();
+  q.gs(Z, 1, 1, false);
+  __syncthreads();
+  q.gs(Z, 0, 2, false);
+  __syncthreads();
+  q.gs(Z, 1, 3, false);
+  __syncthreads();
+  q.gs(Z, 0, 4, false);
+  if (!q.interior()) return;
+  if (Zk) {
+    z64* zk = Zk + slot * vsZk + (int64_t)(st[slot].k - 1) * zcol + q.c;
+    const bool first = st[slot].cycles == 0;
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+      if (q.in[b]) {
+        const z64 ev = cvt<double>(q.z[b]);
+        zk[b] = first ? ev : (zk[b] + ev);
+      }
+    return;
+  }
+  cx<T>* zo = zout + slot * vs + q.c;
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+    if (q.in[b]) zo[b] = q.z[b];
+}
+
 // --------------------------------------------------------------------- tail
 // The V-cycle of every level from `lt` down (levels small enough for one CTA)
 // in one kernel: one block per slot, level vectors in shared memory,
@@ -1868,15 +2058,17 @@ void fused_prepare() {
 template <typename T>
 void launch_pre2d(const LevelHost& F, const LevelHost& C, const SlotState* st, const cx<T>* invd, const z64* taus,
                   const cx<T>* f, cx<T>* z, int64_t vs, cx<T>* fc, int64_t vsc, int nslot, int tile, cudaStream_t s) {
+  const dim3 g(nb(F.nx, tile), nb(F.ny, tile), nslot);
+  const LevelView<T> L = view<T>(F);
   if (tile == 8) {
-    dim3 g(nb(F.nx, 8), nb(F.ny, 8), nslot);
-    launch_pdl(k_pre2d<T, 8, 8>, g, 256, fused_smem<T, 8, 8>(), s, view<T>(F), st, invd, taus, f, z, vs, fc, vsc);
+    launch_pdl(k_pre2d_pairs<T, 8>, g, TilePair<T, 8>::NT, 0, s, L, st, invd, taus, f, z, vs, fc, vsc);
   } else if (tile == 16) {
-    dim3 g(nb(F.nx, 16), nb(F.ny, 16), nslot);
-    launch_pdl(k_pre2d<T, 16, 16>, g, 256, fused_smem<T, 16, 16>(), s, view<T>(F), st, invd, taus, f, z, vs, fc, vsc);
+    if constexpr (sizeof(T) == 4)
+      launch_pdl(k_pre2d_pairs<T, 16>, g, TilePair<T, 16>::NT, 0, s, L, st, invd, taus, f, z, vs, fc, vsc);
+    else
+      launch_pdl(k_pre2d<T, 16, 16>, g, 256, fused_smem<T, 16, 16>(), s, L, st, invd, taus, f, z, vs, fc, vsc);
   } else {
-    dim3 g(nb(F.nx, 32), nb(F.ny, 32), nslot);
-    launch_pdl(k_pre2d<T, 32, 32>, g, 256, fused_smem<T, 32, 32>(), s, view<T>(F), st, invd, taus, f, z, vs, fc, vsc);
+    launch_pdl(k_pre2d<T, 32, 32>, g, 256, fused_smem<T, 32, 32>(), s, L, st, invd, taus, f, z, vs, fc, vsc);
   }
   (void)C;
 }
@@ -1885,18 +2077,21 @@ template <typename T>
 void launch_post2d(const LevelHost& F, const LevelHost& C, uint32_t mask, const SlotState* st, const cx<T>* invd,
                    const cx<T>* f, const cx<T>* z, cx<T>* zout, int64_t vs, const cx<T>* zc, int64_t vsc, int nslot,
                    int tile, cudaStream_t s, z64* Zk, int64_t vsZk, int64_t zcol) {
+  const dim3 g(nb(F.nx, tile), nb(F.ny, tile), nslot);
+  const LevelView<T> L = view<T>(F);
   if (tile == 8) {
-    dim3 g(nb(F.nx, 8), nb(F.ny, 8), nslot);
-    launch_pdl(k_post2d<T, 8, 8>, g, 256, fused_smem<T, 8, 8>(), s, view<T>(F), mask, st, invd, f, z, zout, vs, zc, vsc, Zk,
-                                                             vsZk, zcol);
+    launch_pdl(k_post2d_pairs<T, 8>, g, TilePair<T, 8>::NT, 0, s, L, mask, st, invd, f, z, zout, vs, zc, vsc, Zk, vsZk,
+               zcol);
   } else if (tile == 16) {
-    dim3 g(nb(F.nx, 16), nb(F.ny, 16), nslot);
-    launch_pdl(k_post2d<T, 16, 16>, g, 256, fused_smem<T, 16, 16>(), s, view<T>(F), mask, st, invd, f, z, zout, vs, zc, vsc,
-                                                                 Zk, vsZk, zcol);
+    if constexpr (sizeof(T) == 4)
+      launch_pdl(k_post2d_pairs<T, 16>, g, TilePair<T, 16>::NT, 0, s, L, mask, st, invd, f, z, zout, vs, zc, vsc, Zk,
+                 vsZk, zcol);
+    else
+      launch_pdl(k_post2d<T, 16, 16>, g, 256, fused_smem<T, 16, 16>(), s, L, mask, st, invd, f, z, zout, vs, zc, vsc,
+                 Zk, vsZk, zcol);
   } else {
-    dim3 g(nb(F.nx, 32), nb(F.ny, 32), nslot);
-    launch_pdl(k_post2d<T, 32, 32>, g, 256, fused_smem<T, 32, 32>(), s, view<T>(F), mask, st, invd, f, z, zout, vs, zc, vsc,
-                                                                 Zk, vsZk, zcol);
+    launch_pdl(k_post2d<T, 32, 32>, g, 256, fused_smem<T, 32, 32>(), s, L, mask, st, invd, f, z, zout, vs, zc, vsc, Zk,
+               vsZk, zcol);
   }
   (void)C;
 }
