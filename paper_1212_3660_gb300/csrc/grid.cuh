@@ -109,6 +109,17 @@ template <typename T>
 void launch_gs(const LevelHost& L, const SlotState* st, const cx<T>* invd, const cx<T>* f, cx<T>* z, int64_t vs,
                int nslot, int color, int zero_start, cudaStream_t s, z64* Zk = nullptr, int64_t vsZk = 0,
                int64_t zcol = 0, int bf16 = 0);
+// One whole red-black sweep of a 3D level (sweep.cu), from zin to zout (another
+// buffer), `color` first; bitwise two launch_gs calls. Modes: from z = 0 (zin
+// unused); zin + P zc instead of zin (zc: the correction of the level `below`,
+// coarsened by 2 in every axis);
+// the result added to column k - 1 of Zk instead of written (as launch_gs).
+enum { SWEEP_ZERO = 1, SWEEP_PROLONG = 2, SWEEP_CORRECT = 4 };
+bool sweep3_ok(const LevelHost& L, int nslot, bool fp64);
+template <typename T>
+void launch_sweep3(const LevelHost& L, const LevelHost* below, uint32_t mask, int mode, const SlotState* st,
+                   const cx<T>* invd, const cx<T>* f, const cx<T>* zin, cx<T>* zout, int64_t vs, const cx<T>* zc,
+                   int nslot, int color, z64* Zk, int64_t vsZk, int64_t zcol, int bf16, cudaStream_t s);
 template <typename T>
 void launch_residual_restrict(const LevelHost& F, const LevelHost& C, const SlotState* st, const z64* taus,
                               const cx<T>* f, const cx<T>* z, int64_t vs, cx<T>* fc, int64_t vsc, int nslot,
