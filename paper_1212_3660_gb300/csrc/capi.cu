@@ -2804,14 +2804,16 @@ fks_status fks_sensitivity(fks_op* op, const fks_c128* phi, const fks_c128* psi,
     const size_t blk = sizeof(z64) * (size_t)n * n_f;  // one measurement's n_f phasors
     const bool all_dev = is_device_ptr(phi) && is_device_ptr(psi) && is_device_ptr(j_lnk) && is_device_ptr(j_lns);
     Arena& A = op->lane0.ws;
-    const size_t need = (all_dev ? 0 : 4 * blk) + sizeof(z64) * n_f + 8192;
+    const size_t nw = sensitivity_work(op->levels[0]);
+    const size_t need = (all_dev ? 0 : 4 * blk) + sizeof(z64) * n_f + sizeof(double) * nw + 8192;
     A.reserve(need);
     A.reset();
     z64* sg = A.take<z64>(n_f);
+    double* wk = A.take<double>(nw);
     copy_in(sg, sigma, sizeof(z64) * n_f, s);
     if (all_dev) {
       launch_sensitivity(op->levels[0], op->cond_d, (const z64*)phi, (const z64*)psi, n_m, n_f, sg, (z64*)j_lnk,
-                         (z64*)j_lns, s);
+                         (z64*)j_lns, wk, s);
       CK(cudaGetLastError());
     } else {
       // one measurement at a time through device staging buffers
@@ -2822,7 +2824,7 @@ fks_status fks_sensitivity(fks_op* op, const fks_c128* phi, const fks_c128* psi,
       copy_in(ph, phi, blk, s);
       for (int m = 0; m < n_m; ++m) {
         copy_in(ps, psi + (size_t)m * n * n_f, blk, s);
-        launch_sensitivity(op->levels[0], op->cond_d, ph, ps, 1, n_f, sg, jk, js, s);
+        launch_sensitivity(op->levels[0], op->cond_d, ph, ps, 1, n_f, sg, jk, js, wk, s);
         CK(cudaGetLastError());
         copy_out(j_lnk + (size_t)m * n * n_f, jk, blk, s);
         copy_out(j_lns + (size_t)m * n * n_f, js, blk, s);

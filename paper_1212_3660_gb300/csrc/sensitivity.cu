@@ -8,75 +8,188 @@
 //   interior face to nb:  t K_nb / (K_c + K_nb) (Psi_c - Psi_nb)(Phi_c - Phi_nb)
 //     (t = g 2 K_c K_nb / (K_c + K_nb), so dt/dlnK_c = t K_nb / (K_c + K_nb))
 //   zero-head boundary face: t Psi_c Phi_c  (t = 2 g K_c; no-flow faces carry t = 0)
-// One thread per cell and shift: Phi's neighbourhood, the faces and the
-// conductivities are loaded and folded into one complex weight per face once,
-// then the measurements are looped over. On GB300 the kernel is bound by FP64
-// arithmetic (per cell, shift and measurement: 2 subtractions and 4 fused
-// multiply-adds per face and a complex product), not by memory.
+// On GB300 this is bound by FP64 arithmetic, not by memory: per cell, shift and
+// measurement the differences of Psi, 4 fused multiply-adds per face and a
+// complex product. Three things keep the rest small:
+//   - dt/dlnK_c of every face (a division) depends neither on the shift nor on
+//     the measurement: k_sens_weights forms it once per cell;
+//   - a face's difference is formed once for its two cells (the other's is its
+//     negative, exactly): along x it comes from the neighbouring lane, along
+//     the direction in which a warp marches (y in 2D, z in 3D) from the step
+//     before, so a 2D cell takes 2 complex subtractions instead of 4;
+//   - the weights times Phi's differences are folded once per cell and shift,
+//     for up to SENS_M measurements.
+// 512^2, 200 shifts, 8 measurements: 26.1 ms with a thread per cell and shift
+// that did all of this itself.
 #include "sensitivity.cuh"
 #include "stencil.cuh"
 
 namespace fks {
 
-constexpr int SENS_THREADS = 256;
+constexpr int SENS_M = 8;       // measurements per pass (their differences below wait in shared memory)
+constexpr int SENS_WARPS = 8;
+constexpr int SENS_OUT = 31;    // cells of a row per warp; lane 0 is the cell left of them
 
-__global__ void __launch_bounds__(SENS_THREADS) k_sensitivity(LevelView<double> L, const double* __restrict__ cond,
-                                                              const z64* __restrict__ phi, const z64* __restrict__ psi,
-                                                              int n_m, int n_f, const z64* __restrict__ sigma,
-                                                              z64* __restrict__ jk, z64* __restrict__ js) {
-  const int64_t c = (int64_t)blockIdx.x * SENS_THREADS + threadIdx.x;
-  const int j = blockIdx.y;
+// dt/dlnK_c of cell c's faces: w[a n + c], a in the order x low, x high, y, z
+__global__ void k_sens_weights(LevelView<double> L, const double* __restrict__ cond, double* __restrict__ w) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= L.n) return;
   const Cell p = cell_of((int)c, L.nx, L.ny);
   const Faces<double> f = faces_at(L, p);
   const double kc = cond[c];
   const int64_t sxy = (int64_t)L.nx * L.ny;
-  // per face: neighbour offset (0: boundary face) and a_f = (dt/dlnK_c)(Phi_c - Phi_nb)
-  // (boundary face: (dt/dlnK_c) Phi_c), reused for every measurement
-  const int nfaces = L.nz > 1 ? 6 : 4;
-  int64_t off[6];
-  z64 af[6];
   const double t[6] = {f.xl, f.xh, f.yl, f.yh, f.zl, f.zh};
   const bool inner[6] = {p.i > 0, p.i < L.nx - 1, p.j > 0, p.j < L.ny - 1, p.k > 0, p.k < L.nz - 1};
   const int64_t step[6] = {-1, 1, -(int64_t)L.nx, (int64_t)L.nx, -sxy, sxy};
-  const z64* ph = phi + (int64_t)j * L.n;
-  const z64 phc = ph[c];
 #pragma unroll
   for (int a = 0; a < 6; ++a) {
-    off[a] = 0;
-    af[a] = mk(0.0, 0.0);
-    if (a >= nfaces) continue;
+    if (a >= 4 && L.nz == 1) break;
+    double v = t[a];
     if (inner[a]) {
-      off[a] = step[a];
       const double kn = cond[c + step[a]];
-      af[a] = (t[a] * (kn / (kc + kn))) * (phc - ph[c + step[a]]);
-    } else {
-      af[a] = t[a] * phc;
+      v = t[a] * (kn / (kc + kn));
     }
-  }
-  const z64 smphi = (L.mm[c] * sigma[j]) * phc;  // sigma M_cc Phi_c
-  for (int m = 0; m < n_m; ++m) {
-    const int64_t base = ((int64_t)m * n_f + j) * L.n;
-    const z64* ps = psi + base;
-    const z64 psc = ps[c];
-    z64 acc = mk(0.0, 0.0);
-#pragma unroll
-    for (int a = 0; a < 6; ++a) {
-      if (a >= nfaces) continue;
-      const z64 dpsi = off[a] ? psc - ps[c + off[a]] : psc;
-      // acc += dpsi * a_f in four fused multiply-adds
-      acc.re = fmaT(dpsi.re, af[a].re, fmaT(-dpsi.im, af[a].im, acc.re));
-      acc.im = fmaT(dpsi.re, af[a].im, fmaT(dpsi.im, af[a].re, acc.im));
-    }
-    jk[base + c] = acc;
-    js[base + c] = smphi * psc;
+    w[(int64_t)a * L.n + c] = v;
   }
 }
 
+__device__ __forceinline__ z64 shfl_dn(z64 v) {
+  return mk(__shfl_down_sync(0xffffffffu, v.re, 1), __shfl_down_sync(0xffffffffu, v.im, 1));
+}
+__device__ __forceinline__ z64 shfl_up(z64 v) {
+  return mk(__shfl_up_sync(0xffffffffu, v.re, 1), __shfl_up_sync(0xffffffffu, v.im, 1));
+}
+// sign change with integer instructions (a negation that is not an operand of a
+// multiply-add takes an issue slot of the FP64 pipe)
+__device__ __forceinline__ double neg(double v) {
+  return __hiloint2double(__double2hiint(v) ^ 0x80000000, __double2loint(v));
+}
+__device__ __forceinline__ z64 neg(z64 v) { return mk(neg(v.re), neg(v.im)); }
+// acc + d a in four fused multiply-adds
+__device__ __forceinline__ z64 cfma(z64 d, z64 a, z64 acc) {
+  acc.re = fmaT(d.re, a.re, fmaT(-d.im, a.im, acc.re));
+  acc.im = fmaT(d.re, a.im, fmaT(d.im, a.re, acc.im));
+  return acc;
+}
+
+// A warp owns 31 cells of a row and marches over `len` rows (2D) or planes (3D).
+template <bool D3>
+__global__ void __launch_bounds__(SENS_WARPS * 32, 2)
+    k_sensitivity(LevelView<double> L, const double* __restrict__ wt, const z64* __restrict__ phi,
+                  const z64* __restrict__ psi, int n_m, int n_f, const z64* __restrict__ sigma, z64* __restrict__ jk,
+                  z64* __restrict__ js, int len, int ntx, int ncol) {
+  __shared__ z64 below[SENS_M][SENS_WARPS * 32];  // psi(c) - psi(c + step) of the march step before
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = threadIdx.x, j = blockIdx.y;
+  const int nx = L.nx, ny = L.ny, sxy = nx * ny;
+  const int bx = blockIdx.x % ntx, rest = blockIdx.x / ntx;
+  const int i = bx * SENS_OUT + lane - 1;
+  const int row = D3 ? (rest % ncol) * SENS_WARPS + w : 0;           // the y row of a 3D march
+  const int m0 = (D3 ? rest / ncol : rest * SENS_WARPS + w) * len, nm = D3 ? L.nz : ny;
+  const int m1 = (!D3 || row < ny) ? min(m0 + len, nm) : m0;
+  if (m0 >= m1) return;  // whole warps: the shuffles below are among a warp's lanes
+  const bool in = i >= 0 && i < nx, out = in && lane > 0, xlo = i > 0, xhi = i < nx - 1;
+  const bool ylo = row > 0, yhi = row < ny - 1;
+  const int step = D3 ? sxy : nx;
+  const int64_t n = L.n;
+  const z64* ph = phi + (int64_t)j * n;
+  const z64 none = mk(0.0, 0.0), sg = sigma[j];
+  // v(c) - v(c + 1), for the lane's cell and, from the lane below, its left face
+  auto xdiff = [&](const z64* v, int c, z64 here, z64* lo, z64* hi) {
+    z64 right = shfl_dn(here);
+    if (lane == 31 && in && xhi) right = v[c + 1];
+    *hi = here - right;
+    *lo = neg(shfl_up(*hi));
+  };
+  for (int mc = 0; mc < n_m; mc += SENS_M) {
+    const int nmc = min(SENS_M, n_m - mc);
+    int c = m0 * step + row * nx + i;
+    z64 ph_c = in ? ph[c] : none;
+    z64 ph_lo = none;  // phi(c - step) - phi(c)
+    if (m0 > 0 && in) {
+      ph_lo = ph[c - step] - ph_c;
+      for (int q = 0; q < nmc; ++q) {
+        const z64* ps = psi + ((int64_t)(mc + q) * n_f + j) * n;
+        below[q][t] = ps[c - step] - ps[c];
+      }
+    }
+    for (int m = m0; m < m1; ++m, c += step) {
+      const bool mlo = m > 0, mhi = m + 1 < nm;
+      const z64 ph_n = in && mhi ? ph[c + step] : none;
+      z64 dl, dh;
+      xdiff(ph, c, ph_c, &dl, &dh);
+      const z64 dm = ph_c - ph_n;
+      z64 a[6];
+      z64 smphi = none;
+      if (out) {
+        a[0] = wt[c] * (xlo ? dl : ph_c);
+        a[1] = wt[n + c] * (xhi ? dh : ph_c);
+        if constexpr (D3) {
+          a[2] = wt[2 * n + c] * (ylo ? ph_c - ph[c - nx] : ph_c);
+          a[3] = wt[3 * n + c] * (yhi ? ph_c - ph[c + nx] : ph_c);
+          a[4] = wt[4 * n + c] * (mlo ? neg(ph_lo) : ph_c);
+          a[5] = wt[5 * n + c] * (mhi ? dm : ph_c);
+        } else {
+          a[2] = wt[2 * n + c] * (mlo ? neg(ph_lo) : ph_c);
+          a[3] = wt[3 * n + c] * (mhi ? dm : ph_c);
+        }
+        smphi = (L.mm[c] * sg) * ph_c;  // sigma M_cc Phi_c
+      }
+      ph_lo = dm;
+      ph_c = ph_n;
+      // a measurement's two loads are issued while the one before is summed
+      const z64* ps = psi + ((int64_t)mc * n_f + j) * n;
+      z64 pc = in ? ps[c] : none, pn = in && mhi ? ps[c + step] : none;
+      for (int q = 0; q < nmc; ++q) {
+        const int64_t base = ps - psi;
+        const z64* next = ps + (int64_t)n_f * n;
+        z64 nc = none, nn = none;
+        if (q + 1 < nmc) {
+          nc = in ? next[c] : none;
+          nn = in && mhi ? next[c + step] : none;
+        }
+        z64 xl, xh;
+        xdiff(ps, c, pc, &xl, &xh);
+        const z64 d = pc - pn, lo = below[q][t];
+        below[q][t] = d;
+        if (out) {
+          z64 acc = cfma(xlo ? xl : pc, a[0], none);
+          acc = cfma(xhi ? xh : pc, a[1], acc);
+          if constexpr (D3) {
+            acc = cfma(ylo ? pc - ps[c - nx] : pc, a[2], acc);
+            acc = cfma(yhi ? pc - ps[c + nx] : pc, a[3], acc);
+            acc = cfma(mlo ? neg(lo) : pc, a[4], acc);
+            acc = cfma(mhi ? d : pc, a[5], acc);
+          } else {
+            acc = cfma(mlo ? neg(lo) : pc, a[2], acc);
+            acc = cfma(mhi ? d : pc, a[3], acc);
+          }
+          jk[base + c] = acc;
+          js[base + c] = smphi * pc;
+        }
+        ps = next;
+        pc = nc;
+        pn = nn;
+      }
+    }
+  }
+}
+
+size_t sensitivity_work(const LevelHost& L0) { return (size_t)(L0.nz > 1 ? 6 : 4) * L0.n; }
+
 void launch_sensitivity(const LevelHost& L0, const double* cond, const z64* phi, const z64* psi, int n_m, int n_f,
-                        const z64* sigma, z64* jk, z64* js, cudaStream_t s) {
-  const dim3 g((unsigned)((L0.n + SENS_THREADS - 1) / SENS_THREADS), (unsigned)n_f);
-  k_sensitivity<<<g, SENS_THREADS, 0, s>>>(view<double>(L0), cond, phi, psi, n_m, n_f, sigma, jk, js);
+                        const z64* sigma, z64* jk, z64* js, double* work, cudaStream_t s) {
+  const LevelView<double> L = view<double>(L0);
+  auto up = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+  k_sens_weights<<<(unsigned)up(L0.n, 256), 256, 0, s>>>(L, cond, work);
+  // march length: 16 while that leaves eight blocks per SM
+  const int64_t ntx = up(L0.nx, SENS_OUT), nm = L0.nz > 1 ? L0.nz : L0.ny;
+  const int64_t ncol = L0.nz > 1 ? up(L0.ny, SENS_WARPS) : 1;
+  auto blocks = [&](int len) { return ntx * ncol * up(nm, (int64_t)len * (L0.nz > 1 ? 1 : SENS_WARPS)); };
+  int len = 16;
+  while (len > 1 && blocks(len) * n_f < 8 * 152) len /= 2;
+  const dim3 g((unsigned)blocks(len), (unsigned)n_f);
+  auto kernel = L0.nz > 1 ? k_sensitivity<true> : k_sensitivity<false>;
+  kernel<<<g, SENS_WARPS * 32, 0, s>>>(L, work, phi, psi, n_m, n_f, sigma, jk, js, len, (int)ntx, (int)ncol);
 }
 
 }  // namespace fks
