@@ -268,15 +268,24 @@ struct fks_op {
   std::vector<LevelHost> levels;
   std::vector<LevelHost> levels_bf;  // the same levels with fp32 coefficients replaced by their bf16 roundings
   Lane lane0;  // workspace, graph and instrumentation of fks_solve / fks_precond_apply
-  // 2D levels with at most this many cells use the fused tile kernels
-  // ([0] complex128 cycles, [1] complex64 cycles); set by fks_op_autotune
-  int64_t fuse_max[2] = {65536, INT64_MAX};
-  // fused 2D levels with at most this many cells use 16 x 16 tiles (else 32 x 32)
-  int64_t tile16_max[2] = {16384, 16384};
-  // ... and with at most this many, 8 x 8 tiles (more CTAs on small levels)
-  int64_t tile8_max[2] = {0, 0};
+  // Thresholds of a 2D operator before any tuning ([0] complex128 cycles, [1]
+  // complex64 cycles; fks_op_grid sets a 3D operator's, fks_op_autotune and
+  // the fks_op_set_* calls change them), in cells of a launch (a level's times
+  // the batch's sources). Fused tile kernels: in complex128 their recomputed
+  // halo costs FP64 time once a level fills the chip (1000^2 369 us a cycle per
+  // sweep, 417 fused; 512^2 fused), in complex64 they win throughout (2048^2
+  // 426 against 497 us).
+  int64_t fuse_max[2] = {524288, INT64_MAX};
+  // fused 2D levels with at most this many cells use 16 x 16 tiles (else 32 x
+  // 32: 2048^2 complex64 426 against 441 us a cycle, 1024^2 159 against 153)
+  int64_t tile16_max[2] = {524288, 2097152};
+  // ... and with at most this many, 8 x 8 tiles (289 x 311 complex64 62 against
+  // 66 us; complex128 256^2 18 + 16 against 12 + 10 us, 128^2 7 + 6 against 8 + 7)
+  int64_t tile8_max[2] = {16384, 131072};
   // levels with at most this many cells run in the single-block tail kernel
-  int64_t tail_max[2] = {256, 256};
+  // (64^2 complex128 65 us a cycle with 64, 70 with 256; 289 x 311 complex64
+  // 81 with 256, 66 with 1024)
+  int64_t tail_max[2] = {64, 2048};
   // from the first level with at most this many cells (and a cluster layout)
   // down, the V-cycle runs in the cluster kernel instead of the tail (0: off)
   int64_t cluster_max[2] = {0, 0};
@@ -598,18 +607,20 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   const int64_t fmax = S.op->fuse_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t16 = S.op->tile16_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t8 = S.op->tile8_max[sizeof(VT) == 8 ? 0 : 1];
-  auto tile_of = [&](const LevelHost& L) { return L.n <= t8 ? 8 : (L.n <= t16 ? 16 : 32); };
+  // the batch's sources share a launch: small tiles pay while it leaves SMs idle
+  const int64_t nsl = S.nslot;
+  auto tile_of = [&](const LevelHost& L) { return L.n * nsl <= t8 ? 8 : (L.n * nsl <= t16 ? 16 : 32); };
   const int pix = sizeof(VT) == 8 ? 0 : 1;
   for (int l = 0; l < lp; ++l) {
     const LevelHost& L = Ls[l];
-    if (fused_level_ok(L) && L.n <= fmax) {
+    if (fused_level_ok(L) && L.n * nsl <= fmax) {
       PROF(FKS_K_PRE2D, l, ns * (L.n * (3 * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
            ns * L.n * (2 * (8 * d + 6) + 8 * d + 10),
            launch_pre2d<VT>(L, Ls[l + 1], S.st, I(l), S.taus, F(l), Zl(l), L.n, F(l + 1), Ls[l + 1].n, S.nslot,
                             tile_of(L), s));
       continue;
     }
-    if (fused3d_level_ok(L) && L.n <= fmax) {
+    if (fused3d_level_ok(L) && L.n * nsl <= fmax) {
       PROF(FKS_K_PRE3D, l, ns * (L.n * (3 * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
            ns * L.n * (2 * (8 * d + 6) + 8 * d + 10),
            launch_pre3d<VT>(L, S.st, I(l), S.taus, F(l), Zl(l), L.n, F(l + 1), Ls[l + 1].n, S.nslot, tile_of(L),
@@ -734,7 +745,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   cx<VT>* zfin = Zl(lp);  // final correction of the level below
   for (int l = lp - 1; l >= 0; --l) {
     const LevelHost& L = Ls[l];
-    if (fused_level_ok(L) && L.n <= fmax) {
+    if (fused_level_ok(L) && L.n * nsl <= fmax) {
       cx<VT>* out = (cx<VT>*)S.z2[l];
       const bool add_to_zk = l == 0 && Zk;
       PROF(FKS_K_POST2D, l, ns * (L.n * (4 * cv + d * rv) + cv * Ls[l + 1].n),
@@ -744,7 +755,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
       zfin = add_to_zk ? nullptr : out;
       continue;
     }
-    if (fused3d_level_ok(L) && L.n <= fmax) {
+    if (fused3d_level_ok(L) && L.n * nsl <= fmax) {
       cx<VT>* out = (cx<VT>*)S.z2[l];
       const bool add_to_zk = l == 0 && Zk;
       PROF(FKS_K_POST3D, l, ns * (L.n * (4 * cv + d * rv) + cv * Ls[l + 1].n),
@@ -1946,6 +1957,13 @@ fks_status fks_op_grid(fks_ctx* ctx, int dim, const int64_t ncell[3], const doub
     CK(cudaMalloc(&cond_d, sizeof(double) * n));
     CK(cudaMemcpy(cond_d, cond, sizeof(double) * n, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(op->levels[0].d64[3], mass.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
+    if (nz > 1) {
+      // 3D: level kernels per half sweep or sweep instead of the z-march ones
+      // (128^3 complex64: 134 us against 305 on the finest level), a tail of up
+      // to 8^3 cells in complex128 (64^3: 230 us a cycle, 245 with 64)
+      op->fuse_max[0] = op->fuse_max[1] = 0;
+      op->tail_max[0] = 512;
+    }
     launch_faces_from_cond(op->levels[0], hh, mask, cond_d, s);
     {
       // coarse-face factors of every coarsening from the cells' widths (in
