@@ -353,8 +353,7 @@ __global__ void k_amg_smooth(const AmgLevel<T>* tab, int L, int l, const SlotSta
   if (!amg_live(st, sc, slot)) return;
   const AmgLevel<T>& A = amg_level(tab, st, slot, L, l);
   const int64_t o = slot * n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    xo[o + i] = amg_sweep(A, i, f + o, xi + o);
+  amg_sweep_rows(A, n, f + o, xi + o, xo + o);
 }
 
 // r = f - A x
@@ -365,8 +364,7 @@ __global__ void k_amg_resid(const AmgLevel<T>* tab, int L, int l, const SlotStat
   if (!amg_live(st, sc, slot)) return;
   const AmgLevel<T>& A = amg_level(tab, st, slot, L, l);
   const int64_t o = slot * n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    r[o + i] = amg_resid(A, i, f + o, x + o);
+  amg_resid_rows(A, n, f + o, x + o, r + o);
 }
 
 // fc = P^T r on level l + 1, and there (unless it is the coarsest) the first
@@ -378,11 +376,7 @@ __global__ void k_amg_restrict(const AmgLevel<T>* tab, int L, int l, const SlotS
   if (!amg_live(st, sc, slot)) return;
   const AmgLevel<T>& A = amg_level(tab, st, slot, L, l);
   const AmgLevel<T>& C = amg_level(tab, st, slot, L, l + 1);
-  for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < nc; a += (int64_t)gridDim.x * blockDim.x) {
-    const cx<T> v = amg_row(A.rrp, A.rci, A.rv, a, r + slot * n);
-    fc[slot * nc + a] = v;
-    if (l + 2 < L) xc[slot * nc + a] = amg_first(C, a, v);
-  }
+  amg_restrict_rows(A, C, nc, r + slot * n, fc + slot * nc, xc + slot * nc, l + 2 < L);
 }
 
 // x += P e (e: the next level's result)
@@ -393,8 +387,7 @@ __global__ void k_amg_prolong(const AmgLevel<T>* tab, int L, int l, const SlotSt
   if (!amg_live(st, sc, slot)) return;
   const AmgLevel<T>& A = amg_level(tab, st, slot, L, l);
   const int64_t o = slot * n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    x[o + i] = amg_ld(x + o + i) + amg_row(A.prp, A.pci, A.pv, i, e + slot * nc);
+  amg_prolong_rows(A, n, x + o, e + slot * nc);
 }
 
 // out = Cinv f on the coarsest level, one warp per row
@@ -406,13 +399,18 @@ __global__ void k_amg_coarse(const AmgLevel<T>* tab, int L, const SlotState* st,
   const AmgLevel<T>& A = amg_level(tab, st, slot, L, L - 1);
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); row < n; row += warps) {
+  for (int64_t row = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; row < n; row += warps) {
     const cx<T> v = amg_coarse_row(A, row, f + slot * n, lane);
     if (lane == 0) out[slot * n + row] = v;
   }
 }
 
-inline unsigned amg_blocks(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 1024); }
+// one warp's rows per block until the grid has 1024 blocks
+template <typename T>
+inline unsigned amg_blocks(int64_t n) {
+  const int rw = 32 / AmgLane<T>::LPR;
+  return (unsigned)std::min<int64_t>((n + rw - 1) / rw, 1024);
+}
 
 }  // namespace
 
@@ -425,7 +423,7 @@ int launch_amg_vcycle(const AmgRun<T>& R, const SlotState* st, const BcgScal* sc
   cx<T>* oth[AMG_MAX_LEVELS];
   for (int l = 0; l + 1 < L; ++l) {
     const int64_t n = R.n[l];
-    const dim3 g(amg_blocks(n), nslot);
+    const dim3 g(amg_blocks<T>(n), nslot);
     const cx<T>* f = l == 0 ? f0 : R.f[l];
     cur[l] = R.x[l];   // holds the first sweep (written with f)
     oth[l] = R.y[l];
@@ -435,7 +433,7 @@ int launch_amg_vcycle(const AmgRun<T>& R, const SlotState* st, const BcgScal* sc
       ++cnt;
     }
     k_amg_resid<T><<<g, 256, 0, s>>>(R.tab, L, l, st, sc, f, cur[l], R.r[l], n);
-    k_amg_restrict<T><<<dim3(amg_blocks(R.n[l + 1]), nslot), 256, 0, s>>>(R.tab, L, l, st, sc, R.r[l], R.f[l + 1],
+    k_amg_restrict<T><<<dim3(amg_blocks<T>(R.n[l + 1]), nslot), 256, 0, s>>>(R.tab, L, l, st, sc, R.r[l], R.f[l + 1],
                                                                           R.x[l + 1], n, R.n[l + 1]);
     cnt += 2;
   }
@@ -448,7 +446,7 @@ int launch_amg_vcycle(const AmgRun<T>& R, const SlotState* st, const BcgScal* sc
   }
   for (int l = L - 2; l >= 0; --l) {
     const int64_t n = R.n[l];
-    const dim3 g(amg_blocks(n), nslot);
+    const dim3 g(amg_blocks<T>(n), nslot);
     const cx<T>* f = l == 0 ? f0 : R.f[l];
     cx<T>* out = l == 0 ? out0 : R.r[l];
     k_amg_prolong<T><<<g, 256, 0, s>>>(R.tab, L, l, st, sc, cur[l], R.r[l + 1], n, R.n[l + 1]);
