@@ -1112,12 +1112,17 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
     const TailLevel<T>& Cl = P.lev[P.nlev - 1];
     const cx<T>* F = sh + Cl.off;
     cx<T>* Z = sh + Cl.off + Cl.L.n;
-    const cx<T>* Ainv = (const cx<T>*)(t2_smem + P.ainv_off);
-    for (int r = tid; r < P.nc; r += nt) {
-      cx<T> acc = mk(T(0), T(0));
+    // the products by all threads, in place of the staged inverse; then two
+    // threads per row, one for each part, add them in order
+    cx<T>* as = (cx<T>*)(t2_smem + P.ainv_off);
+    const int nc = P.nc;
+    for (int e = tid; e < nc * nc; e += nt) as[e] = as[e] * F[e / nc];
+    __syncthreads();
+    for (int e = tid; e < 2 * nc; e += nt) {
+      T acc = T(0);
 #pragma unroll 4
-      for (int l = 0; l < P.nc; ++l) acc = acc + Ainv[l * P.nc + r] * F[l];
-      Z[r] = acc;
+      for (int l = 0; l < nc; ++l) acc = acc + ((const T*)as)[2 * l * nc + e];
+      ((T*)Z)[e] = acc;
     }
     __syncthreads();
   }
@@ -1318,22 +1323,29 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
     const cx<T>* Ainv = P.Ainv + (int64_t)tau * P.nc * P.nc;
     const int nc = P.nc, cols = min(nc, P.rlen / nc);
     if (P.nlev == 1) __syncthreads();
-    cx<T> acc = none;  // nc <= NT
+    // the terms by all threads; then two threads per row, one for each part of
+    // the complex sum, add them in order (2 nc <= 2 NT: the second pass of a
+    // thread is row t / 2 + NT / 2)
+    T acc[2] = {T(0), T(0)};
     for (int l0 = 0; l0 < nc; l0 += cols) {
       const int lc = min(cols, nc - l0);
 #pragma unroll 4
       for (int e = t; e < lc * nc; e += NT) R[e] = Ainv[l0 * nc + e] * F[l0 + e / nc];
       __syncthreads();
-      if (t < nc) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (t + h * NT < 2 * nc) {
 #pragma unroll 8
-        for (int l = 0; l < lc; ++l) acc = acc + R[l * nc + t];
-      }
+          for (int l = 0; l < lc; ++l) acc[h] = acc[h] + ((const T*)R)[2 * l * nc + t + h * NT];
+        }
       __syncthreads();
     }
-    if (t < nc) {
-      Z[t] = acc;
-      if (P.nlev == 1) P.z_out[slot * P.vs + t] = acc;
-    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (t + h * NT < 2 * nc) {
+        ((T*)Z)[t + h * NT] = acc[h];
+        if (P.nlev == 1) ((T*)(P.z_out + slot * P.vs))[t + h * NT] = acc[h];
+      }
     __syncthreads();
   }
   for (int l = P.nlev - 2; l >= 0; --l) {
@@ -1617,12 +1629,13 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const cx<T>* __restrict__ 
     pr[e] = r < n ? a[(int64_t)l * n + r] * fs[l] : mk(T(0), T(0));
   }
   __syncthreads();
+  // two threads per row, one for each part of the complex sum
   const int t = threadIdx.x;
-  if (t >= RB || r0 + t >= n) return;
-  cx<T> acc = mk(T(0), T(0));
+  if (t >= 2 * RB || r0 + t / 2 >= n) return;
+  T acc = T(0);
 #pragma unroll 16
-  for (int l = 0; l < n; ++l) acc = acc + pr[l * RB + t];
-  z[slot * vs + r0 + t] = acc;
+  for (int l = 0; l < n; ++l) acc = acc + ((const T*)pr)[2 * l * RB + t];
+  ((T*)(z + slot * vs + r0))[t] = acc;
 }
 
 // --------------------------------------------------------------------- defect correction
@@ -1823,10 +1836,13 @@ __global__ void __launch_bounds__(GX * GY)
   __syncthreads();
   if (lane == 0) { red[0][w] = a; red[1][w] = b; }
   __syncthreads();
+  if (w != 0) return;
+  a = lane < NW ? red[0][lane] : 0.0;
+  b = lane < NW ? red[1][lane] : 0.0;
+  for (int o = NW / 2; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+  if (with_v)
+    for (int o = NW / 2; o > 0; o >>= 1) b += __shfl_down_sync(0xffffffffu, b, o);
   if (tl == 0) {
-    a = 0.0;
-    b = 0.0;
-    for (int q = 0; q < NW; ++q) { a += red[0][q]; b += red[1][q]; }
     D.bcount[slot] = 0;
     int running = decide_slot(st[slot], slot, a, b, zero_z, D.eps, D.max_cycles, D.replay_cycles, D.m_max, D.relax,
                               D.tol);

@@ -360,15 +360,33 @@ __global__ void __launch_bounds__(GV_WARPS * 32) k_givens(SlotState* st, int nf,
   }
   __syncwarp();
   z64* Rc = Rj + (int64_t)(k - 1) * m;
-  if (lane == 0) {
-    cl[k - 1] = cl[k - 1] + mk(1.0, 0.0);
+  // The rotations, a chain over i: new cl[i] = c a + s b and cl[i + 1] = c b -
+  // conj(s) a. Lanes 0..3 each form one of the four real results (4 FP64
+  // instructions of the 16; one lane alone paid 64 clocks for each) and hand
+  // the last two on: what changes from row to row is a = the new cl[i + 1].
+  if (lane < 4) {
+    const int im = lane & 1, lo = lane >> 1;  // part; 0: cl[i], 1: cl[i + 1]
+    const z64 c0 = cl[0];
+    double ax = k == 1 ? c0.re + 1.0 : c0.re, ay = c0.im;  // a of the next rotation
     for (int i = 0; i + 1 < k; ++i) {
-      z64 a = cl[i], b = cl[i + 1];
-      double c = rcs[warp][i];
-      z64 sn = rss[warp][i];
-      cl[i] = c * a + sn * b;
-      cl[i + 1] = c * b - conj(sn) * a;
+      z64 b = cl[i + 1];
+      if (i + 2 == k) b.re = b.re + 1.0;  // the identity's entry in row k - 1
+      const double c = rcs[warp][i];
+      const z64 sn = rss[warp][i];
+      // s b (lo = 0) or conj(s) a (lo = 1), part im
+      const double vr = lo ? ax : b.re, vi = lo ? ay : b.im;
+      const double si = __hiloint2double(__double2hiint(sn.im) ^ (lo ? 0x80000000 : 0), __double2loint(sn.im));
+      const double p = im ? fmaT(sn.re, vi, mulT(si, vr)) : fmaT(sn.re, vr, -mulT(si, vi));
+      const double u = mulT(c, lo ? (im ? b.im : b.re) : (im ? ay : ax));
+      const double r = lo ? u - p : u + p;
+      if (!lo) ((double*)&cl[i])[im] = r;
+      ax = __shfl_sync(0xfu, r, 2);
+      ay = __shfl_sync(0xfu, r, 3);
     }
+    if (lane == 0) cl[k - 1] = mk(ax, ay);
+  }
+  __syncwarp();
+  if (lane == 0) {
     z64 a = cl[k - 1], b = cl[k];
     double aa = cabs(a), bb = cabs(b);
     double c;
