@@ -1324,8 +1324,7 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
     const int nc = P.nc, cols = min(nc, P.rlen / nc);
     if (P.nlev == 1) __syncthreads();
     // the terms by all threads; then two threads per row, one for each part of
-    // the complex sum, add them in order (2 nc <= 2 NT: the second pass of a
-    // thread is row t / 2 + NT / 2)
+    // the complex sum, add them in order (nc <= NT)
     T acc[2] = {T(0), T(0)};
     for (int l0 = 0; l0 < nc; l0 += cols) {
       const int lc = min(cols, nc - l0);
@@ -1436,14 +1435,13 @@ __device__ __forceinline__ void gj_warp_best(unsigned long long* v, int* i) {
 // One elimination step over the whole chip. One block per tau, as this was
 // before, is bound by one SM's FP64 rate (2 fused multiply-adds a clock) and
 // by its reads of the matrix: 265 ms for four 625 x 625 matrices. Here a block
-// updates a 32 x 32 tile, read from S and written to D (the two buffers
+// updates a 32 x 8 tile, read from S and written to D (the two buffers
 // alternate, so a step needs no barrier inside the grid). Every block finds
 // the pivot itself from the step's column, which the step before left
 // contiguous in `cin`. The matrix is banded (5 or 7 diagonals): rows whose
 // entry in the column is zero and tiles whose pivot row is zero are copied.
-// GJ_R rows per warp: one while that still fits the chip a few times over.
+// A tile is 32 columns by 8 rows, one row per warp.
 constexpr int GJ_T = 32;
-template <int GJ_R>
 __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64* __restrict__ D,
                                                  const z64* __restrict__ cin, z64* __restrict__ cout,
                                                  int32_t* __restrict__ piv, int n, int col, int* singular) {
@@ -1455,18 +1453,13 @@ __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64*
   __shared__ unsigned long long sv[8];
   __shared__ int si[8];
   __shared__ z64 srd;
-  const int l = blockIdx.x * GJ_T + lane, r0 = blockIdx.y * 8 * GJ_R;
+  const int l = blockIdx.x * GJ_T + lane, r = blockIdx.y * 8 + w;
   // the tile's rows, before the swap (their latency overlaps the search)
-  z64 v[GJ_R], f[GJ_R];
-#pragma unroll
-  for (int h = 0; h < GJ_R; ++h) {
-    const int r = r0 + w + 8 * h;
-    v[h] = l < n && r < n ? a[(int64_t)r * n + l] : mk(0.0, 0.0);
-    f[h] = r < n ? cc[r] : mk(0.0, 0.0);
-  }
+  const z64 v = l < n && r < n ? a[(int64_t)r * n + l] : mk(0.0, 0.0);
+  const z64 f = r < n ? cc[r] : mk(0.0, 0.0);
   unsigned long long bv = 0ull;
   int bi = INT_MAX;
-  for (int r = col + t; r < n; r += 256) gj_better(gj_key(cc[r]), r, &bv, &bi);
+  for (int e = col + t; e < n; e += 256) gj_better(gj_key(cc[e]), e, &bv, &bi);
   gj_warp_best(&bv, &bi);
   if (lane == 0) {
     sv[w] = bv;
@@ -1488,19 +1481,106 @@ __global__ void __launch_bounds__(256) k_gj_step(const z64* __restrict__ S, z64*
   const z64 rd = srd;
   const bool any = __any_sync(0xffffffffu, l == col || p.re != 0.0 || p.im != 0.0);
   if (any && l < n) p = l == col ? rd : rd * p;
+  if (l >= n || r >= n) return;
+  z64 x = v, fr = f;
+  if (r == pr && pr != col) {
+    x = a[(int64_t)col * n + l];
+    fr = cc[col];
+  }
+  if (l == col) x = mk(0.0, 0.0);
+  if (r == col) x = p;
+  else if (any && (fr.re != 0.0 || fr.im != 0.0)) x = x - fr * p;
+  o[(int64_t)r * n + l] = x;
+  if (l == col + 1) cout[(int64_t)q * n + r] = x;
+}
+
+// The same step for matrices of many tiles, in place and in two launches: one
+// block per tau finds the pivot, scales its row into `row` and exchanges the
+// rows; then the tiles update the rows whose entry in the column is not zero
+// and leave the others alone (k_gj_step copies them, and its blocks, several
+// rounds of them, each wait for the pivot search and the division: 22 us a
+// step of four 729 x 729 matrices).
+__global__ void __launch_bounds__(1024) k_gj_pivot(z64* __restrict__ A, z64* __restrict__ row, z64* __restrict__ cin,
+                                                   int32_t* __restrict__ piv, int n, int col, int* singular) {
+  pdl_enter();
+  const int q = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+  z64* a = A + (int64_t)q * n * n;
+  z64* cc = cin + (int64_t)q * n;
+  __shared__ unsigned long long sv[32];
+  __shared__ int si[32];
+  __shared__ int spr;
+  __shared__ z64 srd;
+  unsigned long long bv = 0ull;
+  int bi = INT_MAX;
+  z64 oc = mk(0.0, 0.0);  // the row at position col before the exchange
+  if (t < n) {
+    oc = a[(int64_t)col * n + t];
+    if (t >= col) gj_better(gj_key(cc[t]), t, &bv, &bi);
+  }
+  gj_warp_best(&bv, &bi);
+  if (lane == 0) {
+    sv[w] = bv;
+    si[w] = bi;
+  }
+  __syncthreads();
+  if (w == 0) {
+    bv = lane < (int)(blockDim.x >> 5) ? sv[lane] : 0ull;
+    bi = lane < (int)(blockDim.x >> 5) ? si[lane] : INT_MAX;
+    gj_warp_best(&bv, &bi);
+    gj_recip(cc[bi], lane, &srd);
+    __syncwarp();
+    if (lane == 0) {
+      spr = bi;
+      piv[(int64_t)q * n + col] = bi;
+      if (bv == 0ull) *singular = 1;
+      if (bi != col) cc[bi] = cc[col];  // the exchanged row's factor
+    }
+  }
+  __syncthreads();
+  if (t >= n) return;
+  const int pr = spr;
+  const z64 x = pr == col ? oc : a[(int64_t)pr * n + t];
+  const z64 p = t == col ? srd : ((x.re != 0.0 || x.im != 0.0) ? srd * x : x);
+  if (pr != col) a[(int64_t)pr * n + t] = oc;
+  a[(int64_t)col * n + t] = p;
+  row[(int64_t)q * n + t] = p;
+}
+
+__global__ void __launch_bounds__(256) k_gj_update(z64* __restrict__ A, const z64* __restrict__ row,
+                                                   const z64* __restrict__ cin, z64* __restrict__ cout, int n,
+                                                   int col) {
+  pdl_enter();
+  const int q = blockIdx.z, lane = threadIdx.x, w = threadIdx.y;
+  z64* a = A + (int64_t)q * n * n;
+  const z64* cc = cin + (int64_t)q * n;
+  const int l = blockIdx.x * GJ_T + lane, r0 = blockIdx.y * GJ_T;
+  const bool next = (int)blockIdx.x == (col + 1) / GJ_T;  // the tile column that holds the next step's column
+  const z64 p = l < n ? row[(int64_t)q * n + l] : mk(0.0, 0.0);
+  const bool any = __any_sync(0xffffffffu, p.re != 0.0 || p.im != 0.0);
+  if (!any && !next) return;
+  z64 f[GJ_T / 8], v[GJ_T / 8];
+  bool on[GJ_T / 8];
 #pragma unroll
-  for (int h = 0; h < GJ_R; ++h) {
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int r = r0 + w + 8 * h;
+    f[h] = r < n && r != col ? cc[r] : mk(0.0, 0.0);
+  }
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
+    const int r = r0 + w + 8 * h;
+    on[h] = any && (f[h].re != 0.0 || f[h].im != 0.0);
+    v[h] = l < n && r < n && (on[h] || next) ? a[(int64_t)r * n + l] : mk(0.0, 0.0);
+  }
+#pragma unroll
+  for (int h = 0; h < GJ_T / 8; ++h) {
     const int r = r0 + w + 8 * h;
     if (l >= n || r >= n) continue;
-    z64 x = v[h], fr = f[h];
-    if (r == pr && pr != col) {
-      x = a[(int64_t)col * n + l];
-      fr = cc[col];
+    z64 x = v[h];
+    if (on[h]) {
+      if (l == col) x = mk(0.0, 0.0);
+      x = x - f[h] * p;
+      a[(int64_t)r * n + l] = x;
     }
-    if (l == col) x = mk(0.0, 0.0);
-    if (r == col) x = p;
-    else if (any && (fr.re != 0.0 || fr.im != 0.0)) x = x - fr * p;
-    o[(int64_t)r * n + l] = x;
     if (l == col + 1) cout[(int64_t)q * n + r] = x;
   }
 }
@@ -1947,11 +2027,13 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
   const int n = (int)L.n;
   const int64_t nn = (int64_t)n * n;
   const bool small = n <= GJ_SMALL;
-  // the steps' column buffers and pivots live in inv's memory until the finish
-  // overwrites it (48 n bytes or fewer of its n^2 sizeof(cx<T>) per tau); the
-  // pivots move to the dead matrix buffer first
-  z64* cb[2] = {(z64*)inv, (z64*)inv + (int64_t)ntau * n};
-  int32_t* piv = (int32_t*)(cb[1] + (int64_t)ntau * n);
+  // the steps' column buffers, pivot row and pivots live in inv's memory until
+  // the finish overwrites it (52 n bytes of its n^2 sizeof(cx<T>) per tau); the
+  // pivots move to the other matrix buffer first
+  const int64_t tn = (int64_t)ntau * n;
+  z64* cb[2] = {(z64*)inv, (z64*)inv + tn};
+  z64* prow = cb[1] + tn;
+  int32_t* piv = (int32_t*)(prow + tn);
   cudaMemsetAsync(work, 0, sizeof(z64) * nn * ntau, s);
   z64* c0 = small ? nullptr : cb[0];
   const dim3 gd(nb(n, 128), ntau);
@@ -1963,13 +2045,17 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
   }
   z64 *src = work, *dst = work2;
   const unsigned nt = nb(n, GJ_T);
-  // one row per warp up to about eight blocks per SM (312 unknowns at four taus)
-  const bool one = (int64_t)nt * nb(n, 8) * ntau <= 8 * 152 + 400;
+  // one launch per step up to about ten blocks per SM (360 unknowns at four taus)
+  const bool one = (int64_t)nt * nb(n, 8) * ntau <= 2048;
   for (int col = 0; col < n; ++col) {
     z64 *ci = cb[col & 1], *co = cb[(col + 1) & 1];
-    if (one) launch_pdl(k_gj_step<1>, dim3(nt, nb(n, 8), ntau), dim3(32, 8), 0, s, src, dst, ci, co, piv, n, col, singular);
-    else launch_pdl(k_gj_step<4>, dim3(nt, nt, ntau), dim3(32, 8), 0, s, src, dst, ci, co, piv, n, col, singular);
-    std::swap(src, dst);
+    if (one) {
+      launch_pdl(k_gj_step, dim3(nt, nb(n, 8), ntau), dim3(32, 8), 0, s, src, dst, ci, co, piv, n, col, singular);
+      std::swap(src, dst);
+    } else {
+      launch_pdl(k_gj_pivot, dim3(ntau), dim3((n + 31) & ~31), 0, s, src, prow, ci, piv, n, col, singular);
+      launch_pdl(k_gj_update, dim3(nt, nt, ntau), dim3(32, 8), 0, s, src, prow, ci, co, n, col);
+    }
   }
   cudaMemcpyAsync(dst, piv, sizeof(int32_t) * n * ntau, cudaMemcpyDeviceToDevice, s);
   k_gj_finish<T><<<dim3(nt, nt, ntau), dim3(32, 8), 0, s>>>(src, (const int32_t*)dst, inv, n);
