@@ -402,8 +402,9 @@ void fks_server_destroy(fks_server* srv);
  * cycles) or all levels (complex64 cycles), on 8 x 8 tiles up to 16384 or 131072
  * cells, 16 x 16 up to 524288 or 2097152, with a tail of at most 64 or 2048
  * cells; 3D operators fuse no level and use a tail of at most 512 or 2048 cells.
- * No cluster kernel. The fusion and tile thresholds count the cells of a
- * launch: a level's, times the sources of the batch.
+ * No cluster kernel. Until the tuner or one of the setters below has chosen
+ * them, the fusion and tile thresholds of a precision count the cells of a
+ * launch: a level's, times the sources of the batch; afterwards a level's.
  * `chosen` (host, may be NULL) receives the fusion threshold (fks_op_tiling
  * reads all four).
  */

@@ -286,6 +286,10 @@ struct fks_op {
   // (64^2 complex128 65 us a cycle with 64, 70 with 256; 289 x 311 complex64
   // 81 with 256, 66 with 1024)
   int64_t tail_max[2] = {64, 2048};
+  // Thresholds that the tuner or a program chose count a level's cells alone:
+  // they are picked with one source, and with nine of them the 112 x 96 levels
+  // that the tuner fuses take a solve of 150 shifts 21.1 ms fused, 30.3 per sweep.
+  bool by_level[2] = {false, false};
   // from the first level with at most this many cells (and a cluster layout)
   // down, the V-cycle runs in the cluster kernel instead of the tail (0: off)
   int64_t cluster_max[2] = {0, 0};
@@ -607,8 +611,8 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   const int64_t fmax = S.op->fuse_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t16 = S.op->tile16_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t8 = S.op->tile8_max[sizeof(VT) == 8 ? 0 : 1];
-  // the batch's sources share a launch: small tiles pay while it leaves SMs idle
-  const int64_t nsl = S.nslot;
+  // the batch's sources share a launch: untuned, small tiles while it leaves SMs idle
+  const int64_t nsl = S.op->by_level[sizeof(VT) == 8 ? 0 : 1] ? 1 : S.nslot;
   auto tile_of = [&](const LevelHost& L) { return L.n * nsl <= t8 ? 8 : (L.n * nsl <= t16 ? 16 : 32); };
   const int pix = sizeof(VT) == 8 ? 0 : 1;
   for (int l = 0; l < lp; ++l) {
@@ -1416,6 +1420,7 @@ static fks_status solve_impl(fks_op* op, Lane* lane, const fks_c128* b, int n_rh
       for (int pz = 0; pz < 2; ++pz)
         for (int l = 0; l < MAX_LEVELS; ++l) key.push_back((double)op->zchunk[pz][l]);
       key.push_back((double)op->coop_max[0]);
+      key.push_back((double)(op->by_level[0] + 2 * op->by_level[1]));
       key.push_back((double)op->coop_max[1]);
       key.push_back((double)pdl_flag());
       if (!lane->graph || lane->graph_key != key) {
@@ -2243,6 +2248,7 @@ fks_status fks_op_set_fusion(fks_op* op, int precision, int64_t max_cells) {
   if (op->csr) { set_error("fks_op_set_fusion: grid operators only"); return FKS_ERR_ARG; }
   if (!prec_ok(precision)) { set_error("fks_op_set_fusion: bad precision"); return FKS_ERR_ARG; }
   op->fuse_max[precision == FKS_PREC_FP64 ? 0 : 1] = max_cells < 0 ? INT64_MAX : max_cells;
+  op->by_level[precision == FKS_PREC_FP64 ? 0 : 1] = true;
   return FKS_OK;
 }
 
@@ -2251,6 +2257,7 @@ fks_status fks_op_set_tiles(fks_op* op, int precision, int64_t max_cells) {
   if (op->csr) { set_error("fks_op_set_tiles: grid operators only"); return FKS_ERR_ARG; }
   if (!prec_ok(precision)) { set_error("fks_op_set_tiles: bad precision"); return FKS_ERR_ARG; }
   op->tile16_max[precision == FKS_PREC_FP64 ? 0 : 1] = max_cells < 0 ? INT64_MAX : max_cells;
+  op->by_level[precision == FKS_PREC_FP64 ? 0 : 1] = true;
   return FKS_OK;
 }
 
@@ -2259,6 +2266,7 @@ fks_status fks_op_set_tiles8(fks_op* op, int precision, int64_t max_cells) {
   if (op->csr) { set_error("fks_op_set_tiles8: grid operators only"); return FKS_ERR_ARG; }
   if (!prec_ok(precision)) { set_error("fks_op_set_tiles8: bad precision"); return FKS_ERR_ARG; }
   op->tile8_max[precision == FKS_PREC_FP64 ? 0 : 1] = max_cells < 0 ? INT64_MAX : max_cells;
+  op->by_level[precision == FKS_PREC_FP64 ? 0 : 1] = true;
   return FKS_OK;
 }
 
@@ -2564,6 +2572,7 @@ fks_status fks_op_autotune(fks_op* op, int precision, fks_c128 tau, void* stream
       op->tail_max[pi] = pickt;
       op->cluster_max[pi] = pickc;
       op->tile8_max[pi] = pick8;
+      op->by_level[pi] = true;
     };
     if (precision == FKS_PREC_FP64) run(double{});
     else run(float{});
@@ -3376,6 +3385,7 @@ struct Batch : BatchBase {
       for (int pz = 0; pz < 2; ++pz)
         for (int l = 0; l < MAX_LEVELS; ++l) key.push_back((double)op->zchunk[pz][l]);
       key.push_back((double)op->coop_max[0]);
+      key.push_back((double)(op->by_level[0] + 2 * op->by_level[1]));
       key.push_back((double)op->coop_max[1]);
       key.push_back((double)pdl_flag());
       if (!lane->graph || lane->graph_key != key) {
