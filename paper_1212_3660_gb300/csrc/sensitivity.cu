@@ -19,8 +19,8 @@
 //     before, so a 2D cell takes 2 complex subtractions instead of 4;
 //   - the weights times Phi's differences are folded once per cell and shift,
 //     for up to SENS_M measurements.
-// 512^2, 200 shifts, 8 measurements: 26.1 ms with a thread per cell and shift
-// that did all of this itself.
+// 512^2, 200 shifts, 8 measurements: 20.0 ms; 26.1 with a thread per cell and
+// shift that did all of this itself.
 #include "sensitivity.cuh"
 #include "stencil.cuh"
 
@@ -28,7 +28,7 @@ namespace fks {
 
 constexpr int SENS_M = 8;       // measurements per pass (their differences below wait in shared memory)
 constexpr int SENS_WARPS = 8;
-constexpr int SENS_OUT = 31;    // cells of a row per warp; lane 0 is the cell left of them
+constexpr int SENS_OUT = 31;    // cells per warp; lane 0 is the cell before them
 
 // dt/dlnK_c of cell c's faces: w[a n + c], a in the order x low, x high, y, z
 __global__ void k_sens_weights(LevelView<double> L, const double* __restrict__ cond, double* __restrict__ w) {
@@ -72,29 +72,33 @@ __device__ __forceinline__ z64 cfma(z64 d, z64 a, z64 acc) {
   return acc;
 }
 
-// A warp owns 31 cells of a row and marches over `len` rows (2D) or planes (3D).
+// The march axis (y in 2D, z in 3D) is cut into strips of `len` steps. A warp
+// owns 31 consecutive cells of the list of all strips' first rows (planes), in
+// the order strip, row, x, and marches with them; a row may end and the next
+// one (or the next strip) begin inside a warp, so narrow grids leave no lanes
+// idle (48 x 32 x 32, 113 shifts, 7 measurements: 3.06 ms, 3.68 with two warps
+// per row).
 template <bool D3>
 __global__ void __launch_bounds__(SENS_WARPS * 32, 2)
     k_sensitivity(LevelView<double> L, const double* __restrict__ wt, const z64* __restrict__ phi,
                   const z64* __restrict__ psi, int n_m, int n_f, const z64* __restrict__ sigma, z64* __restrict__ jk,
-                  z64* __restrict__ js, int len, int ntx, int ncol) {
+                  z64* __restrict__ js, int len, int total) {
   __shared__ z64 below[SENS_M][SENS_WARPS * 32];  // psi(c) - psi(c + step) of the march step before
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = threadIdx.x, j = blockIdx.y;
-  const int nx = L.nx, ny = L.ny, sxy = nx * ny;
-  const int bx = blockIdx.x % ntx, rest = blockIdx.x / ntx;
-  const int i = bx * SENS_OUT + lane - 1;
-  const int row = D3 ? (rest % ncol) * SENS_WARPS + w : 0;           // the y row of a 3D march
-  const int m0 = (D3 ? rest / ncol : rest * SENS_WARPS + w) * len, nm = D3 ? L.nz : ny;
-  const int m1 = (!D3 || row < ny) ? min(m0 + len, nm) : m0;
-  if (m0 >= m1) return;  // whole warps: the shuffles below are among a warp's lanes
-  const bool in = i >= 0 && i < nx, out = in && lane > 0, xlo = i > 0, xhi = i < nx - 1;
+  const int lane = threadIdx.x & 31, t = threadIdx.x, j = blockIdx.y;
+  const int nx = L.nx, ny = L.ny, nm = D3 ? L.nz : ny, step = D3 ? nx * ny : nx;
+  const int g = (int)(blockIdx.x * SENS_WARPS + (t >> 5)) * SENS_OUT + lane - 1;
+  const bool own = g >= 0 && g < total;
+  const int strip = own ? g / step : 0, p = own ? g % step : 0, i = p % nx, row = p / nx;
+  const int m0 = strip * len, c0 = m0 * step + p;
+  // steps of the warp: its last strip may be shorter
+  const int steps = __reduce_max_sync(0xffffffffu, own ? min(len, nm - m0) : 0);
+  const bool xlo = i > 0, xhi = i < nx - 1;
   const bool ylo = row > 0, yhi = row < ny - 1;
-  const int step = D3 ? sxy : nx;
   const int64_t n = L.n;
   const z64* ph = phi + (int64_t)j * n;
   const z64 none = mk(0.0, 0.0), sg = sigma[j];
   // v(c) - v(c + 1), for the lane's cell and, from the lane below, its left face
-  auto xdiff = [&](const z64* v, int c, z64 here, z64* lo, z64* hi) {
+  auto xdiff = [&](const z64* v, int c, bool in, z64 here, z64* lo, z64* hi) {
     z64 right = shfl_dn(here);
     if (lane == 31 && in && xhi) right = v[c + 1];
     *hi = here - right;
@@ -102,21 +106,22 @@ __global__ void __launch_bounds__(SENS_WARPS * 32, 2)
   };
   for (int mc = 0; mc < n_m; mc += SENS_M) {
     const int nmc = min(SENS_M, n_m - mc);
-    int c = m0 * step + row * nx + i;
-    z64 ph_c = in ? ph[c] : none;
+    int c = c0;
+    z64 ph_c = own ? ph[c] : none;
     z64 ph_lo = none;  // phi(c - step) - phi(c)
-    if (m0 > 0 && in) {
+    if (m0 > 0 && own) {
       ph_lo = ph[c - step] - ph_c;
       for (int q = 0; q < nmc; ++q) {
         const z64* ps = psi + ((int64_t)(mc + q) * n_f + j) * n;
         below[q][t] = ps[c - step] - ps[c];
       }
     }
-    for (int m = m0; m < m1; ++m, c += step) {
+    for (int m = m0; m < m0 + steps; ++m, c += step) {
+      const bool in = own && m < nm, out = in && lane > 0;
       const bool mlo = m > 0, mhi = m + 1 < nm;
       const z64 ph_n = in && mhi ? ph[c + step] : none;
       z64 dl, dh;
-      xdiff(ph, c, ph_c, &dl, &dh);
+      xdiff(ph, c, in, ph_c, &dl, &dh);
       const z64 dm = ph_c - ph_n;
       z64 a[6];
       z64 smphi = none;
@@ -148,7 +153,7 @@ __global__ void __launch_bounds__(SENS_WARPS * 32, 2)
           nn = in && mhi ? next[c + step] : none;
         }
         z64 xl, xh;
-        xdiff(ps, c, pc, &xl, &xh);
+        xdiff(ps, c, in, pc, &xl, &xh);
         const z64 d = pc - pn, lo = below[q][t];
         below[q][t] = d;
         if (out) {
@@ -181,15 +186,15 @@ void launch_sensitivity(const LevelHost& L0, const double* cond, const z64* phi,
   const LevelView<double> L = view<double>(L0);
   auto up = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
   k_sens_weights<<<(unsigned)up(L0.n, 256), 256, 0, s>>>(L, cond, work);
-  // march length: 16 while that leaves eight blocks per SM
-  const int64_t ntx = up(L0.nx, SENS_OUT), nm = L0.nz > 1 ? L0.nz : L0.ny;
-  const int64_t ncol = L0.nz > 1 ? up(L0.ny, SENS_WARPS) : 1;
-  auto blocks = [&](int len) { return ntx * ncol * up(nm, (int64_t)len * (L0.nz > 1 ? 1 : SENS_WARPS)); };
-  int len = 16;
+  // strips of 16 steps while that leaves eight blocks per SM, then of equal length
+  const int64_t nm = L0.nz > 1 ? L0.nz : L0.ny, part = L0.n / nm;
+  auto blocks = [&](int64_t len) { return up(part * up(nm, len), SENS_OUT * SENS_WARPS); };
+  int64_t len = 16;
   while (len > 1 && blocks(len) * n_f < 8 * 152) len /= 2;
+  len = up(nm, up(nm, len));
   const dim3 g((unsigned)blocks(len), (unsigned)n_f);
   auto kernel = L0.nz > 1 ? k_sensitivity<true> : k_sensitivity<false>;
-  kernel<<<g, SENS_WARPS * 32, 0, s>>>(L, work, phi, psi, n_m, n_f, sigma, jk, js, len, (int)ntx, (int)ncol);
+  kernel<<<g, SENS_WARPS * 32, 0, s>>>(L, work, phi, psi, n_m, n_f, sigma, jk, js, (int)len, (int)(part * up(nm, len)));
 }
 
 }  // namespace fks
