@@ -149,39 +149,46 @@ __device__ __forceinline__ void digits7(double v, int e, int (&d)[TC_SLICES]) {
 }
 
 // (hi + lo 2^-28) 2^E rounded to the nearest double (ties to even), with integer
-// instructions only: N = hi 2^28 + lo is exact in 128 bits (|hi| < 2^47), its
-// leading 53 bits are rounded by the bits below them, and the exponent is set
-// directly. Equal to scalbn(fma((double)lo, 0x1p-28, (double)hi), E) whenever
-// the result is a normal double; returns false otherwise (the caller then takes
-// that FP64 form).
+// instructions only: N = hi 2^28 + lo is exact (|hi| < 2^47, |lo| < 2^60), its
+// leading 64 bits and a sticky bit for the rest are rounded to 53, and the
+// exponent is set directly. Equal to scalbn(fma((double)lo, 0x1p-28,
+// (double)hi), E) whenever the result is a normal double; returns false
+// otherwise (the caller then takes that FP64 form).
 __device__ __forceinline__ bool int_to_double(long long hi, long long lo, int E, double* out) {
-  const __int128 N = ((__int128)hi << 28) + (__int128)lo;
-  if (N == 0) {
-    *out = 0.0;
-    return true;
+  // N = t 2^28 + l with 0 <= l < 2^28, then |N|
+  long long t = hi + (lo >> 28);
+  unsigned l = (unsigned)lo & 0xfffffffu;
+  const unsigned long long sign = (unsigned long long)t & (1ull << 63);
+  if (sign) {
+    t = ~t + (l == 0u);
+    l = (0u - l) & 0xfffffffu;
   }
-  const unsigned long long sign = N < 0 ? 1ull : 0ull;
-  const unsigned __int128 u = N < 0 ? (unsigned __int128)(-N) : (unsigned __int128)N;
-  const unsigned long long uh = (unsigned long long)(u >> 64), ul = (unsigned long long)u;
-  const int p = uh ? 127 - __clzll((long long)uh) : 63 - __clzll((long long)ul);  // leading bit
-  unsigned long long m;
-  int ex = p;
-  if (p <= 52) {
-    m = ul << (52 - p);
+  const unsigned long long u = (unsigned long long)t;
+  unsigned long long M;  // N's leading 64 bits, left-justified
+  int p;                 // position of the leading bit
+  bool sticky = false;
+  if (u >> 36) {
+    const int n = __clzll((long long)u);  // 15 .. 27
+    M = (u << n) | (l >> (28 - n));
+    sticky = (l << (n + 4)) != 0u;
+    p = 91 - n;
   } else {
-    const int sh = p - 52;  // 1 .. 75
-    const unsigned __int128 q = u >> sh;
-    const unsigned __int128 rem = u - (q << sh), half = (unsigned __int128)1 << (sh - 1);
-    m = (unsigned long long)q;
-    if (rem > half || (rem == half && (m & 1ull))) ++m;
-    if (m == (1ull << 53)) {
-      m >>= 1;
-      ++ex;
+    const unsigned long long v = (u << 28) | l;
+    if (v == 0ull) {
+      *out = 0.0;
+      return true;
     }
+    const int n = __clzll((long long)v);
+    M = v << n;
+    p = 63 - n;
   }
-  const int be = ex + E - 28 + 1023;
-  if (be < 1 || be > 2046) return false;
-  *out = __longlong_as_double((long long)((sign << 63) | ((unsigned long long)be << 52) | (m & ((1ull << 52) - 1))));
+  const int be = p + E - 28 + 1023;
+  if (be < 1 || be > 2045) return false;
+  unsigned long long m = M >> 11;  // 53 bits
+  const unsigned low = (unsigned)M & 0x7ffu;
+  if (low > 0x400u || (low == 0x400u && (sticky || (m & 1ull)))) ++m;
+  // adding m with its leading bit raises the exponent field by one, or by two when the rounding carried
+  *out = __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + m)));
   return true;
 }
 
@@ -280,8 +287,10 @@ __global__ void __launch_bounds__(TC_N) k_tc_slice_b(const SlotState* __restrict
 // write x_j, so a tile's epilogue overlaps the next tile's MMAs: warp w reads
 // TMEM lanes 32 (w mod 4) .. + 31 (one row per thread) and the EPI_COLS columns
 // of group w / 4 of the tile, four warps per SM sub-partition to hide the
-// latency of the integer epilogue. Barriers: full/empty per stage,
-// tfull/tempty per accumulator set.
+// latency of the integer epilogue, whose instructions bound the kernel (two
+// levels joined in 32 bits and int_to_double in 64: 128^3, 200 shifts 4.95 ms;
+// 5.73 with 64-bit and 128-bit arithmetic throughout). Barriers: full/empty per
+// stage, tfull/tempty per accumulator set.
 constexpr int PS = 4;
 constexpr int P_EPI = 16;                  // epilogue warps
 constexpr int EPI_COLS = TC_N * 4 / P_EPI; // columns of a tile per epilogue warp (8)
@@ -463,10 +472,10 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_tc_gemm(const SlotState* __res
             tmem_wait();
 #pragma unroll
             for (int c = 0; c < EPI_COLS; ++c) {
-              const long long a0 = (long long)__float2int_rn(__uint_as_float(v0[c]));
-              const long long a1 = (long long)__float2int_rn(__uint_as_float(v1[c]));
-              if (lev < 4) hi[c] = (hi[c] * 128 + a0) * 128 + a1;
-              else lo[c] = (lo[c] * 128 + a0) * 128 + a1;
+              // two levels in 32 bits: |a0|, |a1| < 8 127^2 128, so |128 a0 + a1| < 2^31
+              const int a = __float2int_rn(__uint_as_float(v0[c])) * 128 + __float2int_rn(__uint_as_float(v1[c]));
+              if (lev < 4) hi[c] = hi[c] * 16384 + a;
+              else lo[c] = lo[c] * 16384 + a;
             }
           }
           tc_fence_before();
