@@ -173,9 +173,31 @@ struct Lane {
     CK(cudaEventCreateWithFlags(&ev_x, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_copied, cudaEventDisableTiming));
   }
+  // page-locked copies of the slots' states after the last two cycles of a
+  // host-driven inner solve, and the events behind them
+  SlotState* poll = nullptr;
+  int poll_slots = 0;
+  cudaEvent_t ev_poll[2] = {};
+  void poll_init(int nslot) {
+    if (!ev_poll[0])
+      for (auto& e : ev_poll) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (poll_slots >= nslot) return;
+    if (poll) cudaFreeHost(poll);
+    poll = nullptr;
+    poll_slots = 0;
+    CK(cudaMallocHost(&poll, 2 * nslot * sizeof(SlotState)));
+    poll_slots = nslot;
+  }
   void release() {
     if (graph) cudaGraphExecDestroy(graph);
     graph = nullptr;
+    if (poll) cudaFreeHost(poll);
+    poll = nullptr;
+    poll_slots = 0;
+    for (auto& e : ev_poll) {
+      if (e) cudaEventDestroy(e);
+      e = nullptr;
+    }
     if (side) {
       cudaStreamSynchronize(side);
       cudaStreamDestroy(side);
@@ -1026,6 +1048,34 @@ static void inner_solve(Solve& S, const z64* V, int64_t vsV, z64* Z, int64_t vsZ
   while (any_inner_running(S)) {
     sec_inner_body<VT>(S, V, vsV, Z, vsZ, 0, 0);
     if (++guard > 100000) break;
+  }
+}
+
+// The same for a grid operator, one cycle ahead of the answer: cycle c is
+// enqueued before the host reads whether the state it starts from still needs
+// it, so the GPU does not wait for the host between cycles (one apply at 512^2
+// complex64 1190 us waiting, 1125 ahead; 16 x 16 x 32 1282 and 1232). The kernels
+// of a cycle that turns out not to be needed return at once and change nothing.
+template <typename VT>
+static void inner_solve_ahead(Solve& S, const z64* V, int64_t vsV, z64* Z, int64_t vsZ) {
+  Lane& L = *S.lane;
+  L.poll_init(S.nslot);
+  auto post = [&](int i) {
+    CK(cudaMemcpyAsync(L.poll + (i & 1) * S.nslot, S.st, sizeof(SlotState) * S.nslot, cudaMemcpyDeviceToHost, S.s));
+    CK(cudaEventRecord(L.ev_poll[i & 1], S.s));
+  };
+  sec_inner_first<VT>(S, V, vsV, Z, vsZ, 0, 0);
+  post(0);
+  for (int c = 0; c < 100000; ++c) {
+    sec_inner_body<VT>(S, V, vsV, Z, vsZ, 0, 0);
+    post(c + 1);
+    CK(cudaEventSynchronize(L.ev_poll[c & 1]));
+    bool running = false;
+    for (int q = 0; q < S.nslot; ++q) {
+      const SlotState& t = L.poll[(c & 1) * S.nslot + q];
+      running |= t.active && !t.inner_done;
+    }
+    if (!running) break;
   }
 }
 
@@ -2916,7 +2966,9 @@ fks_status fks_precond_apply(fks_op* op, fks_c128 tau, const fks_c128* v, fks_c1
       std::vector<SlotState> sh(1);
       S.st_host = sh.data();
       setup_levels<VT>(S);
-      inner_solve<VT>(S, S.V, n, S.Z, n);
+      // per-kernel timing counts only launches that work: not ahead then
+      if (op->csr || S.lane->prof.cls >= 0) inner_solve<VT>(S, S.V, n, S.Z, n);
+      else inner_solve_ahead<VT>(S, S.V, n, S.Z, n);
       CK(cudaGetLastError());
       copy_out(z, S.Z, sizeof(z64) * n, s);
       CK(cudaMemcpyAsync(S.st_host, S.st, sizeof(SlotState), cudaMemcpyDeviceToHost, s));
