@@ -3,7 +3,8 @@
 // k_post2d / k_tail_vcycle in the same order:
 //   Gauss-Seidel   z = invd * (f + t_xl z_xl + t_xh z_xh + t_yl z_yl + t_yh z_yh)
 //   residual       f - ((d + tau m) z - sum t z_nb), d the sum of the cell's faces
-//   restriction    sum of the four children's residuals, children in (y, x) order
+//   restriction    sum of the four children's residuals, children in (y, x)
+//                  order; in complex128 of the two red ones (RED_RESIDUAL)
 //   prolongation   prolong_value_at (cell-centred bilinear)
 //   coarsest       z = Ainv f, row by row.
 #include <cooperative_groups.h>
@@ -192,13 +193,13 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
     fa.zl = T(0);
     fa.zh = T(0);
     const T d = fsum(fa), m = MM[r];
-    cx<T> nb = mk(T(0), T(0));
-    if (i > 0) nb = axpy(fa.xl, Z[r - 1], nb);
-    if (i < A.nx - 1) nb = axpy(fa.xh, Z[r + 1], nb);
-    if (j > 0) nb = axpy(fa.yl, zrow(A, Z, lj - 1, i), nb);
-    if (j < A.ny - 1) nb = axpy(fa.yh, zrow(A, Z, lj + 1, i), nb);
-    const cx<T> Az = mk(fmaT(sft.re, m, d), mulT(sft.im, m)) * Z[r] - nb;
-    return F[r] - Az;
+    return residual_of(F[r], Z[r], mk(fmaT(sft.re, m, d), mulT(sft.im, m)), [&](cx<T> nb) {
+      if (i > 0) nb = axpy(fa.xl, Z[r - 1], nb);
+      if (i < A.nx - 1) nb = axpy(fa.xh, Z[r + 1], nb);
+      if (j > 0) nb = axpy(fa.yl, zrow(A, Z, lj - 1, i), nb);
+      if (j < A.ny - 1) nb = axpy(fa.yh, zrow(A, Z, lj + 1, i), nb);
+      return nb;
+    });
   };
 
   // ---- down: smoothing and restriction on the banded levels
@@ -216,7 +217,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
         const int lJ = t / cnx, I = t - lJ * cnx;
         cx<T> acc = mk(T(0), T(0));
         for (int bb = 0; bb < 2; ++bb)
-          for (int a = 0; a < 2; ++a) acc = acc + residual(A, 2 * I + a, 2 * lJ + bb);
+          for (int a = child_first<T>(bb); a < 2; a += child_step<T>) acc = acc + residual(A, 2 * I + a, 2 * lJ + bb);
         FN[t] = acc;
       }
       cl.sync();
@@ -226,7 +227,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
       cx<T>* RS = (cx<T>*)(csm + P.rs);
       for (int t = tid; t < A.R * A.nx; t += nt) {
         const int lj = t / A.nx, i = t - lj * A.nx;
-        RS[t] = residual(A, i, lj);
+        if (!RED_RESIDUAL<T> || ((i + b * A.R + lj) & 1) == 0) RS[t] = residual(A, i, lj);
       }
       cl.sync();
       if (b == 0) {
@@ -236,7 +237,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 1)
           const int J = t / P.ncx, I = t - J * P.ncx;
           cx<T> acc = mk(T(0), T(0));
           for (int bb = 0; bb < 2; ++bb)
-            for (int a = 0; a < 2; ++a) {
+            for (int a = child_first<T>(bb); a < 2; a += child_step<T>) {
               const int j = 2 * J + bb, i = 2 * I + a;
               const int owner = j / A.R, lj = j - owner * A.R;
               acc = acc + cl.map_shared_rank(RS, owner)[lj * A.nx + i];

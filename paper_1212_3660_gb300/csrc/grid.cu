@@ -311,7 +311,8 @@ __global__ void k_gs_correct(LevelView<T, C> L, const SlotState* st, const cx<T>
 }
 
 // --------------------------------------------------------------------- transfer
-// Coarse right-hand side = sum over the children of the fine residual f - A z.
+// Coarse right-hand side = sum over the children of the fine residual f - A z
+// (restrict_value).
 // Sources as in k_gs (threadIdx.z), so the children's coefficients come from
 // memory once per block.
 template <typename T, typename C>
@@ -332,18 +333,21 @@ __global__ void k_residual_restrict(LevelView<T, C> F, int rx, int ry, int rz, i
 
 // Coarse right-hand side on a 3D level coarsened by 2 in every axis, one
 // source per block. The per-coarse-cell loop of k_residual_restrict computes
-// its eight children one after another; here the block's 256 threads first
-// compute the fine residuals f - A z of a 32 x 8 x 2 tile, one (i, j) column
-// of two planes each, into shared memory, then one thread per coarse cell
-// adds its children in restrict_value's order (z, then y, then x child),
-// skipping those past the fine grid, so the sum is bitwise the same.
+// its children one after another; here the block's 256 threads first compute
+// the fine residuals f - A z of a 32 x 8 x 2 tile, one (i, j) column of two
+// planes each (one red cell in complex128, two cells in complex64), into shared
+// memory, then one thread per coarse cell adds its children in
+// restrict_value's order (z, then y, then x child), skipping those past the
+// fine grid, so the sum is bitwise the same (64 x 48 x 48 complex128 9.9 us a
+// launch with all cells, 5.5 with the red ones).
 template <typename T, typename C>
 __global__ void __launch_bounds__(256) k_residual_restrict3(LevelView<T, C> F, int cnx, int cny, int cnz,
                                                             const SlotState* st, const z64* taus,
                                                             const cx<T>* __restrict__ f, const cx<T>* __restrict__ z,
                                                             int64_t vs, cx<T>* __restrict__ fc, int64_t vsc) {
   pdl_enter();
-  __shared__ cx<T> sr[2][GY][GX];
+  constexpr int NP = RED_RESIDUAL<T> ? 1 : 2;  // cells per column
+  __shared__ cx<T> sr[NP][GY][GX];
   const int slot = blockIdx.z;
   if (!slot_running(st, slot)) return;
   const int nby = (F.ny + GY - 1) / GY;
@@ -353,12 +357,12 @@ __global__ void __launch_bounds__(256) k_residual_restrict3(LevelView<T, C> F, i
   const cx<T>* fs = f + slot * vs;
   const cx<T>* zs = z + slot * vs;
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int k = 2 * K + q;
+  for (int q = 0; q < NP; ++q) {
+    const int k = 2 * K + (NP == 1 ? (i + j) & 1 : q);
     cx<T> r = mk(T(0), T(0));
     if (i < F.nx && j < F.ny && k < F.nz) {
       const int64_t cc = ((int64_t)k * F.ny + j) * F.nx + i;
-      r = fs[cc] - apply_at(F, Cell{i, j, k}, cc, s, zs);
+      r = residual_at(F, Cell{i, j, k}, cc, s, fs, zs);
     }
     sr[q][threadIdx.y][threadIdx.x] = r;
   }
@@ -374,9 +378,9 @@ __global__ void __launch_bounds__(256) k_residual_restrict3(LevelView<T, C> F, i
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
-      for (int a = 0; a < 2; ++a) {
+      for (int a = child_first<T>(b + c); a < 2; a += child_step<T>) {
         if (2 * I + a >= F.nx || 2 * J + b >= F.ny || 2 * K + c >= F.nz) continue;
-        acc = acc + sr[c][2 * tj + b][2 * ti + a];
+        acc = acc + sr[NP == 1 ? 0 : c][2 * tj + b][2 * ti + a];
       }
   fc[slot * vsc + ((int64_t)K * cny + J) * cnx + I] = acc;
 }
@@ -513,27 +517,43 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (TX == 32 ? 6 : 8) : 4) 
     int gx = x0 + FH + xx, gy = y0 + FH + yy;
     if (gx < L.nx && gy < L.ny) zs[gy * L.nx + gx] = sZ[(yy + FH) * RX + xx + FH];
   }
-  // residual + restriction to the (TX/2) x (TY/2) coarse cells of the tile
+  // residual + restriction to the (TX/2) x (TY/2) coarse cells of the tile. Two
+  // lanes per coarse cell, one for each of its rows of children: with one, a
+  // quarter of the threads did it all, on half of the SM's FP64 units (512^2
+  // complex128, all cells: 29.8 us a launch; two lanes, red cells: 27.2)
   const int cnx = (L.nx + 1) >> 1, cny = (L.ny + 1) >> 1;
   cx<T>* fcs = fc + slot * vsc;
-  for (int q = tid; q < (TX / 2) * (TY / 2); q += nt) {
-    int Yl = q / (TX / 2), Xl = q - Yl * (TX / 2);
-    int X = blockIdx.x * (TX / 2) + Xl, Y = blockIdx.y * (TY / 2) + Yl;
-    if (X >= cnx || Y >= cny) continue;
+  constexpr int NC = RED_RESIDUAL<T> ? 1 : 2;    // children per lane
+  for (int q = tid; q < TX * TY / 2; q += nt) {  // whole warps
+    const int h = q & 1, C = q >> 1;
+    const int Yl = C / (TX / 2), Xl = C - Yl * (TX / 2);
+    const int X = blockIdx.x * (TX / 2) + Xl, Y = blockIdx.y * (TY / 2) + Yl;
+    const int gy = 2 * Y + h;
     cx<T> acc = mk(T(0), T(0));
-#pragma unroll 1
-    for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 2; ++a) {
-        int gx = 2 * X + a, gy = 2 * Y + b;
-        if (gx >= L.nx || gy >= L.ny) continue;
-        int r = (gy - y0) * RX + (gx - x0);
-        int c = gy * L.nx + gx;
-        Faces<T> fa = faces_at(L, Cell{gx, gy, 0});
-        T d = sizeof(T) == 8 && L.kd ? L.kd[c] : fsum(fa), m = L.mm[c];
-        cx<T> Az = mk(fmaT(sft.re, m, d), mulT(sft.im, m)) * sZ[r] - nb_sum_tile(L, Cell{gx, gy, 0}, r, RX, sZ);
-        acc = acc + (sF[r] - Az);
-      }
-    fcs[Y * cnx + X] = acc;
+    cx<T> res[NC];
+    bool in[NC];
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+      const int gx = 2 * X + (NC == 1 ? h : a);
+      in[a] = gx < L.nx && gy < L.ny;
+      res[a] = acc;
+      if (!in[a]) continue;
+      const int r = (gy - y0) * RX + (gx - x0);
+      const int c = gy * L.nx + gx;
+      const T d = sizeof(T) == 8 && L.kd ? L.kd[c] : fsum(faces_at(L, Cell{gx, gy, 0})), m = L.mm[c];
+      res[a] = residual_of(sF[r], sZ[r], mk(fmaT(sft.re, m, d), mulT(sft.im, m)),
+                           [&](cx<T> s0) { return nb_sum_tile(L, Cell{gx, gy, 0}, r, RX, sZ, s0); });
+    }
+    // the children in their order: the even lane's, then the odd lane's
+#pragma unroll
+    for (int a = 0; a < NC; ++a)
+      if (in[a]) acc = acc + res[a];
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+      const cx<T> other = mk(__shfl_down_sync(0xffffffffu, res[a].re, 1), __shfl_down_sync(0xffffffffu, res[a].im, 1));
+      if (__shfl_down_sync(0xffffffffu, (int)in[a], 1)) acc = acc + other;
+    }
+    if (h == 0 && in[0]) fcs[Y * cnx + X] = acc;
   }
 }
 
@@ -704,7 +724,8 @@ __global__ void __launch_bounds__(TilePair<T, TX>::NT) k_pre2d_pairs(LevelView<T
   using Tile = TilePair<T, TX>;
   pdl_enter();
   __shared__ cx<T> zmem[Tile::ZN];
-  __shared__ cx<T> res[TX][TX];
+  constexpr int NC = RED_RESIDUAL<T> ? 1 : 2;  // the pair's red cell, or both
+  __shared__ cx<T> res[TX][NC * TX / 2];
   const int slot = blockIdx.z;
   if (!slot_running(st, slot)) return;
   const int tau = st[slot].tau;
@@ -713,14 +734,15 @@ __global__ void __launch_bounds__(TilePair<T, TX>::NT) k_pre2d_pairs(LevelView<T
   Tile q;
   q.load(L, invd + (int64_t)tau * L.n, f + slot * vs);
   const bool mine = q.interior();
-  T d[2] = {T(0), T(0)}, m[2] = {T(0), T(0)};
-  if (mine) {
+  T d[NC], m[NC];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (q.in[h]) {
-        m[h] = L.mm[q.c + h];
-        if (sizeof(T) == 8 && L.kd) d[h] = L.kd[q.c + h];
-      }
+  for (int a = 0; a < NC; ++a) {
+    const int h = NC == 1 ? q.gy & 1 : a;  // gx is even
+    d[a] = m[a] = T(0);
+    if (mine && (h ? q.in[1] : q.in[0])) {
+      m[a] = L.mm[q.c + h];
+      if (sizeof(T) == 8 && L.kd) d[a] = L.kd[q.c + h];
+    }
   }
   for (int e = threadIdx.x; e < Tile::ZN; e += Tile::NT) zmem[e] = mk(T(0), T(0));
   __syncthreads();
@@ -736,12 +758,19 @@ __global__ void __launch_bounds__(TilePair<T, TX>::NT) k_pre2d_pairs(LevelView<T
     cx<T>* zs = z + slot * vs;
     const int yy = q.ry - FH, xx = q.r - q.ry * Tile::RX - FH;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (!q.in[h]) continue;
-      zs[q.c + h] = q.z[h];
-      if (!(sizeof(T) == 8 && L.kd)) d[h] = ((q.x[h] + q.x[h + 1]) + (q.yl[h] + q.yh[h])) + T(0);
-      const cx<T> Az = mk(fmaT(sft.re, m[h], d[h]), mulT(sft.im, m[h])) * q.z[h] - q.nb(Z, h, mk(T(0), T(0)));
-      res[yy][xx + h] = q.f[h] - Az;
+    for (int h = 0; h < 2; ++h)
+      if (q.in[h]) zs[q.c + h] = q.z[h];
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+      const int h = NC == 1 ? q.gy & 1 : a;
+      if (!(h ? q.in[1] : q.in[0])) continue;
+      if (!(sizeof(T) == 8 && L.kd)) {
+        const T x0 = h ? q.x[1] : q.x[0], x1 = h ? q.x[2] : q.x[1];
+        d[a] = ((x0 + x1) + ((h ? q.yl[1] : q.yl[0]) + (h ? q.yh[1] : q.yh[0]))) + T(0);
+      }
+      res[yy][NC == 1 ? xx >> 1 : xx + a] =
+          residual_of(h ? q.f[1] : q.f[0], h ? q.z[1] : q.z[0], mk(fmaT(sft.re, m[a], d[a]), mulT(sft.im, m[a])),
+                      [&](cx<T> s0) { return q.nb(Z, h, s0); });
     }
   }
   __syncthreads();
@@ -755,8 +784,8 @@ __global__ void __launch_bounds__(TilePair<T, TX>::NT) k_pre2d_pairs(LevelView<T
 #pragma unroll
   for (int b = 0; b < 2; ++b)
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
-      if (2 * X + a < L.nx && 2 * Y + b < L.ny) acc = acc + res[2 * Yl + b][2 * Xl + a];
+    for (int a = child_first<T>(b); a < 2; a += child_step<T>)
+      if (2 * X + a < L.nx && 2 * Y + b < L.ny) acc = acc + res[2 * Yl + b][NC == 1 ? Xl : 2 * Xl + a];
   fc[slot * vsc + (int64_t)Y * cnx + X] = acc;
 }
 
@@ -1027,30 +1056,30 @@ __device__ __forceinline__ void tail2d_gs(TailPair<T>& q, int nx, int ny, cx<T>*
   }
 }
 
-// f - (K + s M) z on the two owned cells (apply_at with d the sum of the faces)
+// f - (K + s M) z on cell h of the owned pair (residual_at with d the sum of the faces)
 template <typename T>
-__device__ __forceinline__ void tail2d_residual(const TailPair<T>& q, int nx, int ny, const cx<T>* Z, cx<T> s,
-                                                cx<T>* r0, cx<T>* r1) {
+__device__ __forceinline__ cx<T> tail2d_residual(const TailPair<T>& q, int nx, int ny, const cx<T>* Z, cx<T> s, int h) {
   const T zero = T(0);
-  {
+  if (h == 0) {
     Faces<T> fa{q.fxa, q.fxb, q.yl0, q.yh0, zero, zero};
     const T d = fsum(fa);
-    cx<T> nb = mk(zero, zero);
-    if (q.i0 > 0) nb = axpy(q.fxa, Z[q.c0 - 1], nb);
-    nb = axpy(q.fxb, q.z1, nb);
-    if (q.j > 0) nb = axpy(q.yl0, Z[q.c0 - nx], nb);
-    if (q.j < ny - 1) nb = axpy(q.yh0, Z[q.c0 + nx], nb);
-    *r0 = q.f0 - (mk(fmaT(s.re, q.m0, d), mulT(s.im, q.m0)) * q.z0 - nb);
-  }
-  {
+    return residual_of(q.f0, q.z0, mk(fmaT(s.re, q.m0, d), mulT(s.im, q.m0)), [&](cx<T> nb) {
+      if (q.i0 > 0) nb = axpy(q.fxa, Z[q.c0 - 1], nb);
+      nb = axpy(q.fxb, q.z1, nb);
+      if (q.j > 0) nb = axpy(q.yl0, Z[q.c0 - nx], nb);
+      if (q.j < ny - 1) nb = axpy(q.yh0, Z[q.c0 + nx], nb);
+      return nb;
+    });
+  } else {
     Faces<T> fa{q.fxb, q.fxc, q.yl1, q.yh1, zero, zero};
     const T d = fsum(fa);
-    cx<T> nb = mk(zero, zero);
-    nb = axpy(q.fxb, q.z0, nb);
-    if (q.i0 + 1 < nx - 1) nb = axpy(q.fxc, Z[q.c0 + 2], nb);
-    if (q.j > 0) nb = axpy(q.yl1, Z[q.c0 + 1 - nx], nb);
-    if (q.j < ny - 1) nb = axpy(q.yh1, Z[q.c0 + 1 + nx], nb);
-    *r1 = q.f1 - (mk(fmaT(s.re, q.m1, d), mulT(s.im, q.m1)) * q.z1 - nb);
+    return residual_of(q.f1, q.z1, mk(fmaT(s.re, q.m1, d), mulT(s.im, q.m1)), [&](cx<T> nb) {
+      nb = axpy(q.fxb, q.z0, nb);
+      if (q.i0 + 1 < nx - 1) nb = axpy(q.fxc, Z[q.c0 + 2], nb);
+      if (q.j > 0) nb = axpy(q.yl1, Z[q.c0 + 1 - nx], nb);
+      if (q.j < ny - 1) nb = axpy(q.yh1, Z[q.c0 + 1 + nx], nb);
+      return nb;
+    });
   }
 }
 
@@ -1091,20 +1120,31 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
       tail2d_gs(q, nx, ny, Z, 1, 0);
       __syncthreads();
     }
-    // restriction: the pair in row 2J sums its two residuals, the pair in
-    // row 2J + 1 adds its own onto that (the child order of restrict_value)
+    // restriction: the pair in row 2J sums its residuals (in complex128 its red
+    // cell's is all), the pair in row 2J + 1 adds its own onto that (the child
+    // order of restrict_value)
     const int cnx = B.L.nx;
     cx<T>* FC = sh + B.off;
     cx<T>* S = FC + B.L.n;  // the coarse iterate's storage, free until its first sweep
-    cx<T> r0, r1;
+    constexpr int NC = RED_RESIDUAL<T> ? 1 : 2;
+    cx<T> res[NC];
     if (q.own) {
-      tail2d_residual(q, nx, ny, Z, sft, &r0, &r1);
-      if ((q.j & 1) == 0) S[(q.j >> 1) * cnx + (q.i0 >> 1)] = (mk(T(0), T(0)) + r0) + r1;
+#pragma unroll
+      for (int a = 0; a < NC; ++a) res[a] = tail2d_residual(q, nx, ny, Z, sft, NC == 1 ? q.j & 1 : a);
+      if ((q.j & 1) == 0) {
+        cx<T> acc = mk(T(0), T(0));
+#pragma unroll
+        for (int a = 0; a < NC; ++a) acc = acc + res[a];
+        S[(q.j >> 1) * cnx + (q.i0 >> 1)] = acc;
+      }
     }
     __syncthreads();
     if (q.own && (q.j & 1)) {
       const int C = (q.j >> 1) * cnx + (q.i0 >> 1);
-      FC[C] = (S[C] + r0) + r1;
+      cx<T> acc = S[C];
+#pragma unroll
+      for (int a = 0; a < NC; ++a) acc = acc + res[a];
+      FC[C] = acc;
     }
     __syncthreads();
   }
@@ -1172,7 +1212,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
 // of one row and keeps its coefficients, right-hand side and iterate in
 // registers for the whole visit of the level, so a half sweep is a handful of
 // shared-memory reads and 16 multiply-adds per thread. k_tail_vcycle, which
-// finds its cells again in every half sweep, sums eight residuals per coarse
+// finds its cells again in every half sweep, sums the residuals of a coarse
 // cell one after another and reads the coarsest inverse row by row, was bound
 // by those chains: 16 us for 8^3 and 4^3 cells in complex64.
 // The residuals go through shared memory and are added per coarse cell in
@@ -1292,14 +1332,17 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
     __syncthreads();
     pair_gs(q, L, Z, 1, false);
     __syncthreads();
-    if (q.own) {
+    constexpr int NC = RED_RESIDUAL<T> ? 1 : 2;  // the pair's red cell, or both
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h && !q.right) break;
-        const T d = ((q.x[h] + q.x[h + 1]) + (q.yl[h] + q.yh[h])) + (q.zl[h] + q.zh[h]);
-        const cx<T> Az = mk(fmaT(sft.re, q.m[h], d), mulT(sft.im, q.m[h])) * q.z[h] - pair_nb(q, L, Z, h, none);
-        R[q.c0 + h] = q.f[h] - Az;
-      }
+    for (int a = 0; a < NC; ++a) {
+      const int h = NC == 1 ? (q.j + q.k) & 1 : a;
+      if (!q.own || (h && !q.right)) continue;
+      const T x0 = h ? q.x[1] : q.x[0], x1 = h ? q.x[2] : q.x[1];
+      const T yl = h ? q.yl[1] : q.yl[0], yh = h ? q.yh[1] : q.yh[0];
+      const T zl = h ? q.zl[1] : q.zl[0], zh = h ? q.zh[1] : q.zh[0], m = h ? q.m[1] : q.m[0];
+      const T d = ((x0 + x1) + (yl + yh)) + (zl + zh);
+      R[q.c0 + h] = residual_of(h ? q.f[1] : q.f[0], h ? q.z[1] : q.z[0], mk(fmaT(sft.re, m, d), mulT(sft.im, m)),
+                                [&](cx<T> s0) { return pair_nb(q, L, Z, h, s0); });
     }
     __syncthreads();
     cx<T>* FC = sh + B.off;
@@ -1308,7 +1351,7 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
       cx<T> acc = none;
       for (int c = 0; c < A.rz; ++c)
         for (int b = 0; b < A.ry; ++b)
-          for (int a = 0; a < A.rx; ++a) {
+          for (int a = child_first<T>(A.rx * p.i + A.ry * p.j + b + A.rz * p.k + c); a < A.rx; a += child_step<T>) {
             const int i = A.rx * p.i + a, j = A.ry * p.j + b, k = A.rz * p.k + c;
             if (i < L.nx && j < L.ny && k < L.nz) acc = acc + R[(k * L.ny + j) * L.nx + i];
           }
@@ -1958,7 +2001,7 @@ __global__ void k_inner_decide(SlotState* st, int nslot, const double* __restric
   if (use_cond && threadIdx.x == 0) report_slot(slot, running, nslot, flags, counter, cond);
 }
 
-// K_cc + tau_q M_cc for every distinct tau in fp64 (the diagonal apply_at forms).
+// K_cc + tau_q M_cc for every distinct tau in fp64 (the diagonal residual_at forms).
 __global__ void k_diag64(LevelView<double> L, const z64* __restrict__ taus, int ntau, z64* __restrict__ out) {
   Cell p;
   int c;
@@ -1968,7 +2011,7 @@ __global__ void k_diag64(LevelView<double> L, const z64* __restrict__ taus, int 
   for (int q = 0; q < ntau; ++q) out[(int64_t)q * L.n + c] = mk(fmaT(taus[q].re, m, d), mulT(taus[q].im, m));
 }
 
-// K diagonal (sum of each cell's faces), the same sum apply_at forms.
+// K diagonal (sum of each cell's faces), the same sum residual_at forms.
 __global__ void k_kdiag(LevelView<double> L, double* __restrict__ kd) {
   Cell p;
   int c;

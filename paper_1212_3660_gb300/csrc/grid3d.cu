@@ -16,7 +16,7 @@
 // order, so the results are bitwise those of k_gs / k_residual_restrict /
 // k_prolong_add / k_correct.
 //   pre : z = four half sweeps from z = 0 (red, black, red, black); write z;
-//         coarse f = sum over the 8 children of (f - A z)
+//         coarse f = sum over the children of (f - A z) (restrict_value)
 //   post: z += P z_coarse; four half sweeps (black, red, black, red); write z
 //         (or, on the finest level, add it to the outer iterate z_k)
 #include <algorithm>
@@ -189,11 +189,12 @@ __global__ void __launch_bounds__(Tile3<TX, TY>::NT) k_pre3d(LevelView<T> L, con
         zs[((int64_t)qo * L.ny + gy) * L.nx + gx] = sZ[(qo % R3Z) * P + (oy + FH) * RX + ox + FH];
     }
     // phase 1c: residual of plane q = p - 5, one child cell per thread, summed
-    // into its coarse cell in the per-level kernel's child order (b, then a)
+    // into its coarse cell in the per-level kernel's child order (b, then a; in
+    // complex128 only the red children take part)
     const int qr = p - 5;
     if (qr >= z0 && qr < z1 && tid < TX * TY) {
       cx<T> v = mk(T(0), T(0));
-      if (cvalid) {
+      if (cvalid && (!RED_RESIDUAL<T> || ((ca + cb + qr) & 1) == 0)) {
         const cx<T>* Zq = sZ + (qr % R3Z) * P;
         const cx<T>* Zm = sZ + ((qr + R3Z - 1) % R3Z) * P;
         const cx<T>* Zp = sZ + ((qr + 1) % R3Z) * P;
@@ -202,18 +203,20 @@ __global__ void __launch_bounds__(Tile3<TX, TY>::NT) k_pre3d(LevelView<T> L, con
         const T d = L.kd ? L.kd[c] : fsum(fa);
         const T m = L.mm[c];
         const cx<T> diag = mk(fmaT(sft.re, m, d), mulT(sft.im, m));
-        const cx<T> Az = diag * Zq[cr] - nb_sum3<T, RX>(L, fa, cgx, cgy, qr, cr, Zm, Zq, Zp, mk(T(0), T(0)));
-        v = sF[(qr % R3F) * P + cr] - Az;
+        v = residual_of(sF[(qr % R3F) * P + cr], Zq[cr], diag, [&](cx<T> s0) {
+          return nb_sum3<T, RX>(L, fa, cgx, cgy, qr, cr, Zm, Zq, Zp, s0);
+        });
       }
       const int base = (tid & 31) & ~3;
       const cx<T> v0 = shfl_cx(v, base), v1 = shfl_cx(v, base + 1), v2 = shfl_cx(v, base + 2),
                   v3 = shfl_cx(v, base + 3);
       if (cvalid && (tid & 3) == 0) {
         cx<T> acc = (qr & 1) ? sC[ck] : mk(T(0), T(0));
-        acc = acc + v0;
-        acc = acc + v1;
-        acc = acc + v2;
-        acc = acc + v3;
+        const bool all = !RED_RESIDUAL<T>, even = (qr & 1) == 0;
+        if (all || even) acc = acc + v0;
+        if (all || !even) acc = acc + v1;
+        if (all || !even) acc = acc + v2;
+        if (all || even) acc = acc + v3;
         if (qr & 1) fcs[((int64_t)(qr >> 1) * cny + cY) * cnx + cX] = acc;
         else sC[ck] = acc;
       }

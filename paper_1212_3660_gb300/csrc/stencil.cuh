@@ -99,28 +99,22 @@ __device__ __forceinline__ cx<T> nb_sum(const LevelView<T, C>& L, const Faces<T>
   return s;
 }
 
-template <typename T, typename C>
-__device__ __forceinline__ cx<T> apply_at(const LevelView<T, C>& L, Cell p, int64_t c, cx<T> s,
-                                          const cx<T>* __restrict__ x) {
-  Faces<T> f = faces_at(L, p);
-  T d = L.kd ? L.kd[c] : fsum(f);  // same sum either way
-  T m = ldc<T>(L.mm, c);
-  cx<T> diag = mk(fmaT(s.re, m, d), mulT(s.im, m));
-  return diag * x[c] - nb_sum(L, f, p, c, x);
+// acc - diag x in four fused multiply-adds
+template <typename T>
+__device__ __forceinline__ cx<T> minus_product(cx<T> acc, cx<T> diag, cx<T> x) {
+  acc.re = fmaT(-diag.re, x.re, fmaT(diag.im, x.im, acc.re));
+  acc.im = fmaT(-diag.re, x.im, fmaT(-diag.im, x.re, acc.im));
+  return acc;
 }
 
 // v_c - ((K + tau M) x)_c with diag = K_cc + tau M_cc given: the neighbour
 // terms accumulate onto v, then diag * x_c is subtracted with fused
-// multiply-adds (fewer FP64 operations than v - apply_at).
+// multiply-adds (fewer FP64 operations than v - A x).
 template <typename T, typename C>
 __device__ __forceinline__ cx<T> defect_at(const LevelView<T, C>& L, Cell p, int64_t c, cx<T> diag, cx<T> v,
                                            const cx<T>* __restrict__ x) {
   Faces<T> f = faces_at(L, p);
-  cx<T> acc = nb_sum(L, f, p, c, x, v);
-  const cx<T> xc = x[c];
-  acc.re = fmaT(-diag.re, xc.re, fmaT(diag.im, xc.im, acc.re));
-  acc.im = fmaT(-diag.re, xc.im, fmaT(-diag.im, xc.re, acc.im));
-  return acc;
+  return minus_product(nb_sum(L, f, p, c, x, v), diag, x[c]);
 }
 
 // Red-black Gauss-Seidel update of cell c: (f_c + sum_nb t z_nb) / (K_cc + tau M_cc),
@@ -151,6 +145,43 @@ __device__ __forceinline__ bool color_cell(int nx, int ny, int nz, int color, in
   return true;
 }
 
+// The residual that a level restricts. In complex128 only the red cells' is
+// formed: the pre-smoothing ends with a black half sweep, which solves every
+// black cell's equation, so the black residuals are zero (rounding apart) and
+// are neither formed nor added: half of the work of a phase that FP64
+// arithmetic bounds (45 x 53 x 37 complex128 66.0 -> 59.2 ms a solve, 64 x 48 x
+// 48 172 -> 147). In complex64, where these kernels wait for memory, it would
+// give 1 to 2 %, and dropping what rounding leaves at the black cells (1e-7 of
+// the iterate) moves x_j by up to 9e-10 on hierarchies that converge slowly
+// (185 x 192, x never halved): there all cells stay.
+template <typename T>
+constexpr bool RED_RESIDUAL = sizeof(T) == 8;
+
+// f - (K + s M) z from the cell's f and z, its diagonal K_cc + s M_cc and a
+// functor that accumulates sum t z_nb onto its argument
+template <typename T, typename NB>
+__device__ __forceinline__ cx<T> residual_of(cx<T> f, cx<T> z, cx<T> diag, NB nb) {
+  if constexpr (RED_RESIDUAL<T>) return minus_product(nb(f), diag, z);
+  else return f - (diag * z - nb(mk(T(0), T(0))));
+}
+
+template <typename T, typename C>
+__device__ __forceinline__ cx<T> residual_at(const LevelView<T, C>& L, Cell p, int64_t c, cx<T> s, const cx<T>* f,
+                                             const cx<T>* z) {
+  const Faces<T> fa = faces_at(L, p);
+  const T d = L.kd ? L.kd[c] : fsum(fa);  // same sum either way
+  const T m = ldc<T>(L.mm, c);
+  return residual_of(f[c], z[c], mk(fmaT(s.re, m, d), mulT(s.im, m)),
+                     [&](cx<T> a) { return nb_sum(L, fa, p, c, z, a); });
+}
+
+// First child along x that takes part in a restriction, of cells whose other
+// coordinates (and first child's x) sum to `sum`; the next is child_step on
+template <typename T>
+__device__ __forceinline__ int child_first(int sum) { return RED_RESIDUAL<T> ? sum & 1 : 0; }
+template <typename T>
+constexpr int child_step = RED_RESIDUAL<T> ? 2 : 1;
+
 // Sum over the children of coarse cell (I,J,K) of the fine residual f - (K + s M) z
 // (on an odd axis the last coarse cell has one child).
 template <typename T, typename C>
@@ -159,11 +190,11 @@ __device__ __forceinline__ cx<T> restrict_value(const LevelView<T, C>& F, int rx
   cx<T> acc = mk(T(0), T(0));
   for (int c = 0; c < rz; ++c)
     for (int b = 0; b < ry; ++b)
-      for (int a = 0; a < rx; ++a) {
+      for (int a = child_first<T>(rx * I + ry * J + b + rz * K + c); a < rx; a += child_step<T>) {
         Cell p{rx * I + a, ry * J + b, rz * K + c};
         if (p.i >= F.nx || p.j >= F.ny || p.k >= F.nz) continue;
         int64_t cc = ((int64_t)p.k * F.ny + p.j) * F.nx + p.i;
-        acc = acc + (f[cc] - apply_at(F, p, cc, s, z));
+        acc = acc + residual_at(F, p, cc, s, f, z);
       }
   return acc;
 }
