@@ -630,6 +630,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     return zs ? ns * L.n * 1.5 * cv : ns * L.n * (2 * cv + d * rv);
   };
   auto smooth_f = [&](const LevelHost& L, int zs) { return zs ? ns * L.n * 3.0 : ns * L.n * 0.5 * (8 * d + 6); };
+  const double rr = sizeof(VT) == 8 ? 0.5 : 1.0;  // part of the cells whose residual is formed (RED_RESIDUAL)
   const int64_t fmax = S.op->fuse_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t16 = S.op->tile16_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t8 = S.op->tile8_max[sizeof(VT) == 8 ? 0 : 1];
@@ -641,14 +642,14 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     const LevelHost& L = Ls[l];
     if (fused_level_ok(L) && L.n * nsl <= fmax) {
       PROF(FKS_K_PRE2D, l, ns * (L.n * (3 * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
-           ns * L.n * (2 * (8 * d + 6) + 4 * d + 5),
+           ns * L.n * (2 * (8 * d + 6) + rr * (8 * d + 10)),
            launch_pre2d<VT>(L, Ls[l + 1], S.st, I(l), S.taus, F(l), Zl(l), L.n, F(l + 1), Ls[l + 1].n, S.nslot,
                             tile_of(L), s));
       continue;
     }
     if (fused3d_level_ok(L) && L.n * nsl <= fmax) {
       PROF(FKS_K_PRE3D, l, ns * (L.n * (3 * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
-           ns * L.n * (2 * (8 * d + 6) + 4 * d + 5),
+           ns * L.n * (2 * (8 * d + 6) + rr * (8 * d + 10)),
            launch_pre3d<VT>(L, S.st, I(l), S.taus, F(l), Zl(l), L.n, F(l + 1), Ls[l + 1].n, S.nslot, tile_of(L),
                             S.op->zchunk[pix][l], s));
       continue;
@@ -660,7 +661,8 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
         PROF(FKS_K_SMOOTH, l, smooth_b(L, r == 0) + smooth_b(L, 0), smooth_f(L, r == 0) + smooth_f(L, 0),
              launch_sweep3<VT>(L, nullptr, 0, r == 0 ? SWEEP_ZERO : 0, S.st, I(l), F(l), Zl(l), r == 0 ? Zl(l) : z2,
                                L.n, nullptr, S.nslot, 0, nullptr, 0, 0, bf, s));
-      PROF(FKS_K_RESTRICT, l, ns * (L.n * (1.5 * cv + (d + 1) * rv) + cv * Ls[l + 1].n), ns * L.n * (4 * d + 5),
+      PROF(FKS_K_RESTRICT, l, ns * (L.n * ((1 + rr) * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
+           ns * L.n * rr * (8 * d + 10),
            launch_residual_restrict<VT>(L, Ls[l + 1], S.st, S.taus, F(l), z2, L.n, F(l + 1), Ls[l + 1].n, S.nslot, s,
                                         bf));
       continue;
@@ -672,7 +674,8 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
       PROF(FKS_K_SMOOTH, l, smooth_b(L, 0), smooth_f(L, 0),
            launch_gs<VT>(L, S.st, I(l), F(l), Zl(l), L.n, S.nslot, 1, 0, s, nullptr, 0, 0, bf));
     }
-    PROF(FKS_K_RESTRICT, l, ns * (L.n * (1.5 * cv + (d + 1) * rv) + cv * Ls[l + 1].n), ns * L.n * (4 * d + 5),
+    PROF(FKS_K_RESTRICT, l, ns * (L.n * ((1 + rr) * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
+           ns * L.n * rr * (8 * d + 10),
          launch_residual_restrict<VT>(L, Ls[l + 1], S.st, S.taus, F(l), Zl(l), L.n, F(l + 1), Ls[l + 1].n, S.nslot,
                                       s, bf));
   }

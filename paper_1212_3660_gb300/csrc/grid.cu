@@ -259,19 +259,21 @@ __global__ void __launch_bounds__(GX * GY) k_apply(LevelView<double> L, z64 s, c
 template <typename T, typename C>
 __global__ void k_gs(LevelView<T, C> L, const SlotState* st, const cx<T>* __restrict__ invd,
                      const cx<T>* __restrict__ f, cx<T>* __restrict__ z, int64_t vs, int color, int zero_start,
-                     int nslot) {
+                     int nslot, unsigned mny) {
   pdl_enter();
   const int slot = blockIdx.z * blockDim.z + threadIdx.z;
   if (slot >= nslot || !slot_running(st, slot)) return;
   const int ii = blockIdx.x * GX + threadIdx.x;
   const int row = blockIdx.y * blockDim.y + threadIdx.y;
   if (row >= L.ny * L.nz) return;
-  const int k = row / L.ny, j = row - k * L.ny;
+  int j, k;
+  split_row(row, L.ny, mny, &j, &k);
   const int i = 2 * ii + ((j + k + color) & 1);
   if (i >= L.nx) return;
   const int c = row * L.nx + i;
   const cx<T> id = invd[(int64_t)st[slot].tau * L.n + c];
-  z[slot * vs + c] = gs_value(L, Cell{i, j, k}, c, id, f + slot * vs, z + slot * vs, zero_start);
+  cx<T>* zs = z + slot * vs;
+  zs[c] = gs_row(L, Cell{i, j, k}, row, c, id, f + slot * vs, (const cx<T>*)zs, zero_start);
 }
 
 // The last half sweep of the finest level's post-smoothing fused with the
@@ -283,31 +285,30 @@ __global__ void k_gs(LevelView<T, C> L, const SlotState* st, const cx<T>* __rest
 template <typename T, typename C>
 __global__ void k_gs_correct(LevelView<T, C> L, const SlotState* st, const cx<T>* __restrict__ invd,
                              const cx<T>* __restrict__ f, const cx<T>* __restrict__ z, int64_t vs, int color,
-                             z64* __restrict__ Zk, int64_t vsZk, int64_t zcol, int nslot) {
+                             z64* __restrict__ Zk, int64_t vsZk, int64_t zcol, int nslot, unsigned mny) {
   pdl_enter();
   const int slot = blockIdx.z * blockDim.z + threadIdx.z;
   if (slot >= nslot || !slot_running(st, slot)) return;
   const int ii = blockIdx.x * GX + threadIdx.x;
   const int row = blockIdx.y * blockDim.y + threadIdx.y;
   if (row >= L.ny * L.nz || 2 * ii >= L.nx) return;
-  const int k = row / L.ny, j = row - k * L.ny;
+  int j, k;
+  split_row(row, L.ny, mny, &j, &k);
+  const int c0 = row * L.nx + 2 * ii, h = (j + k + color) & 1, i = 2 * ii + h, c = c0 + h;
   const cx<T>* zs = z + slot * vs;
-  z64* zk = Zk + slot * vsZk + (int64_t)(st[slot].k - 1) * zcol;
-  const bool first = st[slot].cycles == 0;
-  for (int h = 0; h < 2; ++h) {
-    const int i = 2 * ii + h;
-    if (i >= L.nx) break;
-    const int c = row * L.nx + i;
-    cx<T> e;
-    if (((i + j + k) & 1) == color) {
-      const cx<T> id = invd[(int64_t)st[slot].tau * L.n + c];
-      e = gs_value(L, Cell{i, j, k}, c, id, f + slot * vs, zs, 0);
-    } else {
-      e = zs[c];
-    }
-    const z64 ev = cvt<double>(e);
-    zk[c] = first ? ev : (zk[c] + ev);
+  z64* zk = Zk + slot * vsZk + (int64_t)(st[slot].k - 1) * zcol + c0;
+  const bool first = st[slot].cycles == 0, two = 2 * ii + 1 < L.nx;
+  const z64 none = mk(0.0, 0.0);
+  const z64 o0 = first ? none : zk[0], o1 = first || !two ? none : zk[1];
+  cx<T> v = mk(T(0), T(0)), w = v;  // the updated cell, the other
+  if (h == 1 || two) w = zs[c0 + 1 - h];
+  if (i < L.nx) {
+    const cx<T> id = invd[(int64_t)st[slot].tau * L.n + c];
+    v = gs_row(L, Cell{i, j, k}, row, c, id, f + slot * vs, zs, 0);
   }
+  const z64 e0 = cvt<double>(h ? w : v), e1 = cvt<double>(h ? v : w);
+  zk[0] = first ? e0 : (o0 + e0);
+  if (two) zk[1] = first ? e1 : (o1 + e1);
 }
 
 // --------------------------------------------------------------------- transfer
@@ -361,8 +362,8 @@ __global__ void __launch_bounds__(256) k_residual_restrict3(LevelView<T, C> F, i
     const int k = 2 * K + (NP == 1 ? (i + j) & 1 : q);
     cx<T> r = mk(T(0), T(0));
     if (i < F.nx && j < F.ny && k < F.nz) {
-      const int64_t cc = ((int64_t)k * F.ny + j) * F.nx + i;
-      r = residual_at(F, Cell{i, j, k}, cc, s, fs, zs);
+      const int row = k * F.ny + j, c = row * F.nx + i;
+      r = residual_row(F, Cell{i, j, k}, row, c, s, fs, zs);
     }
     sr[q][threadIdx.y][threadIdx.x] = r;
   }
@@ -2121,22 +2122,23 @@ void launch_gs(const LevelHost& L, const SlotState* st, const cx<T>* invd, const
                int nslot, int color, int zero_start, cudaStream_t s, z64* Zk, int64_t vsZk, int64_t zcol, int bf16) {
   const int G = spmm_group(nslot), rb = GY / G;
   const dim3 blk(GX, rb, G), grd(nb((L.nx + 1) / 2, GX), nb((int64_t)L.ny * L.nz, rb), nb(nslot, G));
+  const unsigned mny = row_magic(L.ny);
   if constexpr (sizeof(T) == 4) {
     if (bf16) {
       if (Zk)
         launch_pdl(k_gs_correct<T, __nv_bfloat16>, grd, blk, 0, s, view_as<T, __nv_bfloat16>(L), st, invd, f, z, vs, color,
-                                                           Zk, vsZk, zcol, nslot);
+                                                           Zk, vsZk, zcol, nslot, mny);
       else
         launch_pdl(k_gs<T, __nv_bfloat16>, grd, blk, 0, s, view_as<T, __nv_bfloat16>(L), st, invd, f, z, vs, color,
-                                                   zero_start, nslot);
+                                                   zero_start, nslot, mny);
       return;
     }
   }
   if (Zk) {
-    launch_pdl(k_gs_correct<T, T>, grd, blk, 0, s, view<T>(L), st, invd, f, z, vs, color, Zk, vsZk, zcol, nslot);
+    launch_pdl(k_gs_correct<T, T>, grd, blk, 0, s, view<T>(L), st, invd, f, z, vs, color, Zk, vsZk, zcol, nslot, mny);
     return;
   }
-  launch_pdl(k_gs<T, T>, grd, blk, 0, s, view<T>(L), st, invd, f, z, vs, color, zero_start, nslot);
+  launch_pdl(k_gs<T, T>, grd, blk, 0, s, view<T>(L), st, invd, f, z, vs, color, zero_start, nslot, mny);
 }
 
 template <typename T>
