@@ -580,6 +580,15 @@ static TailPlan tail_plan(const std::vector<LevelHost>& Ls, int lt) {
   return t;
 }
 
+// The tail's way down and way up as two launches around the coarsest product
+// over the chip: in complex128 by pairs, from the size on where one SM's FP64
+// time for the product is above that of the two launches (105 cells: a cycle of
+// 45 x 53 x 37 168 us whole, 149 split; at 64 both take 8)
+template <typename VT>
+static bool tail_split(const TailPlan& t, int nc, int nlev) {
+  return sizeof(VT) == 8 && t.roff && t.threads == 512 && nlev > 1 && nc > COARSE_ALONE;
+}
+
 // Bytes per tau of the tail's staged coefficients and their shared-memory
 // offset (0 bytes when the tail reads its coefficients from global memory).
 template <typename VT>
@@ -747,6 +756,8 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
       T.invd = I(l);
       T.off = off;
       T.cbyte = cbyte[l];
+      T.gf = F(l);
+      T.gz = Zl(l);
       off += 2 * (int)Ls[l].n;
       tb += Ls[l].n * (8 * cv + d * rv);
       tf += Ls[l].n * (8 * d + 6) * 4;
@@ -769,7 +780,15 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
     P.roff = tp.roff;
     P.rlen = tp.rlen;
     P.threads = tp.threads;
-    PROF(FKS_K_TAIL, lt, ns * tb, ns * tf, launch_tail<VT>(P, tp.smem, S.st, S.nslot, s));
+    if (tail_split<VT>(tp, P.nc, P.nlev)) {
+      const double nc = (double)P.nc, cb = cv * nc * nc, cf = 8.0 * nc * nc;
+      PROF(FKS_K_TAIL, lt, ns * (tb - cb) / 2, ns * (tf - cf) / 2, launch_tail<VT>(P, tp.smem, S.st, S.nslot, s, 1));
+      PROF(FKS_K_COARSE, nl - 1, ns * (cb + 2 * cv * nc), ns * cf,
+           launch_coarse_solve<VT>(P.Ainv, P.nc, S.st, F(nl - 1), Zl(nl - 1), P.nc, S.nslot, s));
+      PROF(FKS_K_TAIL, lt, ns * (tb - cb) / 2, ns * (tf - cf) / 2, launch_tail<VT>(P, tp.smem, S.st, S.nslot, s, 2));
+    } else {
+      PROF(FKS_K_TAIL, lt, ns * tb, ns * tf, launch_tail<VT>(P, tp.smem, S.st, S.nslot, s));
+    }
   }
   cx<VT>* zfin = Zl(lp);  // final correction of the level below
   for (int l = lp - 1; l >= 0; --l) {

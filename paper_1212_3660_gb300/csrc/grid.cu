@@ -1220,6 +1220,11 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail2d(TailParams<T> P, con
 // restrict_value's order; the coarsest product's terms are formed by all
 // threads (from coalesced reads, the inverse being transposed) and added per
 // row in order: the bits are k_tail_vcycle's.
+// PART 1 and 2 are its way down and its way up, with k_coarse_solve between
+// them. In complex128 one SM's FP64 units take 17 us for the product of a
+// coarsest level of 105 cells (11 for the terms, 7 for the sums; 30 us the whole
+// tail of 45 x 53 x 37), more than two launches and the product over the chip
+// (6.4 + 6.5 + 5.5 us).
 template <typename T>
 struct PairCell {  // the pair's coefficients: x faces left, inside, right; y and z faces below and above each cell
   T x[3], yl[2], yh[2], zl[2], zh[2], m[2];
@@ -1292,7 +1297,7 @@ __device__ __forceinline__ void pair_gs(PairCell<T>& q, const LevelView<T>& L, c
   Z[q.c0 + h] = v;
 }
 
-template <typename T, int NT>
+template <typename T, int NT, int PART = 0>
 __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const SlotState* st) {
   pdl_enter();
   const int slot = blockIdx.x;
@@ -1304,7 +1309,7 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
   const cx<T> sft = cvt<T>(P.taus[tau]);
   const cx<T> none = mk(T(0), T(0));
   PairCell<T> q;
-  {
+  if (PART != 2) {
     const TailLevel<T>& A = P.lev[0];
     const cx<T>* fin = P.f_in + slot * P.vs;
     if (P.nlev > 1) {
@@ -1317,7 +1322,7 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
       for (int c = t; c < A.L.n; c += NT) sh[A.off + c] = fin[c];
     }
   }
-  for (int l = 0; l + 1 < P.nlev; ++l) {
+  for (int l = 0; PART != 2 && l + 1 < P.nlev; ++l) {
     const TailLevel<T>& A = P.lev[l];
     const TailLevel<T>& B = P.lev[l + 1];
     const LevelView<T>& L = A.L;
@@ -1333,6 +1338,10 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
     __syncthreads();
     pair_gs(q, L, Z, 1, false);
     __syncthreads();
+    if (PART == 1 && q.own) {
+      const int h = (q.j + q.k) & 1;  // the way up reads the red cells alone
+      if (h == 0 || q.right) A.gz[(int64_t)slot * L.n + q.c0 + h] = h ? q.z[1] : q.z[0];
+    }
     constexpr int NC = RED_RESIDUAL<T> ? 1 : 2;  // the pair's red cell, or both
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
@@ -1357,10 +1366,12 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
             if (i < L.nx && j < L.ny && k < L.nz) acc = acc + R[(k * L.ny + j) * L.nx + i];
           }
       FC[C] = acc;
+      if (PART == 1) B.gf[(int64_t)slot * B.L.n + C] = acc;
     }
     __syncthreads();
   }
-  {
+  if (PART == 1) return;
+  if (PART == 0) {
     const TailLevel<T>& Cl = P.lev[P.nlev - 1];
     const cx<T>* F = sh + Cl.off;
     cx<T>* Z = sh + Cl.off + Cl.L.n;
@@ -1395,14 +1406,13 @@ __global__ void __launch_bounds__(NT, 1) k_tail_pairs(TailParams<T> P, const Slo
     const TailLevel<T>& A = P.lev[l];
     const TailLevel<T>& B = P.lev[l + 1];
     const LevelView<T>& L = A.L;
-    cx<T>* F = sh + A.off;
-    cx<T>* Z = F + L.n;
-    const cx<T>* ZC = sh + B.off + B.L.n;
-    pair_load(A, tau, F, t, q);
+    cx<T>* Z = sh + A.off + L.n;
+    const cx<T>* ZC = PART == 2 && l == P.nlev - 2 ? B.gz + (int64_t)slot * B.L.n : sh + B.off + B.L.n;
+    pair_load(A, tau, PART == 2 ? A.gf + (int64_t)slot * L.n : sh + A.off, t, q);
     q.z[0] = q.z[1] = none;
     const int h = (q.j + q.k) & 1;  // the red cell: the black one is overwritten unread
     if (q.own && (h == 0 || q.right)) {
-      const cx<T> v = Z[q.c0 + h] +
+      const cx<T> v = (PART == 2 ? A.gz + (int64_t)slot * L.n : Z)[q.c0 + h] +
                       prolong_value(Cell{q.i0 + h, q.j, q.k}, A.rx, A.ry, A.rz, B.L.nx, B.L.ny, B.L.nz, P.mask, ZC);
       if (h) q.z[1] = v;
       else q.z[0] = v;
@@ -2248,6 +2258,10 @@ void tail_prepare(size_t smem_bytes) {
   cudaFuncSetAttribute(k_tail_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_tail2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_tail_pairs<T, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  if constexpr (sizeof(T) == 8) {
+    cudaFuncSetAttribute(k_tail_pairs<T, 512, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaFuncSetAttribute(k_tail_pairs<T, 512, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  }
   if constexpr (sizeof(T) == 4)
     cudaFuncSetAttribute(k_tail_pairs<T, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2255,8 +2269,13 @@ void tail_prepare(size_t smem_bytes) {
 }
 
 template <typename T>
-void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s) {
-  if (P.pairs)
+void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s, int part) {
+  if (part) {
+    if constexpr (sizeof(T) == 8) {
+      if (part == 1) launch_pdl(k_tail_pairs<T, 512, 1>, nslot, 512, smem_bytes, s, P, st);
+      else launch_pdl(k_tail_pairs<T, 512, 2>, nslot, 512, smem_bytes, s, P, st);
+    }
+  } else if (P.pairs)
     launch_pdl(k_tail2d<T>, nslot, TAIL_THREADS, smem_bytes, s, P, st);
   else if (P.roff && P.threads == 512)
     launch_pdl(k_tail_pairs<T, 512>, nslot, 512, smem_bytes, s, P, st);
@@ -2348,7 +2367,7 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
                                  const cx<T>*, const cx<T>*, cx<T>*, int64_t, const cx<T>*, int64_t, int, int,    \
                                  cudaStream_t, z64*, int64_t, int64_t);                                           \
   template void tail_prepare<T>(size_t);                                                                          \
-  template void launch_tail<T>(const TailParams<T>&, size_t, const SlotState*, int, cudaStream_t);                \
+  template void launch_tail<T>(const TailParams<T>&, size_t, const SlotState*, int, cudaStream_t, int);                \
   template void launch_invd<T>(const LevelHost&, const z64*, int, cx<T>*, cudaStream_t, int);                     \
   template void launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \
                                          int);                                                                    \

@@ -17,6 +17,8 @@ struct TailLevel {
   const cx<T>* invd;       // [n_tau][n] inverse diagonals
   int off;
   int cbyte;               // byte offset of this level's coefficients staged in shared memory
+  cx<T>* gf;               // the level's vectors in device memory (a source's stride n),
+  cx<T>* gz;               // for the tail in two launches
 };
 
 template <typename T>
@@ -73,7 +75,7 @@ void launch_post3d(const LevelHost& F, uint32_t mask, const SlotState* st, const
                    int zch, cudaStream_t s, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zcol = 0);
 // P.pairs selects the register-resident 2D kernel (same results)
 template <typename T>
-void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s);
+void launch_tail(const TailParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot, cudaStream_t s, int part = 0);
 // block size of the pair-per-thread tail of levels lt .. coarsest (0: too large for it)
 int tail_pairs_threads(const std::vector<LevelHost>& Ls, int lt, bool fp64);
 // whether levels lt .. coarsest qualify for the register-resident 2D tail
