@@ -555,7 +555,7 @@ static TailPlan tail_plan(const std::vector<LevelHost>& Ls, int lt) {
   TailPlan t;
   t.smem = tail_smem<VT>(Ls, lt);
   const size_t nc = (size_t)Ls.back().n;
-  if (tail_staged<VT>(Ls, lt) && tail2d_ok(Ls, lt)) {
+  if (tail_staged<VT>(Ls, lt) && tail2d_ok(Ls, lt) && !coarse_in_parts<VT>((int)nc)) {  // (those split, tail_split)
     const size_t a = (t.smem + 15) & ~(size_t)15;
     const size_t b2 = a + nc * nc * sizeof(cx<VT>);
     if (b2 <= TAIL_SMEM_LIMIT) {

@@ -95,6 +95,17 @@ __host__ __device__ __forceinline__ T ldc(const C* p, int64_t i) {
   else return (T)p[i];
 }
 
+// ---------------------------------------------------------------- coarsest level
+// coarsest levels above this run in launch_coarse_solve when no other level is in the tail
+constexpr int COARSE_ALONE = 64;
+// Order of the coarsest product's sum over nc terms: one after another, or, in
+// complex128 above COARSE_ALONE cells, COARSE_PARTS interleaved partial sums,
+// added as (0 + 1) + (2 + 3): a dependent FP64 addition takes 72 clocks, and
+// 297 of them were 10.6 of k_coarse_solve's 14.7 us.
+constexpr int COARSE_PARTS = 4;
+template <typename T>
+__host__ __device__ constexpr bool coarse_in_parts(int nc) { return sizeof(T) == 8 && nc > COARSE_ALONE; }
+
 // ---------------------------------------------------------------- launch overlap
 // Programmatic dependent launch: a kernel launched by launch_pdl may be
 // scheduled while its predecessor in the stream is still running. It waits in

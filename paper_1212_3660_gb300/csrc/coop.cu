@@ -93,9 +93,7 @@ __global__ void __launch_bounds__(COOP_THREADS) k_coop_vcycle(CoopParams<T> P, c
       const int r = (int)(w - (int64_t)(slot - s0) * P.nc);
       const cx<T>* Ai = P.Ainv + (int64_t)st[slot].tau * P.nc * P.nc + r;
       const cx<T>* F = P.f[l] + (int64_t)slot * P.nc;
-      cx<T> acc = mk(T(0), T(0));
-      for (int q = 0; q < P.nc; ++q) acc = acc + Ai[q * P.nc] * F[q];
-      P.z[l][(int64_t)slot * P.nc + r] = acc;
+      P.z[l][(int64_t)slot * P.nc + r] = coarse_sum<T>(P.nc, [&](int q) { return Ai[q * P.nc] * F[q]; });
     }
     barrier();
   }

@@ -947,10 +947,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) k_tail_vcycle(TailParams<T> P
     cx<T>* Z = sh + Cl.off + Cl.L.n;
     const cx<T>* Ainv = P.Ainv + (int64_t)tau * P.nc * P.nc;
     for (int r = tid; r < P.nc; r += nt) {
-      cx<T> acc = mk(T(0), T(0));
-#pragma unroll 8
-      for (int l = 0; l < P.nc; ++l) acc = acc + Ainv[l * P.nc + r] * F[l];
-      Z[r] = acc;
+      Z[r] = coarse_sum<T>(P.nc, [&](int l) { return Ainv[l * P.nc + r] * F[l]; });
     }
     __syncthreads();
   }
@@ -1741,9 +1738,11 @@ __global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<
 
 // z = Ainv[tau] f on the coarsest level when it is a level of its own (Ainv
 // transposed): a block owns CS_BYTES / sizeof rows. All of its threads form the
-// products of those rows, from coalesced reads; then one thread per row adds
-// its products in the order of the tail kernels' loop, so the bits are theirs.
-// The single-block tail reads the n x n inverse through one SM.
+// products of those rows, from coalesced reads; then one warp adds each row's
+// products in the order of the tail kernels' loop (coarse_sum), so the bits are
+// theirs. Complex128 adds in partial sums (a solve of 18 x 22 x 24 cells, 297 of
+// them on the coarsest level, 57.5 -> 54.0 ms). The single-block tail reads the
+// n x n inverse through one SM.
 template <typename T>
 __global__ void __launch_bounds__(256) k_coarse_solve(const cx<T>* __restrict__ Ainv, int n, const SlotState* st,
                                                       const cx<T>* __restrict__ f, cx<T>* __restrict__ z,
@@ -1765,6 +1764,20 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const cx<T>* __restrict__ 
   __syncthreads();
   // two threads per row, one for each part of the complex sum
   const int t = threadIdx.x;
+  if constexpr (sizeof(T) == 8) {
+    if (coarse_in_parts<T>(n)) {  // a lane per partial sum as well (2 RB COARSE_PARTS = 32 lanes)
+      static_assert(2 * coarse_rows<double>() * COARSE_PARTS == 32, "one warp adds");
+      if (t >= 32) return;
+      const int e = t % (2 * RB);
+      T acc = T(0);
+#pragma unroll 16
+      for (int l = t / (2 * RB); l < n; l += COARSE_PARTS) acc = acc + ((const T*)pr)[2 * l * RB + e];
+      acc = acc + __shfl_xor_sync(0xffffffffu, acc, 2 * RB);
+      acc = acc + __shfl_xor_sync(0xffffffffu, acc, 4 * RB);
+      if (t < 2 * RB && r0 + e / 2 < n) ((T*)(z + slot * vs + r0))[e] = acc;
+      return;
+    }
+  }
   if (t >= 2 * RB || r0 + t / 2 >= n) return;
   T acc = T(0);
 #pragma unroll 16

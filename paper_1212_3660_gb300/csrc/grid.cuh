@@ -132,8 +132,6 @@ void launch_prolong_add(const LevelHost& F, const LevelHost& C, uint32_t mask, c
 // rows per block of the coarsest product on its own: 64 KB of products at 1024 unknowns
 template <typename T>
 constexpr int coarse_rows() { return sizeof(T) == 8 ? 4 : 8; }
-// coarsest levels above this run in launch_coarse_solve when no other level is in the tail
-constexpr int COARSE_ALONE = 64;
 template <typename T>
 void launch_coarse_solve(const cx<T>* Ainv, int n, const SlotState* st, const cx<T>* f, cx<T>* z, int64_t vs,
                          int nslot, cudaStream_t s);

@@ -285,6 +285,23 @@ __device__ __forceinline__ cx<T> restrict_value(const LevelView<T, C>& F, int rx
   return acc;
 }
 
+template <typename T, typename Term>
+__device__ __forceinline__ cx<T> coarse_sum(int nc, Term term) {
+  cx<T> a[COARSE_PARTS];
+#pragma unroll
+  for (int p = 0; p < COARSE_PARTS; ++p) a[p] = mk(T(0), T(0));
+  if (!coarse_in_parts<T>(nc)) {
+#pragma unroll 8
+    for (int l = 0; l < nc; ++l) a[0] = a[0] + term(l);
+    return a[0];
+  }
+  for (int l = 0; l < nc; l += COARSE_PARTS)
+#pragma unroll
+    for (int p = 0; p < COARSE_PARTS; ++p)
+      if (l + p < nc) a[p] = a[p] + term(l + p);
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
 // a positive normal float as T (exact), without the FP64 pipe
 template <typename T>
 __device__ __forceinline__ T widen(float w) {

@@ -1,6 +1,7 @@
 """The tail in two launches around the coarsest product (complex128, a coarsest
 level above 64 cells): bit for bit the per-level kernels' V-cycle, one level and
-several, at the first size that splits, for one source and for a batch."""
+several, at the first size that splits, for one source and for a batch; also
+the cooperative lower cycle's, and the single-block tail's where pairs do not fit."""
 import numpy as np
 import pytest
 
@@ -14,7 +15,8 @@ pytestmark = pytest.mark.gpu
 P = fks.FKS_PREC_FP64
 
 
-@pytest.mark.parametrize("shape", [(9, 20, 14), (7, 20, 16), (13, 40), (8, 13, 20)])
+@pytest.mark.parametrize("shape", [(9, 20, 14), (7, 20, 16), (13, 40), (8, 13, 20), (8, 42),
+                                   (24, 21, 4)])
 def test_split_tail_equals_level_kernels(shape):
     need_gpu()
     pr = synth.make_problem(shape, n_f=4, periods=(5.0, 3600.0), n_p=2, seed=53)
@@ -23,13 +25,15 @@ def test_split_tail_equals_level_kernels(shape):
     v = rng.standard_normal(pr.n) + 1j * rng.standard_normal(pr.n)
     b = rng.standard_normal((3, pr.n)) + 0j
     out = []
-    for tail in (1, 1024):
+    for tail, coop in ((1, 0), (1024, 0), (4096, 0), (1, 1 << 30)):
         fks.fks_op_set_tail(s.op, P, tail)
+        fks.fks_op_set_coop(s.op, P, coop)
         z = np.zeros(pr.n, np.complex128)
         fks.fks_precond_apply(s.op, complex(pr.tau_bar[0]), v, z, 1e-10, cycles=2, precision=P)
         x = s.solve(b=b, precision=P, inner_tol=1e-6).X
         out.append((z, np.asarray(x)))
     s.close()
     assert np.isfinite(out[0][0]).all() and np.abs(out[0][1]).max() > 0
-    for a, c in zip(*out):
-        assert np.array_equal(a, c)
+    for other in out[1:]:
+        for a, c in zip(out[0], other):
+            assert np.array_equal(a, c)
