@@ -294,19 +294,20 @@ struct fks_op {
   // complex64 cycles; fks_op_grid sets a 3D operator's, fks_op_autotune and
   // the fks_op_set_* calls change them), in cells of a launch (a level's times
   // the batch's sources). Fused tile kernels: in complex128 their recomputed
-  // halo costs FP64 time once a level fills the chip (1000^2 369 us a cycle per
-  // sweep, 417 fused; 512^2 fused), in complex64 they win throughout (2048^2
-  // 426 against 497 us).
+  // halo costs FP64 time once a level fills the chip (a cycle with the finest
+  // level per sweep and fused: 1000^2 327 and 351 us, 724^2 221 and 237, 512^2
+  // 176 and 170), in complex64 they win throughout (2048^2 434 us a cycle, no level
+  // fused 548).
   int64_t fuse_max[2] = {524288, INT64_MAX};
   // fused 2D levels with at most this many cells use 16 x 16 tiles (else 32 x
-  // 32: 2048^2 complex64 426 against 441 us a cycle, 1024^2 159 against 153)
+  // 32: 2048^2 complex64 424 against 434 us a cycle, 1024^2 140 against 169)
   int64_t tile16_max[2] = {524288, 2097152};
-  // ... and with at most this many, 8 x 8 tiles (289 x 311 complex64 62 against
-  // 66 us; complex128 256^2 18 + 16 against 12 + 10 us, 128^2 7 + 6 against 8 + 7)
+  // ... and with at most this many, 8 x 8 tiles (complex64 289 x 311 even;
+  // complex128 128^2 66 us a cycle against 84, 256^2 kernels 92 against 81)
   int64_t tile8_max[2] = {16384, 131072};
   // levels with at most this many cells run in the single-block tail kernel
-  // (64^2 complex128 65 us a cycle with 64, 70 with 256; 289 x 311 complex64
-  // 81 with 256, 66 with 1024)
+  // (64^2 complex128 even with 64 and 256; 289 x 311 complex64 73 us a cycle
+  // with 256, 60 with 1024 and 2048)
   int64_t tail_max[2] = {64, 2048};
   // Thresholds that the tuner or a program chose count a level's cells alone:
   // they are picked with one source, and with nine of them the 112 x 96 levels
@@ -582,11 +583,13 @@ static TailPlan tail_plan(const std::vector<LevelHost>& Ls, int lt) {
 
 // The tail's way down and way up as two launches around the coarsest product
 // over the chip: in complex128 by pairs, from the size on where one SM's FP64
-// time for the product is above that of the two launches (105 cells: a cycle of
-// 45 x 53 x 37 168 us whole, 149 split; at 64 both take 8)
+// time for the product is above that of the two launches (a cycle whole and
+// split: 105 cells of 45 x 53 x 37 170 and 150 us, 65 of 13 x 40 104 and 96, 60 of
+// 15 x 16 73 and 66; 45 of 24 x 24 x 20 and 36 of 64 x 48 x 48 even)
+constexpr int SPLIT_CELLS = 48;
 template <typename VT>
 static bool tail_split(const TailPlan& t, int nc, int nlev) {
-  return sizeof(VT) == 8 && t.roff && t.threads == 512 && nlev > 1 && nc > COARSE_ALONE;
+  return sizeof(VT) == 8 && t.roff && t.threads == 512 && nlev > 1 && nc > SPLIT_CELLS;
 }
 
 // Bytes per tau of the tail's staged coefficients and their shared-memory
@@ -2036,8 +2039,8 @@ fks_status fks_op_grid(fks_ctx* ctx, int dim, const int64_t ncell[3], const doub
     CK(cudaMemcpy(op->levels[0].d64[3], mass.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
     if (nz > 1) {
       // 3D: level kernels per half sweep or sweep instead of the z-march ones
-      // (128^3 complex64: 134 us against 305 on the finest level), a tail of up
-      // to 8^3 cells in complex128 (64^3: 230 us a cycle, 245 with 64)
+      // (128^3 complex64: 288 us a cycle against 725), a tail of up
+      // to 8^3 cells in complex128 (64^3: 197 us a cycle, 213 with 64)
       op->fuse_max[0] = op->fuse_max[1] = 0;
       op->tail_max[0] = 512;
     }

@@ -1,6 +1,6 @@
 """The tail in two launches around the coarsest product (complex128, a coarsest
-level above 64 cells): bit for bit the per-level kernels' V-cycle, one level and
-several, at the first size that splits, for one source and for a batch; also
+level above 48 cells): bit for bit the per-level kernels' V-cycle, one level and
+several, at 60 and 65 cells, for one source and for a batch; also
 the cooperative lower cycle's, and the single-block tail's where pairs do not fit."""
 import numpy as np
 import pytest
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 P = fks.FKS_PREC_FP64
 
 
-@pytest.mark.parametrize("shape", [(9, 20, 14), (7, 20, 16), (13, 40), (8, 13, 20), (8, 42),
+@pytest.mark.parametrize("shape", [(9, 20, 14), (7, 20, 16), (13, 40), (16, 15), (8, 13, 20), (8, 42),
                                    (24, 21, 4)])
 def test_split_tail_equals_level_kernels(shape):
     need_gpu()
