@@ -398,7 +398,7 @@ void fks_server_destroy(fks_server* srv);
  * cycle precision `precision` and shift `tau`, and keeps the fastest in the
  * operator for later solves; then, for that choice, which of the smallest fused
  * levels run on 8 x 8 tiles.
- * Before any tuning, 2D operators fuse levels up to 524288 cells (complex128
+ * Before any tuning, 2D operators fuse levels up to 393216 cells (complex128
  * cycles) or all levels (complex64 cycles), on 8 x 8 tiles up to 16384 or 131072
  * cells, 16 x 16 up to 524288 or 2097152, with a tail of at most 64 or 2048
  * cells; 3D operators fuse no level and use a tail of at most 512 or 2048 cells.

@@ -298,7 +298,7 @@ struct fks_op {
   // level per sweep and fused: 1000^2 327 and 351 us, 724^2 221 and 237, 512^2
   // 176 and 170), in complex64 they win throughout (2048^2 434 us a cycle, no level
   // fused 548).
-  int64_t fuse_max[2] = {524288, INT64_MAX};
+  int64_t fuse_max[2] = {393216, INT64_MAX};
   // fused 2D levels with at most this many cells use 16 x 16 tiles (else 32 x
   // 32: 2048^2 complex64 424 against 434 us a cycle, 1024^2 140 against 169)
   int64_t tile16_max[2] = {524288, 2097152};
