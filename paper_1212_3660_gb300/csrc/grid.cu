@@ -1737,7 +1737,7 @@ __global__ void __launch_bounds__(512) k_gj_small(const z64* __restrict__ A, cx<
 }
 
 // z = Ainv[tau] f on the coarsest level when it is a level of its own (Ainv
-// transposed): a block owns CS_BYTES / sizeof rows. All of its threads form the
+// transposed): a block owns coarse_rows rows. All of its threads form the
 // products of those rows, from coalesced reads; then one warp adds each row's
 // products in the order of the tail kernels' loop (coarse_sum), so the bits are
 // theirs. Complex128 adds in partial sums (a solve of 18 x 22 x 24 cells, 297 of
