@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(GV_WARPS * 32) k_givens(SlotState* st, int nf,
   if (lane < 4) {
     const int im = lane & 1, lo = lane >> 1;  // part; 0: cl[i], 1: cl[i + 1]
     const z64 c0 = cl[0];
+    __syncwarp(0xfu);  // all four have read cl[0] before the first rotation overwrites it
     double ax = k == 1 ? c0.re + 1.0 : c0.re, ay = c0.im;  // a of the next rotation
     for (int i = 0; i + 1 < k; ++i) {
       z64 b = cl[i + 1];
