@@ -508,8 +508,6 @@ static int cluster_level(const fks_op* op, ClusterParams<VT>* P = nullptr, size_
   return cluster_level_for<VT>(op->levels, op->cluster_max[sizeof(VT) == 8 ? 0 : 1], P, smem);
 }
 
-constexpr size_t TAIL_SMEM_LIMIT = 220 * 1024;
-
 // Shared memory of the tail kernel: f and z of every tail level, then (when it
 // fits) each level's coefficients (faces, storage, inverse diagonals for the
 // current tau). Returns the bytes; `coef_byte` receives each level's offset.
@@ -1247,11 +1245,10 @@ static void setup_levels(Solve& S) {
   const int bf = bf16_of(S) ? 1 : 0;
   {
     std::lock_guard<std::mutex> build_lock(g_build_mu);
-    tail_prepare<VT>(tail_plan<VT>(Ls, tail_level<VT>(Ls, tail_max_of<VT>(S.op))).smem);
+    tail_prepare<VT>();
     fused_prepare<VT>();
     fused3d_prepare<VT>();
-    size_t csm = 0;
-    if (cluster_level<VT>(S.op, nullptr, &csm) >= 0) cluster_prepare<VT>(csm);
+    if (cluster_level<VT>(S.op) >= 0) cluster_prepare<VT>();
   }
   for (size_t l = 0; l < Ls.size(); ++l)
     PROF(-1, -1, 0, 0, launch_invd<VT>(Ls[l], S.taus, S.n_tau, (cx<VT>*)S.invd[l], S.s, bf));
@@ -2553,12 +2550,7 @@ fks_status fks_op_autotune(fks_op* op, int precision, fks_c128 tau, void* stream
         op->tail_max[pi] = ch.tail;
         op->cluster_max[pi] = ch.cl;
         op->tile8_max[pi] = ch.t8;
-        {
-          // the tail's shared memory and coefficient blob follow the threshold
-          std::lock_guard<std::mutex> build_lock(g_build_mu);
-          tail_prepare<VT>(tail_plan<VT>(op->levels, tail_level<VT>(op->levels, ch.tail)).smem);
-        }
-        Arena probe2;
+        Arena probe2;  // the coefficient blobs follow the thresholds
         carve<VT>(S, probe2, false);
         op->lane0.ws.reserve(probe2.off + 4096);
         carve<VT>(S, op->lane0.ws, false);

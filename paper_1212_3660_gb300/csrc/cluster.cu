@@ -311,14 +311,15 @@ void launch_cluster_blob(const std::vector<LevelHost>& Ls, int l0, const Cluster
   k_cluster_blob<T><<<dim3(CL_SIZE, ntau), 256, 0, s>>>(P, A, blob);
 }
 
+// one value for the whole process, as tail_prepare
 template <typename T>
-void cluster_prepare(size_t smem_bytes) {
-  cudaFuncSetAttribute(k_cluster_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+void cluster_prepare() {
+  cudaFuncSetAttribute(k_cluster_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_LIMIT);
 }
 
 template <typename T>
 bool cluster_launchable(size_t smem_bytes) {
-  cluster_prepare<T>(smem_bytes);
+  cluster_prepare<T>();
   cudaLaunchConfig_t cfg = {};  // the cluster shape is the kernel's compile-time one
   cfg.gridDim = dim3(CL_SIZE);
   cfg.blockDim = dim3(CL_THREADS);
@@ -342,7 +343,7 @@ void launch_cluster_vcycle(const ClusterParams<T>& P, size_t smem_bytes, const S
   template bool cluster_layout<T>(const std::vector<LevelHost>&, int, ClusterParams<T>*, size_t*);          \
   template void launch_cluster_blob<T>(const std::vector<LevelHost>&, int, const ClusterParams<T>&,          \
                                        const cx<T>* const*, const cx<T>*, int, unsigned char*, cudaStream_t); \
-  template void cluster_prepare<T>(size_t);                                                                 \
+  template void cluster_prepare<T>();                                                                       \
   template bool cluster_launchable<T>(size_t);                                                              \
   template void launch_cluster_vcycle<T>(const ClusterParams<T>&, size_t, const SlotState*, int, cudaStream_t);
 

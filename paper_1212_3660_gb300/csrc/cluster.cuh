@@ -54,7 +54,7 @@ template <typename T>
 void launch_cluster_blob(const std::vector<LevelHost>& Ls, int l0, const ClusterParams<T>& P, const cx<T>* const* invd,
                          const cx<T>* Ainv, int ntau, unsigned char* blob, cudaStream_t s);
 template <typename T>
-void cluster_prepare(size_t smem_bytes);
+void cluster_prepare();
 template <typename T>
 void launch_cluster_vcycle(const ClusterParams<T>& P, size_t smem_bytes, const SlotState* st, int nslot,
                            cudaStream_t s);

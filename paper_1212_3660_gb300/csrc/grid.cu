@@ -2266,19 +2266,24 @@ void launch_post2d(const LevelHost& F, const LevelHost& C, uint32_t mask, const 
   (void)C;
 }
 
+// The attribute belongs to the kernel, not to a launch, and every context of the
+// process shares it: always the same value, so that no operator's setup takes
+// shared memory away from the launch or capture that another thread is about to
+// make. (A launch's occupancy follows what it asks for itself.)
 template <typename T>
-void tail_prepare(size_t smem_bytes) {
-  cudaFuncSetAttribute(k_tail_vcycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-  cudaFuncSetAttribute(k_tail2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-  cudaFuncSetAttribute(k_tail_pairs<T, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+void tail_prepare() {
+  auto grant = [](auto kernel, size_t bytes) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  grant(k_tail_vcycle<T>, TAIL_SMEM_LIMIT);
+  grant(k_tail2d<T>, TAIL_SMEM_LIMIT);
+  grant(k_tail_pairs<T, 512>, TAIL_SMEM_LIMIT);
   if constexpr (sizeof(T) == 8) {
-    cudaFuncSetAttribute(k_tail_pairs<T, 512, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    cudaFuncSetAttribute(k_tail_pairs<T, 512, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    grant(k_tail_pairs<T, 512, 1>, TAIL_SMEM_LIMIT);
+    grant(k_tail_pairs<T, 512, 2>, TAIL_SMEM_LIMIT);
   }
-  if constexpr (sizeof(T) == 4)
-    cudaFuncSetAttribute(k_tail_pairs<T, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-  cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(MAX_COARSE * coarse_rows<T>() * sizeof(cx<T>)));
+  if constexpr (sizeof(T) == 4) grant(k_tail_pairs<T, 1024>, TAIL_SMEM_LIMIT);
+  grant(k_coarse_solve<T>, MAX_COARSE * coarse_rows<T>() * sizeof(cx<T>));
 }
 
 template <typename T>
@@ -2379,7 +2384,7 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
   template void launch_post2d<T>(const LevelHost&, const LevelHost&, uint32_t, const SlotState*, const cx<T>*,     \
                                  const cx<T>*, const cx<T>*, cx<T>*, int64_t, const cx<T>*, int64_t, int, int,    \
                                  cudaStream_t, z64*, int64_t, int64_t);                                           \
-  template void tail_prepare<T>(size_t);                                                                          \
+  template void tail_prepare<T>();                                                                                \
   template void launch_tail<T>(const TailParams<T>&, size_t, const SlotState*, int, cudaStream_t, int);                \
   template void launch_invd<T>(const LevelHost&, const z64*, int, cx<T>*, cudaStream_t, int);                     \
   template void launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \

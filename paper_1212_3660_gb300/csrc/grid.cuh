@@ -5,6 +5,8 @@
 namespace fks {
 
 constexpr int TAIL_THREADS = 512;
+// most dynamic shared memory of a tail launch
+constexpr size_t TAIL_SMEM_LIMIT = 220 * 1024;
 // halo of the fused level kernels: four half sweeps, one cell each
 constexpr int FH = 4;
 
@@ -47,7 +49,7 @@ struct TailParams {
 };
 
 template <typename T>
-void tail_prepare(size_t smem_bytes);
+void tail_prepare();
 bool fused_level_ok(const LevelHost& L);
 template <typename T>
 void fused_prepare();
