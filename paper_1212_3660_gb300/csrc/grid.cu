@@ -225,15 +225,15 @@ __global__ void __launch_bounds__(GX * GY) k_apply(LevelView<double> L, z64 s, c
   double lo = fl[c];
   for (int m = m0; m < m1; ++m, c += step) {
     const bool top = m + 1 < nm;
-    const double hi = fl[c + step];
+    const double hi = fl[next_face(c, step)];
     const z64 above = top ? v[c + step] : mk(0.0, 0.0);
     const int row = D3 ? m * ny + j : m;
     const double mm = L.mm[c], d = fmaT(s.re, mm, L.kd[c]), e = mulT(s.im, mm);
     z64 a = mk(0.0, 0.0);
-    if (i > 0) a = axpy(L.fx[c + row], v[c - 1], a);
-    if (i < nx - 1) a = axpy(L.fx[c + row + 1], v[c + 1], a);
+    if (i > 0) a = axpy(L.fx[x_face(c, row)], v[c - 1], a);
+    if (i < nx - 1) a = axpy(L.fx[x_face(c, row) + 1], v[c + 1], a);
     if constexpr (D3) {
-      const int fy = c + m * nx;
+      const int64_t fy = y_face(c, m, nx);
       if (j > 0) a = axpy(L.fy[fy], v[c - nx], a);
       if (j < ny - 1) a = axpy(L.fy[fy + nx], v[c + nx], a);
     }
@@ -1912,23 +1912,24 @@ __global__ void __launch_bounds__(GX * GY)
     const z64* dg = diag64 + (int64_t)tau * L.n;
     int c = m0 * step + j * nx + i;
     z64 below = m0 > 0 ? zz[c - step] : mk(0.0, 0.0), here = zz[c];
-    // the faces below and above along the march: one load per cell
-    int fm = c;  // face below cell c: fz[c] in 3D, fy[c] in 2D
+    // the faces below and above along the march: one load per cell (the face
+    // below cell c: fz[c] in 3D, fy[c] in 2D)
     const double* fl = D3 ? L.fz : L.fy;
-    double lo = fl[fm];
-    for (int m = m0; m < m1; ++m, c += step, fm += step) {
+    double lo = fl[c];
+    for (int m = m0; m < m1; ++m, c += step) {
       const bool top = m + 1 < nm;
-      const double hi = fl[fm + step];
+      const double hi = fl[next_face(c, step)];
       const z64 above = top ? zz[c + step] : mk(0.0, 0.0);
       const int row = D3 ? m * ny + j : m;
-      const double xl = L.fx[c + row], xh = L.fx[c + row + 1];
+      const int64_t fx = x_face(c, row);
+      const double xl = L.fx[fx], xh = L.fx[fx + 1];
       z64 a = vv[c];
       const z64 d = dg[c];
       // the neighbours in nb_sum's order, then the diagonal as in defect_at
       if (i > 0) a = axpy(xl, zz[c - 1], a);
       if (i < nx - 1) a = axpy(xh, zz[c + 1], a);
       if constexpr (D3) {
-        const int fy = c + m * nx;
+        const int64_t fy = y_face(c, m, nx);
         if (j > 0) a = axpy(L.fy[fy], zz[c - nx], a);
         if (j < ny - 1) a = axpy(L.fy[fy + nx], zz[c + nx], a);
       }

@@ -636,15 +636,15 @@ __global__ void __launch_bounds__(GX * GY) k_tres_partial(LevelView<double> L, c
     double lo = fl[c];
     for (int m = m0; m < m1; ++m, c += step) {
       const bool top = m + 1 < nm;
-      const double hi = fl[c + step];
+      const double hi = fl[next_face(c, step)];
       const z64 above = top ? x[c + step] : mk(0.0, 0.0);
       const int row = D3 ? m * ny + j : m;
       const double mc = L.mm[c], d = fmaT(sg.re, mc, L.kd[c]), e = mulT(sg.im, mc);
       z64 a = bs[c];
-      if (i > 0) a = axpy(L.fx[c + row], x[c - 1], a);
-      if (i < nx - 1) a = axpy(L.fx[c + row + 1], x[c + 1], a);
+      if (i > 0) a = axpy(L.fx[x_face(c, row)], x[c - 1], a);
+      if (i < nx - 1) a = axpy(L.fx[x_face(c, row) + 1], x[c + 1], a);
       if constexpr (D3) {
-        const int fy = c + m * nx;
+        const int64_t fy = y_face(c, m, nx);
         if (j > 0) a = axpy(L.fy[fy], x[c - nx], a);
         if (j < ny - 1) a = axpy(L.fy[fy + nx], x[c + nx], a);
       }

@@ -63,6 +63,14 @@ __device__ __forceinline__ void split_row(int row, int ny, unsigned mny, int* j,
   *k = q;
 }
 
+// Flat indices of a cell's faces (c = row nx + i, row = k ny + j): the face
+// arrays hold up to ny nz (x), nx nz (y) or nx ny (z) entries more than the
+// fewer than 2^31 cells, so these take 64 bits. The high faces: + 1, + nx.
+__host__ __device__ __forceinline__ int64_t x_face(int c, int row) { return (int64_t)c + row; }
+__host__ __device__ __forceinline__ int64_t y_face(int c, int k, int nx) { return c + (int64_t)k * nx; }
+// of the cell's faces along the axis that a march takes (`step` cells apart)
+__host__ __device__ __forceinline__ int64_t next_face(int c, int step) { return (int64_t)c + step; }
+
 template <typename T>
 struct Faces {
   T xl, xh, yl, yh, zl, zh;
@@ -118,8 +126,8 @@ __device__ __forceinline__ cx<T> nb_sum(const LevelView<T, C>& L, const Faces<T>
 // FP64 arithmetic is the bound, keeps the ones above.
 template <typename T, typename C>
 __device__ __forceinline__ Faces<T> faces_row(const LevelView<T, C>& L, int k, int row, int c) {
-  const C* fx = L.fx + (unsigned)(c + row);
-  const C* fy = L.fy + (unsigned)(c + k * L.nx);
+  const C* fx = L.fx + ((unsigned)c + (unsigned)row);
+  const C* fy = L.fy + ((unsigned)c + (unsigned)(k * L.nx));
   const C* fz = L.fz + c;
   Faces<T> f{ldc<T>(fx, 0), ldc<T>(fx, 1), ldc<T>(fy, 0), ldc<T>(fy, L.nx), T(0), T(0)};
   if (L.nz > 1) {
