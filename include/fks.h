@@ -404,7 +404,9 @@ void fks_server_destroy(fks_server* srv);
  * cells; 3D operators fuse no level and use a tail of at most 512 or 2048 cells.
  * No cluster kernel. Until the tuner or one of the setters below has chosen
  * them, the fusion and tile thresholds of a precision count the cells of a
- * launch: a level's, times the sources of the batch; afterwards a level's.
+ * launch: a level's, times the sources of the batch; afterwards a level's. In a
+ * server's batch the complex128 thresholds count the geometric mean of the
+ * sources that start it and of its slots, the complex64 ones its slots.
  * `chosen` (host, may be NULL) receives the fusion threshold (fks_op_tiling
  * reads all four).
  */

@@ -6,6 +6,7 @@
 // correction in complex128. All per-step state lives in device memory; the
 // host only enqueues kernels and reads small flags to decide when a loop ends.
 #include <algorithm>
+#include <cmath>
 #include <atomic>
 #include <limits>
 #include <complex>
@@ -390,6 +391,13 @@ struct Solve {
   Lane* lane;
   cudaStream_t s;
   int nslot, n_f, n_tau, m, sched_len, precision, variant;
+  // slots that a server batch reserves for requests that join it later: it may
+  // run with any number of sources from those it starts with up to nslot
+  int spare = 0;
+  int sources() const { return nslot - spare; }
+  // the number that the untuned thresholds of its complex128 levels count: the
+  // geometric mean of the two (fks_solve: all sources)
+  int64_t expected() const { return (int64_t)std::sqrt((double)sources() * nslot); }
   int64_t n;
   double tol, eps;
   int max_cycles;
@@ -644,8 +652,17 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   const int64_t fmax = S.op->fuse_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t16 = S.op->tile16_max[sizeof(VT) == 8 ? 0 : 1];
   const int64_t t8 = S.op->tile8_max[sizeof(VT) == 8 ? 0 : 1];
-  // the batch's sources share a launch: untuned, small tiles while it leaves SMs idle
-  const int64_t nsl = S.op->by_level[sizeof(VT) == 8 ? 0 : 1] ? 1 : S.nslot;
+  // the batch's sources share a launch: untuned, small tiles while it leaves SMs
+  // idle. In a server batch complex128 counts expected() sources, whose
+  // arithmetic fills them; complex64 all slots, because the many blocks of small
+  // tiles cost an idle slot most (4096 blocks that return at once take 5 us).
+  // A served source of 256^2 complex128 with 16 spare slots takes 52.4 ms (69.5
+  // counting slots, 51.7 sources), 128^2 36.7 (42.3, 35.9), 64^2 27.3 (31.5, 27.4),
+  // 160 x 150 183 (178, 183); all 17 slots busy 256^2 522 (491, 543), 128^2 159 (162 to
+  // 171, 180), 64^2 48 (44, 48), 160 x 150 533 (526, 539); complex64 224^2 with one
+  // source 27.9 ms counting slots, 36.4 sources, 311 x 289 40.8 and 59.9.
+  const bool by_level = S.op->by_level[sizeof(VT) == 8 ? 0 : 1];
+  const int64_t nsl = by_level ? 1 : (sizeof(VT) == 8 ? S.expected() : S.nslot);
   auto tile_of = [&](const LevelHost& L) { return L.n * nsl <= t8 ? 8 : (L.n * nsl <= t16 ? 16 : 32); };
   const int pix = sizeof(VT) == 8 ? 0 : 1;
   for (int l = 0; l < lp; ++l) {
@@ -1124,10 +1141,10 @@ static void sec_step_end(Solve& S, int step, int use_cond, cudaGraphConditionalH
     z64* hp = S.h12 + pass * MAX_M;
     if (pass == 0 && S.V32)
       PROF(FKS_K_MDOT, -1, ns * (8 * nn * kk + 16 * nn), ns * 8 * nn * kk,
-           launch_mdot32(S.st, S.V32, vsV, S.w, n, S.mdpart, kmax, n_rhs, S.s));
+           launch_mdot32(S.st, S.V32, vsV, S.w, n, S.mdpart, kmax, n_rhs, S.sources(), S.s));
     else
       PROF(FKS_K_MDOT, -1, ns * 16 * nn * (kk + 1), ns * 8 * nn * kk,
-           launch_mdot(S.st, S.V, vsV, S.w, n, S.mdpart, kmax, n_rhs, S.s));
+           launch_mdot(S.st, S.V, vsV, S.w, n, S.mdpart, kmax, n_rhs, S.sources(), S.s));
     PROF(-1, -1, 0, 0, launch_hreduce(S.st, S.mdpart, n, hp, 2 * MAX_M, n_rhs, S.s));
     PROF(FKS_K_MAXPY, -1, ns * 16 * nn * (kk + 2), ns * 8 * nn * kk,
          launch_maxpy(S.st, S.V, vsV, hp, 2 * MAX_M, S.w, n, n_rhs, S.s));
@@ -3416,6 +3433,7 @@ struct Batch : BatchBase {
     S.lane = lane;
     S.s = s;
     S.nslot = cap;
+    S.spare = cap - std::min(cap, std::max(1, r0.n_rhs - first->next_src));
     S.n_f = r0.n_f;
     S.n_tau = r0.n_tau;
     S.m = o.m_max;
@@ -3457,7 +3475,7 @@ struct Batch : BatchBase {
                                  (double)S.inner_steps, (double)op->tile16_max[0], (double)op->tile16_max[1], S.relax,
                                  (double)op->tail_max[0], (double)op->tail_max[1], (double)op->cluster_max[0],
                                  (double)op->cluster_max[1], (double)op->tile8_max[0], (double)op->tile8_max[1], 0.0,
-                                 (double)(S.amg ? op->amg.gen : -1), (double)S.amg_L, 1.0};
+                                 (double)(S.amg ? op->amg.gen : -1), (double)S.amg_L, 1.0 + S.spare};
       for (int pz = 0; pz < 2; ++pz)
         for (int l = 0; l < MAX_LEVELS; ++l) key.push_back((double)op->zchunk[pz][l]);
       key.push_back((double)op->coop_max[0]);

@@ -721,16 +721,18 @@ int mdot_blocks(int64_t n) { return (int)nbk(n, MD_THREADS * MD_ROWS); }
 // one SM's FP64 pipe busy for 4.6 us, so with 16 columns each the few row
 // blocks of a small problem left most SMs idle (65 us per projection from 4096
 // rows up to 512^2). Fewer columns per block until 24 of them (a usual step)
-// give two blocks per SM; w is then read again per chunk, from L2.
-static int mdot_cols(int64_t n, int nslot) {
-  const int64_t rb = (int64_t)mdot_blocks(n) * nslot;
+// give two blocks per SM; w is then read again per chunk, from L2. A server
+// batch's spare slots do not count: they do no arithmetic (one source of 224^2
+// with 16 of them 27.9 -> 26.4 ms a solve in complex64, 56.4 -> 53.6 in complex128).
+static int mdot_cols(int64_t n, int nsrc) {
+  const int64_t rb = (int64_t)mdot_blocks(n) * nsrc;
   int c = MD_COLS;
   while (c > 1 && rb * 24 < (int64_t)c * 304) c /= 2;
   return c;
 }
 void launch_mdot(const SlotState* st, const z64* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
-                 int nslot, cudaStream_t s) {
-  const int cols = mdot_cols(n, nslot);
+                 int nslot, int nsrc, cudaStream_t s) {
+  const int cols = mdot_cols(n, nsrc);
   const dim3 g(mdot_blocks(n), nslot, nbk(kmax, cols));
   switch (cols) {
     case 1: k_mdot<1><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;
@@ -741,8 +743,8 @@ void launch_mdot(const SlotState* st, const z64* V, int64_t vsV, const z64* w, i
   }
 }
 void launch_mdot32(const SlotState* st, const z32* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
-                   int nslot, cudaStream_t s) {
-  const int cols = mdot_cols(n, nslot);
+                   int nslot, int nsrc, cudaStream_t s) {
+  const int cols = mdot_cols(n, nsrc);
   const dim3 g(mdot_blocks(n), nslot, nbk(kmax, cols));
   switch (cols) {
     case 1: k_mdot32<1><<<g, MD_THREADS, 0, s>>>(st, V, vsV, w, n, partial); break;

@@ -27,10 +27,10 @@ void launch_step_begin(SlotState* st, int nslot, const int32_t* sched, int sched
 void launch_mass(const SlotState* st, const double* mm, const z64* Z, int64_t vsZ, z64* w, int64_t n, double* partial,
                  int nslot, cudaStream_t s);
 void launch_mdot(const SlotState* st, const z64* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
-                 int nslot, cudaStream_t s);
+                 int nslot, int nsrc, cudaStream_t s);
 // the first CGS projection from the complex64 copy of the basis (fp32 sums)
 void launch_mdot32(const SlotState* st, const z32* V, int64_t vsV, const z64* w, int64_t n, z64* partial, int kmax,
-                   int nslot, cudaStream_t s);
+                   int nslot, int nsrc, cudaStream_t s);
 void launch_hreduce(const SlotState* st, const z64* partial, int64_t n, z64* h, int64_t hstride, int nslot,
                     cudaStream_t s);
 void launch_maxpy(const SlotState* st, const z64* V, int64_t vsV, const z64* h, int64_t hstride, z64* w, int64_t n,
