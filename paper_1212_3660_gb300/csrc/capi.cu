@@ -420,6 +420,7 @@ struct Solve {
   int32_t *cyc, *sst, *mj, *sched, *rep_cyc, *rep_mj, *singular, *flags, *counter, *bcount;
   // multigrid, cycle precision
   std::vector<void*> f, z, z2, invd;
+  std::vector<SweepGeom> sweeps;  // tiles of the levels that run one-launch sweeps (vcycle fills them)
   void* cinv;      // coarse inverses in cycle precision, transposed
   z64* cwork;      // dense coarse matrices
   z64* cwork2;     // the inversion's second buffer
@@ -665,6 +666,12 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   const int64_t nsl = by_level ? 1 : (sizeof(VT) == 8 ? S.expected() : S.nslot);
   auto tile_of = [&](const LevelHost& L) { return L.n * nsl <= t8 ? 8 : (L.n * nsl <= t16 ? 16 : 32); };
   const int pix = sizeof(VT) == 8 ? 0 : 1;
+  S.sweeps.resize(Ls.size());
+  auto sweep_of = [&](int l) -> const SweepGeom& {
+    SweepGeom& G = S.sweeps[l];
+    if (!G.ntx) G = sweep_geom<VT>(Ls[l], S.nslot);
+    return G;
+  };
   for (int l = 0; l < lp; ++l) {
     const LevelHost& L = Ls[l];
     if (fused_level_ok(L) && L.n * nsl <= fmax) {
@@ -686,7 +693,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
       cx<VT>* z2 = (cx<VT>*)S.z2[l];
       for (int r = 0; r < NU1; ++r)
         PROF(FKS_K_SMOOTH, l, smooth_b(L, r == 0) + smooth_b(L, 0), smooth_f(L, r == 0) + smooth_f(L, 0),
-             launch_sweep3<VT>(L, nullptr, 0, r == 0 ? SWEEP_ZERO : 0, S.st, I(l), F(l), Zl(l), r == 0 ? Zl(l) : z2,
+             launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, r == 0 ? SWEEP_ZERO : 0, S.st, I(l), F(l), Zl(l), r == 0 ? Zl(l) : z2,
                                L.n, nullptr, S.nslot, 0, nullptr, 0, 0, bf, s));
       PROF(FKS_K_RESTRICT, l, ns * (L.n * ((1 + rr) * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
            ns * L.n * rr * (8 * d + 10),
@@ -840,12 +847,12 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
         PROF(FKS_K_PROLONG, l, ns * (2 * cv * L.n + cv * Ls[l + 1].n), ns * L.n * (4.0 * (1 << S.op->dim) + 2),
              launch_prolong_add<VT>(L, Ls[l + 1], S.op->mask, S.st, zfin, Ls[l + 1].n, z2, L.n, S.nslot, s));
       PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + ns * cv * Ls[l + 1].n, 2 * smooth_f(L, 0) + ns * L.n * 18.0,
-           launch_sweep3<VT>(L, &Ls[l + 1], S.op->mask, by2 ? SWEEP_PROLONG : 0, S.st, I(l), F(l), z2, Zl(l), L.n, zfin,
-                             S.nslot, 1, nullptr, 0, 0, bf, s));
+           launch_sweep3<VT>(L, sweep_of(l), &Ls[l + 1], S.op->mask, by2 ? SWEEP_PROLONG : 0, S.st, I(l), F(l), z2,
+                             Zl(l), L.n, zfin, S.nslot, 1, nullptr, 0, 0, bf, s));
       PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + (add_to_zk ? ns * L.n * 32.0 : 0.0),
            2 * smooth_f(L, 0) + (add_to_zk ? ns * L.n * 2.0 : 0.0),
-           launch_sweep3<VT>(L, nullptr, 0, add_to_zk ? SWEEP_CORRECT : 0, S.st, I(l), F(l), Zl(l), z2, L.n, nullptr,
-                             S.nslot, 1, add_to_zk ? Zk : nullptr, vsZk, zcol, bf, s));
+           launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, add_to_zk ? SWEEP_CORRECT : 0, S.st, I(l), F(l), Zl(l), z2,
+                             L.n, nullptr, S.nslot, 1, add_to_zk ? Zk : nullptr, vsZk, zcol, bf, s));
       zfin = add_to_zk ? nullptr : z2;
       continue;
     }

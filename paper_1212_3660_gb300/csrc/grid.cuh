@@ -1,6 +1,7 @@
 // Launchers of the structured-grid and multigrid kernels (grid.cu).
 #pragma once
 #include "common.cuh"
+#include "sweep.cuh"
 
 namespace fks {
 
@@ -120,10 +121,14 @@ void launch_gs(const LevelHost& L, const SlotState* st, const cx<T>* invd, const
 // the result added to column k - 1 of Zk instead of written (as launch_gs).
 enum { SWEEP_ZERO = 1, SWEEP_PROLONG = 2, SWEEP_CORRECT = 4 };
 bool sweep3_ok(const LevelHost& L, int nslot, bool fp64);
+// tile of a level's sweeps (searched on the host: once per solve, not per launch)
 template <typename T>
-void launch_sweep3(const LevelHost& L, const LevelHost* below, uint32_t mask, int mode, const SlotState* st,
-                   const cx<T>* invd, const cx<T>* f, const cx<T>* zin, cx<T>* zout, int64_t vs, const cx<T>* zc,
-                   int nslot, int color, z64* Zk, int64_t vsZk, int64_t zcol, int bf16, cudaStream_t s);
+SweepGeom sweep_geom(const LevelHost& L, int nslot);
+template <typename T>
+void launch_sweep3(const LevelHost& L, const SweepGeom& G, const LevelHost* below, uint32_t mask, int mode,
+                   const SlotState* st, const cx<T>* invd, const cx<T>* f, const cx<T>* zin, cx<T>* zout, int64_t vs,
+                   const cx<T>* zc, int nslot, int color, z64* Zk, int64_t vsZk, int64_t zcol, int bf16,
+                   cudaStream_t s);
 template <typename T>
 void launch_residual_restrict(const LevelHost& F, const LevelHost& C, const SlotState* st, const z64* taus,
                               const cx<T>* f, const cx<T>* z, int64_t vs, cx<T>* fc, int64_t vsc, int nslot,

@@ -26,9 +26,6 @@
 // Every update repeats k_gs's arithmetic in its order (a neighbour outside the
 // grid adds t * 0 instead of nothing), so the results are bitwise those of the
 // half sweeps.
-#include <algorithm>
-#include <cmath>
-
 #include "grid.cuh"
 #include "stencil.cuh"
 
@@ -39,12 +36,6 @@ template <typename T>
 constexpr int sweep_threads() { return sizeof(T) == 8 ? 256 : 384; }
 template <typename T>
 constexpr int sweep_blocks() { return sizeof(T) == 8 ? 1 : 2; }
-
-struct SweepGeom {
-  int opx, oy, oz;    // pairs, rows and planes a block writes
-  int txp;            // pairs of its region, the ring included; its rows are oy + 4
-  int ntx, nty, ntz;
-};
 
 template <typename T>
 struct SweepProl {  // the correction of the level below (coarsened by 2 in every axis)
@@ -269,40 +260,12 @@ __global__ void __launch_bounds__(sweep_threads<T>(), sweep_blocks<T>())
   }
 }
 
-// Tile and chunk of a level: the least estimated time over the tiles that fit.
 template <typename T>
-static SweepGeom sweep_geom(const LevelHost& L, int nslot) {
-  const int NT = sweep_threads<T>(), np = (L.nx + 1) / 2;
-  SweepGeom best{};
-  double cost = 1e300;
-  for (int ntx = 1; ntx <= np; ++ntx) {
-    const int opx = (np + ntx - 1) / ntx, txp = std::min(opx + (ntx > 2 ? 2 : ntx - 1), np);
-    if (txp * 5 > NT) continue;
-    if (ntx > 1 && (np + opx - 1) / opx != ntx) continue;
-    if (cost < 1e300 && opx < 8) break;
-    for (int oy = 1; oy <= L.ny && txp * (oy + 4) <= NT; ++oy) {
-      const int nty = (L.ny + oy - 1) / oy;
-      if (oy > 1 && (L.ny + oy - 2) / (oy - 1) == nty) continue;  // the same tiles with fewer rows
-      const int nt = (txp * (oy + 4) + 31) & ~31;
-      const int per = sweep_blocks<T>() * std::max(1, NT / nt) * 152;
-      for (int oz = 1; oz <= L.nz; ++oz) {
-        const int ntz = (L.nz + oz - 1) / oz;
-        if (ntz > 65535 || (oz > 1 && (L.nz + oz - 2) / (oz - 1) == ntz)) continue;
-        const double blocks = (double)ntx * nty * ntz * nslot, rounds = std::ceil(blocks / per);
-        // a step is 0.5 us of latency, or the SM's share of the traffic (19 words per pair, 46 GB/s)
-        const double step = std::max(0.5, std::min(blocks / 152, (double)per / 152) * nt * 19.0 * sizeof(T) / 46000.0);
-        const double c = rounds * (oz + 2.5) * step;
-        if (c < cost) {
-          cost = c;
-          best = SweepGeom{opx, oy, oz, txp, ntx, nty, ntz};
-        }
-      }
-    }
-  }
-  return best;
+SweepGeom sweep_geom(const LevelHost& L, int nslot) {
+  return sweep_geometry(L.nx, L.ny, L.nz, nslot, sweep_threads<T>(), sweep_blocks<T>(), (int)sizeof(T));
 }
 
-// Cells (times sources) up to which the march beats the half sweeps: 48^3 in
+// Cells (times the batch's slots) up to which the march beats the half sweeps: 48^3 in
 // complex64 (20.3 us of sweeps per V-cycle against 26.5; 64^3 is even). Not in
 // complex128 (45 x 53 x 37 with 23 x 27 x 19 and 12 x 14 x 10 below: 99.2 ms a
 // solve against 98.4), where the recomputed ring costs FP64 time.
@@ -327,10 +290,9 @@ static void launch_c(const LevelHost& L, const SweepGeom& G, int mode, const Slo
 }
 
 template <typename T>
-void launch_sweep3(const LevelHost& L, const LevelHost* below, uint32_t mask, int mode, const SlotState* st,
-                   const cx<T>* invd, const cx<T>* f, const cx<T>* zin, cx<T>* zout, int64_t vs, const cx<T>* zc,
+void launch_sweep3(const LevelHost& L, const SweepGeom& G, const LevelHost* below, uint32_t mask, int mode,
+                   const SlotState* st, const cx<T>* invd, const cx<T>* f, const cx<T>* zin, cx<T>* zout, int64_t vs, const cx<T>* zc,
                    int nslot, int color, z64* Zk, int64_t vsZk, int64_t zcol, int bf16, cudaStream_t s) {
-  const SweepGeom G = sweep_geom<T>(L, nslot);
   SweepProl<T> P{};
   if (mode & SWEEP_PROLONG) P = SweepProl<T>{mask, below->nx, below->ny, below->nz, zc, below->n};
   auto go = [&](auto c) {
@@ -348,9 +310,10 @@ void launch_sweep3(const LevelHost& L, const LevelHost* below, uint32_t mask, in
 }
 
 #define SW_INST(T)                                                                                                 \
-  template void launch_sweep3<T>(const LevelHost&, const LevelHost*, uint32_t, int, const SlotState*, const cx<T>*, \
-                                 const cx<T>*, const cx<T>*, cx<T>*, int64_t, const cx<T>*, int, int, z64*,         \
-                                 int64_t, int64_t, int, cudaStream_t);
+  template SweepGeom sweep_geom<T>(const LevelHost&, int);                                                         \
+  template void launch_sweep3<T>(const LevelHost&, const SweepGeom&, const LevelHost*, uint32_t, int,              \
+                                 const SlotState*, const cx<T>*, const cx<T>*, const cx<T>*, cx<T>*, int64_t,      \
+                                 const cx<T>*, int, int, z64*, int64_t, int64_t, int, cudaStream_t);
 SW_INST(double)
 SW_INST(float)
 
