@@ -590,7 +590,7 @@ def jacobian_bench(args, rank, world, local, dist):
         t1.record(stream)
         torch.cuda.synchronize()
         replicas.barrier()
-    launches = fks.fks_profile_read(solver.op)["all_launches"] - l0 + args.steps  # + the sensitivity kernel
+    launches = fks.fks_profile_read(solver.op)["all_launches"] - l0 + 2 * args.steps  # + the face weights and the sensitivity kernel
     ms = t0.elapsed_time(t1) / args.steps
     value = replicas.throughput(rows / args.steps, ms / 1000.0)
     parts /= args.steps

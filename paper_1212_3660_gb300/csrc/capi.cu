@@ -1304,8 +1304,8 @@ static void setup_levels(Solve& S) {
   CK(cudaMemsetAsync(S.singular, 0, sizeof(int), S.s));
   CK(cudaMemsetAsync(S.counter, 0, sizeof(int), S.s));
   CK(cudaMemsetAsync(S.bcount, 0, sizeof(int) * S.nslot, S.s));
-  S.lane->prof.all_launches += 3;
-  launch_coarse_inverse<VT>(C, S.taus, S.n_tau, S.cwork, S.cwork2, (cx<VT>*)S.cinv, S.singular, S.s, bf);
+  S.lane->prof.all_launches += launch_coarse_inverse<VT>(C, S.taus, S.n_tau, S.cwork, S.cwork2, (cx<VT>*)S.cinv,
+                                                         S.singular, S.s, bf);
   ClusterParams<VT> CP{};
   const int lc = cluster_level<VT>(S.op, &CP);
   if (lc >= 0) {

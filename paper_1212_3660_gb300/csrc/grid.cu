@@ -2090,8 +2090,8 @@ void launch_invd(const LevelHost& L, const z64* taus, int ntau, cx<T>* out, cuda
 }
 
 template <typename T>
-void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
-                           int* singular, cudaStream_t s, int from_f32) {
+int launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
+                          int* singular, cudaStream_t s, int from_f32) {
   const int n = (int)L.n;
   const int64_t nn = (int64_t)n * n;
   const bool small = n <= GJ_SMALL;
@@ -2109,7 +2109,7 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
   else k_coarse_dense<double><<<gd, 128, 0, s>>>(view<double>(L), taus, work, c0);
   if (small) {
     k_gj_small<T><<<ntau, 512, 0, s>>>(work, inv, n, singular);
-    return;
+    return 2;
   }
   z64 *src = work, *dst = work2;
   const unsigned nt = nb(n, GJ_T);
@@ -2127,6 +2127,7 @@ void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* w
   }
   cudaMemcpyAsync(dst, piv, sizeof(int32_t) * n * ntau, cudaMemcpyDeviceToDevice, s);
   k_gj_finish<T><<<dim3(nt, nt, ntau), dim3(32, 8), 0, s>>>(src, (const int32_t*)dst, inv, n);
+  return 2 + (one ? n : 2 * n);
 }
 
 void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, cudaStream_t s) {
@@ -2388,7 +2389,7 @@ void launch_inner_decide(SlotState* st, int nslot, const double* partial, int nb
   template void tail_prepare<T>();                                                                                \
   template void launch_tail<T>(const TailParams<T>&, size_t, const SlotState*, int, cudaStream_t, int);                \
   template void launch_invd<T>(const LevelHost&, const z64*, int, cx<T>*, cudaStream_t, int);                     \
-  template void launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \
+  template int launch_coarse_inverse<T>(const LevelHost&, const z64*, int, z64*, z64*, cx<T>*, int*, cudaStream_t, \
                                          int);                                                                    \
   template void launch_gs<T>(const LevelHost&, const SlotState*, const cx<T>*, const cx<T>*, cx<T>*, int64_t, int,  \
                              int, int, cudaStream_t, z64*, int64_t, int64_t, int);                                \

@@ -99,10 +99,10 @@ void launch_to_f32(const double* a, float* b, int64_t n, cudaStream_t s);
 template <typename T>
 void launch_invd(const LevelHost& L, const z64* taus, int ntau, cx<T>* out, cudaStream_t s, int from_f32 = 0);
 // inv[q] = (K + tau_q M)^{-1} of the coarsest level in the cycle precision,
-// transposed; work, work2: n_tau n^2 values each.
+// transposed; work, work2: n_tau n^2 values each. Returns the number of launches.
 template <typename T>
-void launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
-                           int* singular, cudaStream_t s, int from_f32 = 0);
+int launch_coarse_inverse(const LevelHost& L, const z64* taus, int ntau, z64* work, z64* work2, cx<T>* inv,
+                          int* singular, cudaStream_t s, int from_f32 = 0);
 // b = a rounded to bf16, r = the same value as fp32
 void launch_round_bf16(const double* a, __nv_bfloat16* b, float* r, int64_t n, cudaStream_t s);
 // y = (K + sh M) x for nvec vectors of the finest level, vs elements apart
