@@ -669,7 +669,7 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   S.sweeps.resize(Ls.size());
   auto sweep_of = [&](int l) -> const SweepGeom& {
     SweepGeom& G = S.sweeps[l];
-    if (!G.ntx) G = sweep_geom<VT>(Ls[l], S.nslot);
+    if (!G.ntx) G = sweep_geom(Ls[l], S.nslot);
     return G;
   };
   for (int l = 0; l < lp; ++l) {
@@ -688,18 +688,20 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
                             S.op->zchunk[pix][l], s));
       continue;
     }
-    if (sweep3_ok(L, S.nslot, sizeof(VT) == 8)) {
-      // both half sweeps of a sweep in one launch: zero start into z, then z into z2
-      cx<VT>* z2 = (cx<VT>*)S.z2[l];
-      for (int r = 0; r < NU1; ++r)
-        PROF(FKS_K_SMOOTH, l, smooth_b(L, r == 0) + smooth_b(L, 0), smooth_f(L, r == 0) + smooth_f(L, 0),
-             launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, r == 0 ? SWEEP_ZERO : 0, S.st, I(l), F(l), Zl(l), r == 0 ? Zl(l) : z2,
-                               L.n, nullptr, S.nslot, 0, nullptr, 0, 0, bf, s));
-      PROF(FKS_K_RESTRICT, l, ns * (L.n * ((1 + rr) * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
-           ns * L.n * rr * (8 * d + 10),
-           launch_residual_restrict<VT>(L, Ls[l + 1], S.st, S.taus, F(l), z2, L.n, F(l + 1), Ls[l + 1].n, S.nslot, s,
-                                        bf));
-      continue;
+    if constexpr (sizeof(VT) == 4) {
+      if (sweep3_ok(L, S.nslot)) {
+        // both half sweeps of a sweep in one launch: zero start into z, then z into z2
+        cx<VT>* z2 = (cx<VT>*)S.z2[l];
+        for (int r = 0; r < NU1; ++r)
+          PROF(FKS_K_SMOOTH, l, smooth_b(L, r == 0) + smooth_b(L, 0), smooth_f(L, r == 0) + smooth_f(L, 0),
+               launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, r == 0 ? SWEEP_ZERO : 0, S.st, I(l), F(l), Zl(l),
+                                 r == 0 ? Zl(l) : z2, L.n, nullptr, S.nslot, 0, nullptr, 0, 0, bf, s));
+        PROF(FKS_K_RESTRICT, l, ns * (L.n * ((1 + rr) * cv + (d + 1) * rv) + cv * Ls[l + 1].n),
+             ns * L.n * rr * (8 * d + 10),
+             launch_residual_restrict<VT>(L, Ls[l + 1], S.st, S.taus, F(l), z2, L.n, F(l + 1), Ls[l + 1].n, S.nslot, s,
+                                          bf));
+        continue;
+      }
     }
     for (int r = 0; r < NU1; ++r) {
       int zs = r == 0 ? 1 : 0;
@@ -839,22 +841,24 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
       continue;
     }
     const bool add_to_zk = l == 0 && Zk;
-    if (sweep3_ok(L, S.nslot, sizeof(VT) == 8)) {
-      // interpolation and the first sweep from z2 into z, the second into z2 or onto z_k
-      cx<VT>* z2 = (cx<VT>*)S.z2[l];
-      const bool by2 = L.rx == 2 && L.ry == 2 && L.rz == 2;
-      if (!by2)
-        PROF(FKS_K_PROLONG, l, ns * (2 * cv * L.n + cv * Ls[l + 1].n), ns * L.n * (4.0 * (1 << S.op->dim) + 2),
-             launch_prolong_add<VT>(L, Ls[l + 1], S.op->mask, S.st, zfin, Ls[l + 1].n, z2, L.n, S.nslot, s));
-      PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + ns * cv * Ls[l + 1].n, 2 * smooth_f(L, 0) + ns * L.n * 18.0,
-           launch_sweep3<VT>(L, sweep_of(l), &Ls[l + 1], S.op->mask, by2 ? SWEEP_PROLONG : 0, S.st, I(l), F(l), z2,
-                             Zl(l), L.n, zfin, S.nslot, 1, nullptr, 0, 0, bf, s));
-      PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + (add_to_zk ? ns * L.n * 32.0 : 0.0),
-           2 * smooth_f(L, 0) + (add_to_zk ? ns * L.n * 2.0 : 0.0),
-           launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, add_to_zk ? SWEEP_CORRECT : 0, S.st, I(l), F(l), Zl(l), z2,
-                             L.n, nullptr, S.nslot, 1, add_to_zk ? Zk : nullptr, vsZk, zcol, bf, s));
-      zfin = add_to_zk ? nullptr : z2;
-      continue;
+    if constexpr (sizeof(VT) == 4) {
+      if (sweep3_ok(L, S.nslot)) {
+        // interpolation and the first sweep from z2 into z, the second into z2 or onto z_k
+        cx<VT>* z2 = (cx<VT>*)S.z2[l];
+        const bool by2 = L.rx == 2 && L.ry == 2 && L.rz == 2;
+        if (!by2)
+          PROF(FKS_K_PROLONG, l, ns * (2 * cv * L.n + cv * Ls[l + 1].n), ns * L.n * (4.0 * (1 << S.op->dim) + 2),
+               launch_prolong_add<VT>(L, Ls[l + 1], S.op->mask, S.st, zfin, Ls[l + 1].n, z2, L.n, S.nslot, s));
+        PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + ns * cv * Ls[l + 1].n, 2 * smooth_f(L, 0) + ns * L.n * 18.0,
+             launch_sweep3<VT>(L, sweep_of(l), &Ls[l + 1], S.op->mask, by2 ? SWEEP_PROLONG : 0, S.st, I(l), F(l), z2,
+                               Zl(l), L.n, zfin, S.nslot, 1, nullptr, 0, 0, bf, s));
+        PROF(FKS_K_SMOOTH, l, 2 * smooth_b(L, 0) + (add_to_zk ? ns * L.n * 32.0 : 0.0),
+             2 * smooth_f(L, 0) + (add_to_zk ? ns * L.n * 2.0 : 0.0),
+             launch_sweep3<VT>(L, sweep_of(l), nullptr, 0, add_to_zk ? SWEEP_CORRECT : 0, S.st, I(l), F(l), Zl(l), z2,
+                               L.n, nullptr, S.nslot, 1, add_to_zk ? Zk : nullptr, vsZk, zcol, bf, s));
+        zfin = add_to_zk ? nullptr : z2;
+        continue;
+      }
     }
     PROF(FKS_K_PROLONG, l, ns * (2 * cv * L.n + cv * Ls[l + 1].n), ns * L.n * (4.0 * (1 << S.op->dim) + 2),
          launch_prolong_add<VT>(L, Ls[l + 1], S.op->mask, S.st, zfin, Ls[l + 1].n, Zl(l), L.n, S.nslot, s));

@@ -1925,7 +1925,7 @@ __global__ void __launch_bounds__(GX * GY)
       const double xl = L.fx[fx], xh = L.fx[fx + 1];
       z64 a = vv[c];
       const z64 d = dg[c];
-      // the neighbours in nb_sum's order, then the diagonal as in defect_at
+      // the neighbours in nb_sum's order, then the diagonal as in minus_product
       if (i > 0) a = axpy(xl, zz[c - 1], a);
       if (i < nx - 1) a = axpy(xh, zz[c + 1], a);
       if constexpr (D3) {

@@ -114,15 +114,14 @@ template <typename T>
 void launch_gs(const LevelHost& L, const SlotState* st, const cx<T>* invd, const cx<T>* f, cx<T>* z, int64_t vs,
                int nslot, int color, int zero_start, cudaStream_t s, z64* Zk = nullptr, int64_t vsZk = 0,
                int64_t zcol = 0, int bf16 = 0);
-// One whole red-black sweep of a 3D level (sweep.cu), from zin to zout (another
+// One whole red-black sweep of a 3D level in complex64 (sweep.cu), from zin to zout (another
 // buffer), `color` first; bitwise two launch_gs calls. Modes: from z = 0 (zin
 // unused); zin + P zc instead of zin (zc: the correction of the level `below`,
 // coarsened by 2 in every axis);
 // the result added to column k - 1 of Zk instead of written (as launch_gs).
 enum { SWEEP_ZERO = 1, SWEEP_PROLONG = 2, SWEEP_CORRECT = 4 };
-bool sweep3_ok(const LevelHost& L, int nslot, bool fp64);
+bool sweep3_ok(const LevelHost& L, int nslot);
 // tile of a level's sweeps (searched on the host: once per solve, not per launch)
-template <typename T>
 SweepGeom sweep_geom(const LevelHost& L, int nslot);
 template <typename T>
 void launch_sweep3(const LevelHost& L, const SweepGeom& G, const LevelHost* below, uint32_t mask, int mode,

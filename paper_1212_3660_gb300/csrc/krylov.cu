@@ -608,7 +608,7 @@ __global__ void k_assemble(const z64* __restrict__ Z, int64_t vsZ, const z64* __
 // Partial sums of |b - (K + sigma_j M) x_j|^2, one (source, shift) per
 // gridDim.z. Bound by the FP64 pipe (a 3D cell takes 12 fused multiply-adds for
 // its neighbours, 4 + 2 for the diagonal, 2 for the norm; the arithmetic and
-// its order are defect_at's): as in the defect kernel a thread marches over R
+// its order are the defect kernel's): as there, a thread marches over R
 // cells along z (3D) or y (2D), which leaves the block's reduction a small
 // share.
 template <bool D3>

@@ -176,16 +176,6 @@ __device__ __forceinline__ cx<T> minus_product(cx<T> acc, cx<T> diag, cx<T> x) {
   return acc;
 }
 
-// v_c - ((K + tau M) x)_c with diag = K_cc + tau M_cc given: the neighbour
-// terms accumulate onto v, then diag * x_c is subtracted with fused
-// multiply-adds (fewer FP64 operations than v - A x).
-template <typename T, typename C>
-__device__ __forceinline__ cx<T> defect_at(const LevelView<T, C>& L, Cell p, int64_t c, cx<T> diag, cx<T> v,
-                                           const cx<T>* __restrict__ x) {
-  Faces<T> f = faces_at(L, p);
-  return minus_product(nb_sum(L, f, p, c, x, v), diag, x[c]);
-}
-
 // Red-black Gauss-Seidel update of cell c: (f_c + sum_nb t z_nb) / (K_cc + tau M_cc),
 // the neighbours taken as zero when `zero_start`.
 template <typename T, typename C>

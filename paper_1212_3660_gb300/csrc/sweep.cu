@@ -31,11 +31,8 @@
 
 namespace fks {
 
-// threads per block, two blocks per SM
-template <typename T>
-constexpr int sweep_threads() { return sizeof(T) == 8 ? 256 : 384; }
-template <typename T>
-constexpr int sweep_blocks() { return sizeof(T) == 8 ? 1 : 2; }
+constexpr int SWEEP_THREADS = 384;  // most threads per block
+constexpr int SWEEP_BLOCKS = 2;     // blocks per SM
 
 template <typename T>
 struct SweepProl {  // the correction of the level below (coarsened by 2 in every axis)
@@ -88,13 +85,13 @@ __device__ __forceinline__ void pair_r(const C* p, bool second, T* o) {
 }
 
 template <typename T, typename C, int MODE, bool EVEN>
-__global__ void __launch_bounds__(sweep_threads<T>(), sweep_blocks<T>())
+__global__ void __launch_bounds__(SWEEP_THREADS, SWEEP_BLOCKS)
     k_sweep3(LevelView<T, C> L, SweepGeom G, const SlotState* st, const cx<T>* __restrict__ invd,
              const cx<T>* __restrict__ f, const cx<T>* __restrict__ zin, cx<T>* __restrict__ zout, int64_t vs,
              int color, SweepProl<T> P, z64* __restrict__ Zk, int64_t vsZk, int64_t zcol) {
   pdl_enter();
   constexpr bool ZERO = MODE & SWEEP_ZERO, PROL = MODE & SWEEP_PROLONG, CORR = MODE & SWEEP_CORRECT;
-  constexpr int NT = sweep_threads<T>();
+  constexpr int NT = SWEEP_THREADS;
   __shared__ cx<T> sA[2][NT];  // old second colour
   __shared__ cx<T> sB[2][NT];  // new first colour
   const int slot = blockIdx.z;
@@ -260,18 +257,18 @@ __global__ void __launch_bounds__(sweep_threads<T>(), sweep_blocks<T>())
   }
 }
 
-template <typename T>
 SweepGeom sweep_geom(const LevelHost& L, int nslot) {
-  return sweep_geometry(L.nx, L.ny, L.nz, nslot, sweep_threads<T>(), sweep_blocks<T>(), (int)sizeof(T));
+  return sweep_geometry(L.nx, L.ny, L.nz, nslot, SWEEP_THREADS, SWEEP_BLOCKS, (int)sizeof(float));
 }
 
-// Cells (times the batch's slots) up to which the march beats the half sweeps: 48^3 in
-// complex64 (20.3 us of sweeps per V-cycle against 26.5; 64^3 is even). Not in
-// complex128 (45 x 53 x 37 with 23 x 27 x 19 and 12 x 14 x 10 below: 99.2 ms a
-// solve against 98.4), where the recomputed ring costs FP64 time.
-bool sweep3_ok(const LevelHost& L, int nslot, bool fp64) {
-  return L.nz > 1 && !fp64 && L.n * nslot <= 131072;
-}
+// Cells (times the batch's slots) up to which the march beats the half sweeps:
+// 48^3 in complex64 (20.3 us of sweeps per V-cycle against 26.5; 64^3 is even).
+// complex128 has none: the recomputed ring costs FP64 time, and they gained on
+// some grids and lost on others (solves with the half sweeps and with the march
+// on levels up to 2000, 16384 and 131072 cells: 45 x 53 x 37 77.2, 77.6, 78.3 and
+// 87.8 ms; 18 x 22 x 24 41.8, 39.0, 38.6 and 38.6; 64 x 48 x 48 73.1, 73.2, 72.5 and
+// 68.0).
+bool sweep3_ok(const LevelHost& L, int nslot) { return L.nz > 1 && L.n * nslot <= 131072; }
 
 template <typename T, typename C, bool EVEN>
 static void launch_c(const LevelHost& L, const SweepGeom& G, int mode, const SlotState* st, const cx<T>* invd,
@@ -300,21 +297,12 @@ void launch_sweep3(const LevelHost& L, const SweepGeom& G, const LevelHost* belo
     if (L.nx % 2 == 0) launch_c<T, C, true>(L, G, mode, st, invd, f, zin, zout, vs, nslot, color, P, Zk, vsZk, zcol, s);
     else launch_c<T, C, false>(L, G, mode, st, invd, f, zin, zout, vs, nslot, color, P, Zk, vsZk, zcol, s);
   };
-  if constexpr (sizeof(T) == 4) {
-    if (bf16) {
-      go(__nv_bfloat16{});
-      return;
-    }
-  }
-  go(T{});
+  if (bf16) go(__nv_bfloat16{});
+  else go(T{});
 }
 
-#define SW_INST(T)                                                                                                 \
-  template SweepGeom sweep_geom<T>(const LevelHost&, int);                                                         \
-  template void launch_sweep3<T>(const LevelHost&, const SweepGeom&, const LevelHost*, uint32_t, int,              \
-                                 const SlotState*, const cx<T>*, const cx<T>*, const cx<T>*, cx<T>*, int64_t,      \
-                                 const cx<T>*, int, int, z64*, int64_t, int64_t, int, cudaStream_t);
-SW_INST(double)
-SW_INST(float)
+template void launch_sweep3<float>(const LevelHost&, const SweepGeom&, const LevelHost*, uint32_t, int,
+                                   const SlotState*, const z32*, const z32*, const z32*, z32*, int64_t, const z32*,
+                                   int, int, z64*, int64_t, int64_t, int, cudaStream_t);
 
 }  // namespace fks
