@@ -303,12 +303,15 @@ struct fks_op {
   // fused 2D levels with at most this many cells use 16 x 16 tiles (else 32 x
   // 32: 2048^2 complex64 424 against 434 us a cycle, 1024^2 140 against 169)
   int64_t tile16_max[2] = {524288, 2097152};
-  // ... and with at most this many, 8 x 8 tiles (complex64 289 x 311 even;
-  // complex128 128^2 66 us a cycle against 84, 256^2 kernels 92 against 81)
+  // ... and with at most this many, 8 x 8 tiles (complex64, a cycle without them
+  // and with: 256^2 49.3 and 47.0 us, 192^2 45.5 and 44.1, 289 x 311 59.8 and 59.6;
+  // complex128 128^2 84 and 66 us, 256^2, whose finest level does not take them,
+  // 81 without and 92 if it did)
   int64_t tile8_max[2] = {16384, 131072};
   // levels with at most this many cells run in the single-block tail kernel
-  // (64^2 complex128 even with 64 and 256; 289 x 311 complex64 73 us a cycle
-  // with 256, 60 with 1024 and 2048)
+  // (a cycle of complex128 with 16, 64 and 256: 40 x 48 68.1, 55.3 and 53.6 us,
+  // 64^2 52.4, 55.8 and 55.3, 128^2 63.9, 66.6 and 69.0, 256^2 101.5, 101.7 and 99.4;
+  // 289 x 311 complex64 73 us with 256, 60 with 1024 and 2048)
   int64_t tail_max[2] = {64, 2048};
   // Thresholds that the tuner or a program chose count a level's cells alone:
   // they are picked with one source, and with nine of them the 112 x 96 levels

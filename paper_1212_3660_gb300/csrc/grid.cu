@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(256) k_prolong_add3(LevelView<T> F, int cnx, i
 //   pre : z = four half sweeps from z = 0 (red, black, red, black); write z;
 //         coarse f = sum over children of (f - A z)
 //   post: z += P z_coarse; four half sweeps (black, red, black, red); write z
+
 // sum over existing neighbours of t_face * z_nb for a 2D cell held at r in a
 // shared tile of row length RX (same order as nb_sum)
 template <typename T>
@@ -1485,7 +1486,7 @@ __device__ __forceinline__ void gj_warp_best(unsigned long long* v, int* i) {
 
 // One elimination step over the whole chip. One block per tau, as this was
 // before, is bound by one SM's FP64 rate (2 fused multiply-adds a clock) and
-// by its reads of the matrix: 265 ms for four 625 x 625 matrices. Here a block
+// by its reads of the matrix: 260 ms for four 625 x 625 matrices. Here a block
 // updates a 32 x 8 tile, read from S and written to D (the two buffers
 // alternate, so a step needs no barrier inside the grid). Every block finds
 // the pivot itself from the step's column, which the step before left
