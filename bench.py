@@ -141,7 +141,7 @@ def parse():
 
 # The CUDA sources that define each kernel class (its translation unit and the
 # headers it includes); DRAM traffic recorded for another digest of them is stale.
-_GRID_SOURCES = ("grid.cu", "grid.cuh", "stencil.cuh", "common.cuh")
+_GRID_SOURCES = ("grid.cu", "grid.cuh", "stencil.cuh", "sweep.cuh", "common.cuh")
 CLASS_SOURCES = {"smooth": _GRID_SOURCES, "restrict": _GRID_SOURCES, "prolong": _GRID_SOURCES,
                  "pre2d": _GRID_SOURCES, "post2d": _GRID_SOURCES, "tail": _GRID_SOURCES, "defect": _GRID_SOURCES,
                  "sensitivity": ("sensitivity.cu", "sensitivity.cuh", "stencil.cuh", "common.cuh")}
