@@ -660,11 +660,12 @@ static cx<VT>* vcycle(Solve& S, z64* Zk = nullptr, int64_t vsZk = 0, int64_t zco
   // idle. In a server batch complex128 counts expected() sources, whose
   // arithmetic fills them; complex64 all slots, because the many blocks of small
   // tiles cost an idle slot most (4096 blocks that return at once take 5 us).
-  // A served source of 256^2 complex128 with 16 spare slots takes 52.4 ms (69.5
-  // counting slots, 51.7 sources), 128^2 36.7 (42.3, 35.9), 64^2 27.3 (31.5, 27.4),
-  // 160 x 150 183 (178, 183); all 17 slots busy 256^2 522 (491, 543), 128^2 159 (162 to
-  // 171, 180), 64^2 48 (44, 48), 160 x 150 533 (526, 539); complex64 224^2 with one
-  // source 27.9 ms counting slots, 36.4 sources, 311 x 289 40.8 and 59.9.
+  // ms with 16 spare slots, counting slots, expected() and sources: one source of
+  // 256^2 complex128 67.8, 52.1, 51.7; 192^2 53.5, 44.0, -; 128^2 41.8, 36.5, 35.9; 64^2
+  // 31.8, 27.3, 27.4; 150 x 160 174, 180, 180. Four: 128^2 55, 57, 55; 64^2 36.3, 33.2, 33.3;
+  // 150 x 160 268, 278, 277. All 17: 256^2, 192^2 and 128^2 the same within their spread
+  // (497 to 535, 294 to 315, 159 to 173), 64^2 44.1, 48.0, 48.0; 40 x 48 42.9, 37.5, -.
+  // One source of complex64, slots and sources: 224^2 27.9, 36.4; 289 x 311 40.8, 59.9.
   const bool by_level = S.op->by_level[sizeof(VT) == 8 ? 0 : 1];
   const int64_t nsl = by_level ? 1 : (sizeof(VT) == 8 ? S.expected() : S.nslot);
   auto tile_of = [&](const LevelHost& L) { return L.n * nsl <= t8 ? 8 : (L.n * nsl <= t16 ? 16 : 32); };
